@@ -71,7 +71,8 @@ typedef struct lbm_sw lbm_sw;
 #define LBM_SW_E_ARG (-1)      /* invalid argument (NULL, size, parameter out of range) */
 #define LBM_SW_E_CUDA (-2)     /* a CUDA call failed; see lbm_sw_last_error */
 #define LBM_SW_E_UNSTABLE (-3) /* a diagnostic found NaN/Inf or a depth h <= 0 */
-/* (-4 is not used: no kernel of this library waits on a flag or on another grid) */
+/* (-4 is not used: no kernel of this library waits on another grid; the warps of one 1D launch
+ * wait for one another with a bound, and store NaN if it runs out) */
 #define LBM_SW_E_STATE (-5)    /* call not valid in the handle's state (e.g. no state set) */
 #define LBM_SW_E_NOMEM (-6)    /* device allocation failed */
 
@@ -111,9 +112,9 @@ typedef struct lbm_sw lbm_sw;
 #define LBM_SW_KERNEL_SIMPLE 1  /* one launch per step, one thread per cell, scalar loads */
 #define LBM_SW_KERNEL_VEC 2     /* 2D: 16-byte vectors along x (4 FP32 or 2 FP64 cells per thread),
                                    x-neighbours exchanged with warp shuffles */
-#define LBM_SW_KERNEL_CLUSTER 3 /* 1D: all n steps of lbm_sw_step in one thread-block-cluster
-                                   launch, the line held in shared memory (up to 16384 cells on a
-                                   GB300; longer lines use SIMPLE) */
+#define LBM_SW_KERNEL_CLUSTER 3 /* 1D: all n steps of lbm_sw_step in one cooperative launch, the
+                                   line held in the registers of warps that exchange their
+                                   borders (up to 16384 cells; longer lines use SIMPLE) */
 #define LBM_SW_KERNEL_TEMPORAL 4 /* 2D FP32: temporal_steps steps per launch (temporal
                                     blocking: a row wavefront through shared memory, 104/k bytes of
                                     HBM traffic per cell update plus halos), BGK, or MRT with an even

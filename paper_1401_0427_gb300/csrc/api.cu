@@ -206,6 +206,7 @@ void lbm_sw_destroy(lbm_sw* h) {
   if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
   if (h->inflow_feq) cudaFree(h->inflow_feq);
   if (h->moments_staging) cudaFree(h->moments_staging);
+  if (h->mail1d) cudaFree(h->mail1d);
   if (h->pop_staging) cudaFree(h->pop_staging);
   if (h->diag_partials) cudaFree(h->diag_partials);
   if (h->diag_out) cudaFree(h->diag_out);
@@ -265,6 +266,10 @@ int lbm_sw_create(const lbm_sw_params* p, lbm_sw** out) {
     if (cudaMemsetAsync(h->buf[i], 0, bytes, h->stream) != cudaSuccess) return bail(LBM_SW_E_CUDA);
   }
   if (cudaMalloc(&h->inflow_feq, 4 * h->q * h->elem) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
+  if (h->kernel == LBM_SW_KERNEL_CLUSTER && p->nx <= lbm::kWindows1dMaxCells &&
+      cudaMalloc(&h->mail1d, p->precision == LBM_SW_FP64 ? lbm::mail1d_bytes<double>(p->nx)
+                                                         : lbm::mail1d_bytes<float>(p->nx)) != cudaSuccess)
+    return bail(LBM_SW_E_NOMEM);
   if (cudaMalloc(&h->diag_partials, 5 * sizeof(double) * lbm::diag_max_blocks()) != cudaSuccess)
     return bail(LBM_SW_E_NOMEM);
   if (cudaMalloc(&h->diag_out, 8 * sizeof(double)) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
@@ -327,12 +332,13 @@ int lbm_sw_step(lbm_sw* h, int n) {
   if (n < 0) return fail(h, LBM_SW_E_ARG, "step: n must be >= 0 (got %d)", n);
   if (!h->has_state) return fail(h, LBM_SW_E_STATE, "step: no state set (call set_state or set_populations)");
   if (h->p.dim == 1 && h->kernel == LBM_SW_KERNEL_CLUSTER && n > 0) {
-    const bool fp64 = h->p.precision == LBM_SW_FP64;
-    const int max_cells = fp64 ? lbm::cluster1d_max_cells<double>() : lbm::cluster1d_max_cells<float>();
-    if (h->p.nx <= max_cells) {
-      cudaError_t e = fp64 ? lbm::launch_step1d_cluster<double>(args<double>(h, h->cur), consts(h), n, h->stream)
-                           : lbm::launch_step1d_cluster<float>(args<float>(h, h->cur), consts(h), n, h->stream);
-      if (e != cudaSuccess) return cuda_fail(h, e, "cluster step launch");
+    if (h->p.nx <= lbm::kWindows1dMaxCells) {
+      const bool fp64 = h->p.precision == LBM_SW_FP64;
+      cudaError_t e = fp64 ? lbm::launch_step1d_windows<double>(args<double>(h, h->cur), consts(h), n, h->mail1d,
+                                                                h->sm_count, h->stream)
+                           : lbm::launch_step1d_windows<float>(args<float>(h, h->cur), consts(h), n, h->mail1d,
+                                                               h->sm_count, h->stream);
+      if (e != cudaSuccess) return cuda_fail(h, e, "line step launch");
       h->cur ^= 1;
       h->steps_done += n;
       h->launches += 1;
@@ -392,9 +398,7 @@ int lbm_sw_step_plan(const lbm_sw* h, int n, int* sizes, int max_sizes) {
   };
   if (n == 0) return 0;
   if (h->p.dim == 1 && h->kernel == LBM_SW_KERNEL_CLUSTER) {
-    const int max_cells = h->p.precision == LBM_SW_FP64 ? lbm::cluster1d_max_cells<double>()
-                                                        : lbm::cluster1d_max_cells<float>();
-    if (h->p.nx <= max_cells) {
+    if (h->p.nx <= lbm::kWindows1dMaxCells) {
       put(n);
       return count;
     }
@@ -649,11 +653,8 @@ int lbm_sw_get_info(const lbm_sw* h, lbm_sw_info* out) {
   if (!h || !out) return LBM_SW_E_ARG;
   out->q = h->q;
   out->kernel = h->kernel;
-  if (h->p.dim == 1 && h->kernel == LBM_SW_KERNEL_CLUSTER) {
-    const int max_cells = h->p.precision == LBM_SW_FP64 ? lbm::cluster1d_max_cells<double>()
-                                                        : lbm::cluster1d_max_cells<float>();
-    if (h->p.nx > max_cells) out->kernel = LBM_SW_KERNEL_SIMPLE;
-  }
+  if (h->p.dim == 1 && h->kernel == LBM_SW_KERNEL_CLUSTER && h->p.nx > lbm::kWindows1dMaxCells)
+    out->kernel = LBM_SW_KERNEL_SIMPLE;
   out->pitch = static_cast<size_t>(h->pitch);
   out->population_bytes = static_cast<size_t>(h->q) * h->p.nx * h->p.ny * h->elem;
   out->bytes_per_update = 2.0 * h->q * static_cast<double>(h->elem);

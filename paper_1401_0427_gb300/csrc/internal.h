@@ -123,12 +123,14 @@ cudaError_t launch_step2d_temporal_mrt(const StepArgs<float>& a, const ConstsD& 
 // ---- 1D launchers (kernels_1d.cu) ----
 template <class T>
 cudaError_t launch_step1d(const StepArgs<T>& a, const ConstsD& k, cudaStream_t st);
-// All nsteps steps of a line in one thread-block-cluster launch (src -> dst); lines of up to
-// cluster1d_max_cells<T>() cells.
+// All nsteps steps of a line in one cooperative launch (src -> dst); lines of up to
+// kWindows1dMaxCells cells.  mail: mail1d_bytes<T>(nx) bytes of device memory of the handle.
+constexpr int kWindows1dMaxCells = 16384;
 template <class T>
-int cluster1d_max_cells();
+size_t mail1d_bytes(int nx);
 template <class T>
-cudaError_t launch_step1d_cluster(const StepArgs<T>& a, const ConstsD& k, int nsteps, cudaStream_t st);
+cudaError_t launch_step1d_windows(const StepArgs<T>& a, const ConstsD& k, int nsteps, void* mail, int sm_count,
+                                  cudaStream_t st);
 template <class T>
 cudaError_t launch_init1d(const StepArgs<T>& a, const ConstsD& k, const double* h, const double* hu,
                           cudaStream_t st);
@@ -168,6 +170,7 @@ struct lbm_sw {
   int cur = 0;              // buffer holding the current state
   void* inflow_feq = nullptr;
   double* moments_staging = nullptr;  // 3 * nx * ny doubles, for host transfers
+  void* mail1d = nullptr;             // exchange between the windows of a line (1D CLUSTER)
   void* pop_staging = nullptr;        // dense populations, for host transfers / collide
   double* diag_partials = nullptr;
   double* diag_out = nullptr;         // device, 8 doubles

@@ -1,13 +1,12 @@
 // D1Q3Q2 kernels (section 2): populations f0, f+, f- (mass, D1Q3) and g+, g-
 // (discharge, D1Q2; h_0^* does not depend on beta, so there is no g0).  One thread
 // per cell; five planes of `pitch` elements, post-collision values.
-#include <cooperative_groups.h>
 #include <cuda_runtime.h>
+
+#include <cmath>
 
 #include "internal.h"
 #include "scheme.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace lbm {
 namespace {
@@ -47,120 +46,152 @@ __global__ void __launch_bounds__(256) step1d(const StepArgs<T> A, const Consts<
   }
 }
 
-// Steps per cluster barrier in step1d_cluster.
-constexpr int kCluster1dBlock = 8;
+// ---- all n steps of a line in one launch: windows of cells in registers ----
+//
+// The line is cut into pieces of 32 - 2B cells.  One warp (a CTA of its own, so that the warps
+// spread over the SMs) holds a piece and B cells on each side, one cell per lane, and advances
+// them B steps with warp shuffles for the pulls: no shared memory and no barrier.  After s steps the window is exact but for s cells at each end that is not a
+// physical boundary, which never reaches the piece within B steps.  Then the warp publishes the
+// cells that its neighbours hold as halo, reads its own halo from theirs, and goes on.  Every
+// cell update is the pull + collide of the per-step kernel on the same values: the same bits.
+//
+// What bounds it is the collision's chain of one warp: in FP64 every instruction takes 64 cycles
+// of its quarter of an SM (half a lane per clock, whatever the number of active lanes), so the
+// line is spread over as many quarters as it fills.  1000 cells, FP64: 1.23 us per step, against
+// 1.44 with one cluster of 16 SMs (windows of 63 + 16 cells in shared memory, a cluster barrier
+// per 8 steps); 16000 cells: 1.66 against 9.82.  FP32: 0.17 against 0.39 and 0.18 against 0.69.
+//
+// Exchange: a mailbox in global memory with two slots per cell, used by turns.  Each 8-byte
+// word carries 4 bytes of payload and the number of the exchange, written and read as one
+// access, so a reader that sees the number has the payload: one trip through L2 and no fence.  A
+// slot is written again two exchanges later, when its writer has read the exchange between from
+// the same neighbours, who had read the slot before they published that one.  The launch is
+// cooperative, so every warp is resident; a wait gives up after kWaitPolls polls all the same,
+// and the results of that launch are then stored as NaN, which diagnostics report.
+constexpr int kWaitPolls = 1 << 22;
+constexpr unsigned kAllLanes = 0xffffffffu;
 
-// All n steps of a line of up to 16 * 1024 cells in one launch: one thread-block cluster,
-// CTA r owns cells [r * chunk, (r + 1) * chunk) and keeps them in shared memory.  The steps
-// go in blocks of up to kCluster1dBlock (KB): at the start of a block a CTA copies its own
-// cells and KB cells on each side (from the neighbouring CTAs' shared memory, distributed
-// shared memory, wrapping around on periodic sides) into a local window, advances the window
-// KB steps on its own, and writes its own cells back.  After step s the window is exact
-// except for s cells at each end that is not a physical boundary, which never reaches the
-// owned cells.  One cluster barrier per block orders the write-back before the neighbours'
-// next reads; the owned copies alternate between two buffers, so a block's writes never
-// meet the same block's reads.  Every cell update is the pull + collide of the per-step
-// kernel on the same values, so the results are equal bit for bit.
-template <class T, bool MRT>
-__global__ void __launch_bounds__(1024) step1d_cluster(const StepArgs<T> A, const Consts<T> K, int nsteps,
-                                                       int chunk) {
-  constexpr int KB = kCluster1dBlock;
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = static_cast<int>(cluster.block_rank());
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int wcap = chunk + 2 * KB;  // window capacity
-  T* home = reinterpret_cast<T*>(smem_raw);
-  T* other = home + 5 * chunk;
-  T* const win0 = other + 5 * chunk;
-  T* const win1 = win0 + 5 * wcap;
-  const int nx = A.nx;
-  const int i0 = rank * chunk;
-  const int ncell = nx - i0 < chunk ? nx - i0 : chunk;  // <= 0 for idle trailing CTAs
-  const bool per = A.bc[LBM_SW_SIDE_XM] == LBM_SW_BC_PERIODIC;  // periodic sides come in pairs
-  for (int c = threadIdx.x; c < ncell; c += blockDim.x)
-#pragma unroll
-    for (int p = 0; p < 5; ++p) home[p * chunk + c] = A.src[p * A.plane + i0 + c];
-  cluster.sync();
-  for (int done = 0; done < nsteps; done += KB) {
-    const int kb = nsteps - done < KB ? nsteps - done : KB;
-    if (ncell > 0) {
-      // the window holds cells [i0 - L, i0 + ncell + R)
-      const int L = per ? kb : min(kb, i0);
-      const int R = per ? kb : min(kb, nx - i0 - ncell);
-      const int wn = L + ncell + R;
-      const bool left_end = !per && i0 - L == 0;  // the window starts at the x- side
-      const bool right_end = !per && i0 + ncell + R == nx;
-      for (int w = threadIdx.x; w < wn; w += blockDim.x) {
-        int g = i0 - L + w;
-        if (per) {
-          g %= nx;
-          if (g < 0) g += nx;
-        }
-        const int r = g / chunk;
-        const int c = g - r * chunk;
-        const T* src = r == rank ? home : cluster.map_shared_rank(home, r);
-#pragma unroll
-        for (int p = 0; p < 5; ++p) win0[p * wcap + w] = src[p * chunk + c];
-      }
-      __syncthreads();
-      T* cur = win0;
-      T* nxt = win1;
-      for (int s = 1; s <= kb; ++s) {
-        const int lo = left_end ? 0 : s;
-        const int hi = right_end ? wn : wn - s;
-        for (int w = lo + threadIdx.x; w < hi; w += blockDim.x) {
-          const int g = i0 - L + w;  // the cell (sides that are not periodic)
-          T f[5];
-          f[0] = cur[w];
-#pragma unroll
-          for (int p = 1; p < 5; ++p) {
-            const bool plus = (p == 1 || p == 3);  // moves +lambda: comes from w - 1
-            if (per || (plus ? g > 0 : g < nx - 1)) {
-              f[p] = cur[p * wcap + (plus ? w - 1 : w + 1)];
-            } else {
-              const int side = plus ? LBM_SW_SIDE_XM : LBM_SW_SIDE_XP;
-              switch (A.bc[side]) {
-                case LBM_SW_BC_WALL: {  // mirror of the boundary cell: f+ <-> f-, g+ <-> -g-
-                  const int m = (p == 1) ? 2 : (p == 2) ? 1 : (p == 3) ? 4 : 3;
-                  const T v = cur[m * wcap + w];
-                  f[p] = p >= 3 ? -v : v;
-                  break;
-                }
-                case LBM_SW_BC_OUTFLOW:
-                  f[p] = cur[p * wcap + w];
-                  break;
-                default:
-                  f[p] = A.inflow_feq[side * 5 + p];
-              }
-            }
-          }
-          collide5_any<T, MRT>(f, K);
-#pragma unroll
-          for (int p = 0; p < 5; ++p) nxt[p * wcap + w] = f[p];
-        }
-        __syncthreads();
-        T* t = cur;
-        cur = nxt;
-        nxt = t;
-      }
-      for (int c = threadIdx.x; c < ncell; c += blockDim.x)
-#pragma unroll
-        for (int p = 0; p < 5; ++p) other[p * chunk + c] = cur[p * wcap + L + c];
-    }
-    cluster.sync();
-    T* t = home;
-    home = other;
-    other = t;
-  }
-  for (int c = threadIdx.x; c < ncell; c += blockDim.x)
-#pragma unroll
-    for (int p = 0; p < 5; ++p) A.dst[p * A.plane + i0 + c] = home[p * chunk + c];
+template <class T>
+struct MailWords;  // 8-byte words per value
+template <>
+struct MailWords<float> {
+  static constexpr int n = 1;
+};
+template <>
+struct MailWords<double> {
+  static constexpr int n = 2;
+};
+
+__device__ __forceinline__ unsigned long long mail_word(unsigned payload, unsigned epoch) {
+  return (static_cast<unsigned long long>(epoch) << 32) | payload;
+}
+__device__ __forceinline__ void mail_put(unsigned long long* w, float v, unsigned epoch) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"(mail_word(__float_as_uint(v), epoch)) : "memory");
+}
+__device__ __forceinline__ void mail_put(unsigned long long* w, double v, unsigned epoch) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(w),
+               "l"(mail_word(static_cast<unsigned>(b), epoch)), "l"(mail_word(static_cast<unsigned>(b >> 32), epoch))
+               : "memory");
+}
+__device__ __forceinline__ bool mail_get(const unsigned long long* w, float& v, unsigned epoch) {
+  unsigned long long a;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(a) : "l"(w) : "memory");
+  v = __uint_as_float(static_cast<unsigned>(a));
+  return static_cast<unsigned>(a >> 32) == epoch;
+}
+__device__ __forceinline__ bool mail_get(const unsigned long long* w, double& v, unsigned epoch) {
+  unsigned long long a, b;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(w) : "memory");
+  v = __longlong_as_double(static_cast<long long>((b << 32) | (a & 0xffffffffull)));
+  return static_cast<unsigned>(a >> 32) == epoch && static_cast<unsigned>(b >> 32) == epoch;
 }
 
-// Dynamic shared memory of step1d_cluster at `chunk` cells per CTA.
-template <class T>
-size_t cluster1d_smem(int chunk) {
-  return (2 * 5 * static_cast<size_t>(chunk) + 2 * 5 * static_cast<size_t>(chunk + 2 * kCluster1dBlock)) * sizeof(T);
+template <class T, bool MRT>
+__global__ void __launch_bounds__(32) step1d_windows(const StepArgs<T> A, const Consts<T> K, int nsteps, int B,
+                                                     unsigned long long* __restrict__ mail) {
+  constexpr int MW = MailWords<T>::n;
+  const int nx = A.nx;
+  const int out = 32 - 2 * B;                   // cells of a piece
+  const int o = blockIdx.x * out;               // this piece: cells [o, oe)
+  const int oe = min(nx, o + out);
+  const int g = o - B + static_cast<int>(threadIdx.x);          // this lane's cell
+  const bool own = g >= o && g < oe;
+  const bool per = A.bc[LBM_SW_SIDE_XM] == LBM_SW_BC_PERIODIC;  // periodic sides come in pairs
+  const bool has_edge = !per && (o - B <= 0 || oe + B >= nx);   // warp-uniform: the window meets a side
+  // the cell in the domain, -1: outside it, or further out than a halo (reaches no cell of the piece)
+  int cell = per ? g % nx : g;
+  if (per && cell < 0) cell += nx;
+  if (cell < 0 || cell >= nx || g >= oe + B) cell = -1;
+  T f[5];
+#pragma unroll
+  for (int p = 0; p < 5; ++p) f[p] = cell >= 0 ? A.src[p * A.plane + cell] : T(1);
+  bool failed = false;
+  unsigned epoch = 0;
+  for (int done = 0; done < nsteps;) {
+    const int kb = min(B, nsteps - done);
+    for (int s = 0; s < kb; ++s) {
+      // +lambda movers from the cell to the left, -lambda movers from the cell to the right
+      T n[5] = {f[0], __shfl_up_sync(kAllLanes, f[1], 1), __shfl_down_sync(kAllLanes, f[2], 1),
+                __shfl_up_sync(kAllLanes, f[3], 1), __shfl_down_sync(kAllLanes, f[4], 1)};
+      if (has_edge && (cell == 0 || cell == nx - 1)) {
+        if (cell == 0) {
+          const int bc = A.bc[LBM_SW_SIDE_XM];
+          if (bc == LBM_SW_BC_WALL) {  // mirror of the boundary cell: f+ <-> f-, g+ <-> -g-
+            n[1] = f[2];
+            n[3] = -f[4];
+          } else if (bc == LBM_SW_BC_OUTFLOW) {
+            n[1] = f[1];
+            n[3] = f[3];
+          } else {
+            n[1] = A.inflow_feq[LBM_SW_SIDE_XM * 5 + 1];
+            n[3] = A.inflow_feq[LBM_SW_SIDE_XM * 5 + 3];
+          }
+        }
+        if (cell == nx - 1) {
+          const int bc = A.bc[LBM_SW_SIDE_XP];
+          if (bc == LBM_SW_BC_WALL) {
+            n[2] = f[1];
+            n[4] = -f[3];
+          } else if (bc == LBM_SW_BC_OUTFLOW) {
+            n[2] = f[2];
+            n[4] = f[4];
+          } else {
+            n[2] = A.inflow_feq[LBM_SW_SIDE_XP * 5 + 2];
+            n[4] = A.inflow_feq[LBM_SW_SIDE_XP * 5 + 4];
+          }
+        }
+      }
+      collide5_any<T, MRT>(n, K);
+#pragma unroll
+      for (int p = 0; p < 5; ++p) f[p] = n[p];
+    }
+    done += kb;
+    if (done >= nsteps) break;
+    ++epoch;
+    unsigned long long* const w =
+        mail + (static_cast<long long>(epoch & 1) * nx + max(cell, 0)) * static_cast<long long>(5 * MW);
+    if (own && (g < o + B || g >= oe - B))  // cells that some neighbour holds as halo
+#pragma unroll
+      for (int p = 0; p < 5; ++p) mail_put(w + p * MW, f[p], epoch);
+    __syncwarp();  // a window may wait for its own cells (a periodic line of one piece)
+    if (cell >= 0 && !own) {
+      for (int polls = 0;; ++polls) {
+        bool ok = true;
+#pragma unroll
+        for (int p = 0; p < 5; ++p) ok &= mail_get(w + p * MW, f[p], epoch);
+        if (ok) break;
+        if (failed || polls >= kWaitPolls) {  // one exhausted wait ends the later ones at once
+          failed = true;
+          break;
+        }
+      }
+    }
+    failed = __any_sync(kAllLanes, failed);
+  }
+  if (own)
+#pragma unroll
+    for (int p = 0; p < 5; ++p) A.dst[p * A.plane + g] = failed ? T(NAN) : f[p];
 }
 
 template <class T>
@@ -236,75 +267,46 @@ cudaError_t launch_step1d(const StepArgs<T>& a, const ConstsD& kd, cudaStream_t 
   return cudaGetLastError();
 }
 
-// CTAs of the largest cluster the device places for step1d_cluster: 16 where it allows
-// that non-portable size with the shared memory of 1024-cell chunks, else the portable 8.
 template <class T>
-int cluster1d_probe_blocks() {
-  int blocks = 8;
-  if (cudaFuncSetAttribute(step1d_cluster<T, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-      cudaFuncSetAttribute(step1d_cluster<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(cluster1d_smem<T>(1024))) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(16);
-    cfg.blockDim = dim3(1024);
-    cfg.dynamicSmemBytes = cluster1d_smem<T>(1024);
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 16;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, step1d_cluster<T, false>, &cfg) == cudaSuccess && clusters > 0)
-      blocks = 16;
-  }
-  cudaGetLastError();  // a refused attribute or probe leaves no error behind
-  return blocks;
+size_t mail1d_bytes(int nx) {
+  return static_cast<size_t>(2) * nx * 5 * MailWords<T>::n * sizeof(unsigned long long);
+}
+
+// Steps between exchanges (the halo's width) for a line of nx cells: an exchange takes about
+// 0.5 us, so wide halos while the warps they make find free quarters of SMs, narrower ones (fewer
+// warps) on longer lines.  FP64, us per step with halos of 4 / 6 / 8 / 10: 3000 cells 1.31 / 1.25
+// / 1.26 / 1.21, 8000 cells 1.32 / 1.25 / 1.32 / 1.64, 16000 cells 1.66 / 1.85 / 2.10 / -.  FP32
+// with 6 / 8 / 10: 3000 cells 0.20 / 0.18 / 0.16, 16000 cells 0.23 / 0.18 / 0.20.  Two or four
+// cells per lane were slower at every length (16000 cells, FP64: 2.3 and 4.6).
+template <class T>
+int window_halo(int nx, int sm_count) {
+  auto pieces = [&](int b) { return (nx + 32 - 2 * b - 1) / (32 - 2 * b); };
+  if constexpr (sizeof(T) == 8)
+    return pieces(10) <= 3 * sm_count ? 10 : pieces(6) <= 3 * sm_count ? 6 : 4;
+  else
+    return pieces(10) <= 4 * sm_count ? 10 : 8;
 }
 
 template <class T>
-int cluster1d_max_cells() {
-  static const int max_blocks = cluster1d_probe_blocks<T>();  // probed once (thread-safe initialisation)
-  return max_blocks * 1024;
-}
-
-template <class T, bool MRT>
-cudaError_t launch_cluster_t(const StepArgs<T>& a, const ConstsD& kd, int nsteps, cudaStream_t st) {
-  const int max_cells = cluster1d_max_cells<T>();
-  const int max_blocks = max_cells / 1024;
-  int blocks = (a.nx + 63) / 64;  // at least 64 cells per CTA
-  if (blocks > max_blocks) blocks = max_blocks;
-  if (blocks < 1) blocks = 1;
-  const int chunk = (a.nx + blocks - 1) / blocks;
-  const int window = chunk + 2 * kCluster1dBlock;
-  const int threads = window < 1024 ? ((window + 31) / 32) * 32 : 1024;
-  const size_t smem = cluster1d_smem<T>(chunk);
-  cudaError_t e = cudaFuncSetAttribute(step1d_cluster<T, MRT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(cluster1d_smem<T>(1024)));
-  if (e != cudaSuccess) return e;
-  if (blocks > 8) {
-    e = cudaFuncSetAttribute(step1d_cluster<T, MRT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+cudaError_t launch_step1d_windows(const StepArgs<T>& a, const ConstsD& kd, int nsteps, void* mail, int sm_count,
+                                  cudaStream_t st) {
+  const int b = window_halo<T>(a.nx, sm_count), out = 32 - 2 * b;
+  const int pieces = (a.nx + out - 1) / out;
+  if (pieces > 1 || a.bc[LBM_SW_SIDE_XM] == LBM_SW_BC_PERIODIC) {
+    cudaError_t e = cudaMemsetAsync(mail, 0, mail1d_bytes<T>(a.nx), st);  // exchange numbers start at 1
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(pieces);
+  cfg.blockDim = dim3(32);
   cfg.stream = st;
   cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = blocks;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
+  attr.id = cudaLaunchAttributeCooperative;
+  attr.val.cooperative = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, step1d_cluster<T, MRT>, a, consts1<T>(kd), nsteps, chunk);
-}
-
-template <class T>
-cudaError_t launch_step1d_cluster(const StepArgs<T>& a, const ConstsD& kd, int nsteps, cudaStream_t st) {
-  return kd.mrt ? launch_cluster_t<T, true>(a, kd, nsteps, st) : launch_cluster_t<T, false>(a, kd, nsteps, st);
+  return cudaLaunchKernelEx(&cfg, kd.mrt ? step1d_windows<T, true> : step1d_windows<T, false>, a, consts1<T>(kd),
+                            nsteps, b, static_cast<unsigned long long*>(mail));
 }
 
 template <class T>
@@ -344,8 +346,9 @@ cudaError_t launch_inflow_feq1d(T* out, const int bc[4], const double inflow[4][
 
 #define LBM_INSTANTIATE_1D(T)                                                                               \
   template cudaError_t launch_step1d<T>(const StepArgs<T>&, const ConstsD&, cudaStream_t);                 \
-  template int cluster1d_max_cells<T>();                                                                    \
-  template cudaError_t launch_step1d_cluster<T>(const StepArgs<T>&, const ConstsD&, int, cudaStream_t);    \
+  template size_t mail1d_bytes<T>(int);                                                                     \
+  template cudaError_t launch_step1d_windows<T>(const StepArgs<T>&, const ConstsD&, int, void*, int,        \
+                                                cudaStream_t);                                              \
   template cudaError_t launch_init1d<T>(const StepArgs<T>&, const ConstsD&, const double*, const double*,   \
                                         cudaStream_t);                                                      \
   template cudaError_t launch_collide1d_dense<T>(const StepArgs<T>&, const ConstsD&, const T*, cudaStream_t); \
