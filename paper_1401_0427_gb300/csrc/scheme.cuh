@@ -35,20 +35,29 @@ __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, 
 __device__ __forceinline__ float fmad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmad(double a, double b, double c) { return __fma_rn(a, b, c); }
 // FP32: the fast reciprocal intrinsic (at most 2 ulp; the FP32 path is compared with the
-// FP64 oracle at 1e-5).  FP64: Newton-Raphson for 1/a, two iterations of r <- r + r (1 - a r)
-// (each residual and update one fused multiply-add) from the PTX approximation
-// rcp.approx.ftz.f64; for positive normal depths it equals the IEEE round-to-nearest
-// reciprocal (0 ulp on 2.7e8 sampled inputs in [1e-3, 1e3)) at fewer FP64 operations, the
-// resource that bounds the FP64 kernels on GB300.  Either is a fixed function of h, so
-// mirror-image cells still round alike.
+// FP64 oracle at 1e-5).  FP64: the PTX approximation rcp.approx.ftz.f64 (relative error e of about
+// 2^-20) and one step r <- r + r (e + e^2) (the geometric series of 1 / (1 - e) up to its second
+// power; the rest, e^3 of about 2^-60, is below the rounding): three fused multiply-adds of the
+// unit that bounds the FP64 kernels on GB300, where two Newton-Raphson steps take four.  Either is
+// a fixed function of h, so mirror-image cells still round alike.
 __device__ __forceinline__ float recip(float a) { return __fdividef(1.0f, a); }
 __device__ __forceinline__ double recip(double a) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  double e = __fma_rn(-a, r, 1.0);
-  r = __fma_rn(r, e, r);
-  e = __fma_rn(-a, r, 1.0);
-  return __fma_rn(r, e, r);
+  const double e = __fma_rn(-a, r, 1.0);
+  return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+// x times 2^k (NEG: -2^k), exactly, by the exponent field: a few integer operations, where an FP64
+// multiplication takes 64 cycles of a quarter of an SM.  Zeros keep their value; denormals,
+// infinities, NaN and results out of the normal range take the multiplication.
+template <int k, bool NEG>
+__device__ __forceinline__ double times_pow2(double x) {
+  constexpr int flip = NEG ? static_cast<int>(0x80000000u) : 0;
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  if (e > (k < 0 ? -k : 0) && e < (k < 0 ? 0x7ff : 0x7ff - k)) return __hiloint2double((hi + k * (1 << 20)) ^ flip, lo);
+  if (((hi & 0x7fffffff) | lo) == 0) return __hiloint2double(hi ^ flip, 0);
+  return __dmul_rn(x, (NEG ? -1.0 : 1.0) * (k < 0 ? 1.0 / (1 << -k) : static_cast<double>(1 << (k < 0 ? 0 : k))));
 }
 
 // Scheme constants in the storage precision.
@@ -83,6 +92,8 @@ struct Consts {
   T s_p;    // s c g / 2
   T s_c;    // s c
   T s_4;    // s / 4
+  // 1D, FP64: f0 = a_2 h + a_4g u^2
+  T a_2, a_4g;
 };
 
 template <class T>
@@ -107,6 +118,8 @@ __host__ Consts<T> make_consts(double g, double lambda, double s, double a) {
   k.s_p = static_cast<T>(st * c * g / 2.0);
   k.s_c = static_cast<T>(st * c);
   k.s_4 = static_cast<T>(st / 4.0);
+  k.a_2 = static_cast<T>(a / 2.0);
+  k.a_4g = static_cast<T>(-a / (4.0 * g));
   for (int i = 0; i < 10; ++i) k.r[i] = k.s;
   set_mrt_folded(k);
   return k;
@@ -203,6 +216,36 @@ __device__ __forceinline__ void collide13(T f[13], const Consts<T>& k, T& h, T& 
   f[10] = fmad(om, f[10], add(y4, pyy));
   f[11] = fmad(om, f[11], sub(y4, pxy));
   f[12] = fmad(om, f[12], sub(y4, pyy));
+}
+
+// FP64: the same operator in 52 operations of the FP64 unit instead of 59 (the unit bounds every
+// FP64 kernel: 64 cycles per warp instruction on its quarter of an SM).  The two terms of each
+// equilibrium meet in one fused multiply-add, s r +- s c q and s q / 4 +- (s c h) t with
+// t = u^2 + g h / 2, v^2 + g h / 2 or u v, so the products s c q and s c (q u + p) are not formed;
+// each population rounds once less than above.  Mirror images still round alike.
+__device__ __forceinline__ void collide13(double f[13], const Consts<double>& k, double& h, double& qx, double& qy) {
+  moments13(f, h, qx, qy);
+  const double rh = recip(h);
+  const double u = mul(qx, rh), v = mul(qy, rh);
+  const double uu = mul(u, u), vv = mul(v, v), uv = mul(u, v);
+  const double z = fmad(add(uu, vv), k.s_a4g, mul(k.s_a2, h));  // -s f0^eq / 4
+  const double r = fmad(h, k.s_4, z);                           // s (h - f0^eq) / 4
+  const double tx = fmad(k.half_g, h, uu), ty = fmad(k.half_g, h, vv);
+  const double hc = mul(h, k.s_c), x4 = mul(qx, k.s_4), y4 = mul(qy, k.s_4);
+  const double om = k.om;
+  f[0] = fmad(om, f[0], times_pow2<2, true>(z));
+  f[1] = fmad(om, f[1], fmad(k.s_c, qx, r));
+  f[2] = fmad(om, f[2], fmad(k.s_c, qy, r));
+  f[3] = fmad(om, f[3], fmad(-k.s_c, qx, r));
+  f[4] = fmad(om, f[4], fmad(-k.s_c, qy, r));
+  f[5] = fmad(om, f[5], fmad(hc, tx, x4));
+  f[6] = fmad(om, f[6], fmad(hc, uv, x4));
+  f[7] = fmad(om, f[7], fmad(-hc, tx, x4));
+  f[8] = fmad(om, f[8], fmad(-hc, uv, x4));
+  f[9] = fmad(om, f[9], fmad(hc, uv, y4));
+  f[10] = fmad(om, f[10], fmad(hc, ty, y4));
+  f[11] = fmad(om, f[11], fmad(-hc, uv, y4));
+  f[12] = fmad(om, f[12], fmad(-hc, ty, y4));
 }
 
 template <class T>
@@ -507,6 +550,24 @@ __device__ __forceinline__ void collide5(T f[5], const Consts<T>& k) {
   moments5(f, h, q);
   T e[5];
   equilibrium5(h, q, k, e);
+#pragma unroll
+  for (int j = 0; j < 5; ++j) f[j] = fmad(k.s, sub(e[j], f[j]), f[j]);
+}
+
+// FP64 in 1D: the same f + s (f^eq - f) with 26 operations of the FP64 unit instead of 32 (a
+// line's steps are one warp's chain of them): the halves by the exponent field, the flux
+// c (q u + p) as (c h) (u^2 + g h / 2) inside the fused multiply-adds of g+-.  The folded
+// (1 - s) f + s f^eq would save four more, but its depth drifts: on 1000 cells after 500 steps
+// the error of h against quadruple precision is 6e-16 in this form and the one above, 2e-15 folded.
+__device__ __forceinline__ void collide5(double f[5], const Consts<double>& k) {
+  double h, q;
+  moments5(f, h, q);
+  const double u = mul(q, recip(h)), uu = mul(u, u);
+  const double f0 = fmad(uu, k.a_4g, mul(h, k.a_2));
+  const double r = times_pow2<-1, false>(sub(h, f0));  // (h - f0) / 2
+  const double t = fmad(k.half_g, h, uu);
+  const double hc = mul(h, k.c), q2 = times_pow2<-1, false>(q);
+  const double e[5] = {f0, fmad(k.c, q, r), fmad(-k.c, q, r), fmad(hc, t, q2), fmad(-hc, t, q2)};
 #pragma unroll
   for (int j = 0; j < 5; ++j) f[j] = fmad(k.s, sub(e[j], f[j]), f[j]);
 }
