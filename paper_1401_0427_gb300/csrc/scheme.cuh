@@ -34,13 +34,18 @@ __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b);
 __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ float fmad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmad(double a, double b, double c) { return __fma_rn(a, b, c); }
-// FP32: the fast reciprocal intrinsic (at most 2 ulp; the FP32 path is compared with the
-// FP64 oracle at 1e-5).  FP64: the PTX approximation rcp.approx.ftz.f64 (relative error e of about
+// FP32: the PTX approximation rcp.approx.ftz.f32 (1 ulp; the FP32 path is compared with the FP64
+// oracle at 1e-5), the value of __fdividef(1, a) for every a but denormals, without its scaling of
+// large arguments (five instructions more per cell).  FP64: the PTX approximation rcp.approx.ftz.f64 (relative error e of about
 // 2^-20) and one step r <- r + r (e + e^2) (the geometric series of 1 / (1 - e) up to its second
 // power; the rest, e^3 of about 2^-60, is below the rounding): three fused multiply-adds of the
 // unit that bounds the FP64 kernels on GB300, where two Newton-Raphson steps take four.  Either is
 // a fixed function of h, so mirror-image cells still round alike.
-__device__ __forceinline__ float recip(float a) { return __fdividef(1.0f, a); }
+__device__ __forceinline__ float recip(float a) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return r;
+}
 __device__ __forceinline__ double recip(double a) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
