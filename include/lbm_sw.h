@@ -108,7 +108,9 @@ typedef struct lbm_sw lbm_sw;
 #define LBM_SW_KERNEL_AUTO 0    /* library choice: TEMPORAL for 2D FP32 grids of >= 3 * 2^17 cells
                                    (628^2 and up) with every side periodic or an even
                                    temporal_steps (with MRT relaxation: >= 2^19 cells), else VEC in
-                                   2D; CLUSTER in 1D */
+                                   2D; CLUSTER in 1D.  FP32 grids below 5 * 2^17 cells without
+                                   obstacles and with temporal_steps = 0 take 4 to 8 steps per
+                                   launch on tiles held in registers, with the same results */
 #define LBM_SW_KERNEL_SIMPLE 1  /* one launch per step, one thread per cell, scalar loads */
 #define LBM_SW_KERNEL_VEC 2     /* 2D: 16-byte vectors along x (4 FP32 or 2 FP64 cells per thread),
                                    x-neighbours exchanged with warp shuffles */
@@ -150,7 +152,8 @@ typedef struct lbm_sw_info {
   long long kernel_launches; /* kernels this handle has launched */
   int steps_per_launch;      /* steps one step-kernel launch advances: temporal_steps where
                                 TEMPORAL fuses steps (see LBM_SW_KERNEL_TEMPORAL), 0 for CLUSTER
-                                (all n steps of lbm_sw_step in one launch), else 1 */
+                                (all n steps of lbm_sw_step in one launch), else 1; AUTO may
+                                join further steps in a launch (lbm_sw_step_plan lists them) */
 } lbm_sw_info;
 
 /* Fill *p with defaults: dim 2, FP32, g = 1, lambda = 8, s = 1.8, a = 0.05,
@@ -185,6 +188,8 @@ LBM_SW_API int lbm_sw_set_state(lbm_sw* h, const double* depth, const double* hu
  *             single step), e.g. 20 = 6 + 6 + 4 + 4 at K = 6;
  *             lbm_sw_step_plan lists the launches;
  *   CLUSTER:  one launch for all n steps (1D lines up to 16384 cells);
+ *   AUTO on FP32 grids below 5 * 2^17 cells without obstacles (temporal_steps = 0): launches of
+ *             up to 8 steps, as even as they come (lbm_sw_step_plan);
  *   VEC, SIMPLE, obstacles: one launch per step; long runs replay a captured CUDA graph of
  *             graph_chunk steps.
  * Every mapping gives the same bits.  Errors: LBM_SW_E_ARG (n < 0), LBM_SW_E_STATE (no

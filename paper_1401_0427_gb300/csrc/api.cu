@@ -19,6 +19,11 @@ namespace {
 // slower.
 constexpr long long kAutoTemporalCells = 3LL << 17;
 
+// 2D FP32 grids below this size (cells) take several steps per launch on register tiles under
+// AUTO: 800^2 4.3 us per step against 4.5 for the wavefront (walls, inflow and outflow 5.1 / 5.4,
+// MRT 6.0 / 6.2), 900^2 5.4 against 5.3 (6.3 / 6.0, 7.5 / 7.0).
+constexpr long long kTileCells = 5LL << 17;
+
 int fail(lbm_sw* h, int code, const char* fmt, ...) {
   if (h) {
     char buf[512];
@@ -63,6 +68,24 @@ bool temporal_active(const lbm_sw* h) {
   // +14 % fused at K = 4; 724^2 even, 628^2 -12 %)
   const bool large = static_cast<long long>(h->p.nx) * h->p.ny >= (1LL << 19);
   return lbm::temporal_mrt_supported(h->p.bc, h->p.nx, h->temporal_k) && (large || !h->auto_kernel);
+}
+
+// Whether lbm_sw_step takes register tiles (tile2d.cu): AUTO without a wish for temporal_steps.
+bool tile_active(const lbm_sw* h) {
+  return h->auto_kernel && h->p.temporal_steps == 0 && h->p.dim == 2 && h->p.precision == LBM_SW_FP32 &&
+         !h->has_obstacles && static_cast<long long>(h->p.nx) * h->p.ny < kTileCells;
+}
+
+// The launches of n > 0 steps on register tiles, as even as they come: launch(steps) for each.
+template <class F>
+int for_tile_launches(const lbm_sw* h, int n, F&& launch) {
+  const int k = lbm::tile_steps(h->p.nx, h->p.ny, std::max(h->sm_count, 1));
+  const int count = (n + k - 1) / k, base = n / count, extra = n % count;
+  for (int i = 0; i < count; ++i) {
+    const int rc = launch(i < extra ? base + 1 : base);
+    if (rc != LBM_SW_OK) return rc;
+  }
+  return LBM_SW_OK;
 }
 
 // Launch plan of a fused handle (launch_plan.h): K, and whether odd sizes above one may run
@@ -345,6 +368,17 @@ int lbm_sw_step(lbm_sw* h, int n) {
       return LBM_SW_OK;
     }
   }
+  if (n > 0 && tile_active(h))
+    return for_tile_launches(h, n, [&](int k) {
+      const auto a = args<float>(h, h->cur);
+      const cudaError_t e = k == 1 ? lbm::launch_step2d<float>(a, consts(h), LBM_SW_KERNEL_VEC, h->stream)
+                                   : lbm::launch_step2d_tile(a, consts(h), k, h->stream, h->sm_count);
+      if (e != cudaSuccess) return cuda_fail(h, e, "tile step launch");
+      h->cur ^= 1;
+      h->steps_done += k;
+      h->launches += 1;
+      return static_cast<int>(LBM_SW_OK);
+    });
   if (temporal_active(h)) {
     int plan[64];
     while (n > 0) {
@@ -402,6 +436,13 @@ int lbm_sw_step_plan(const lbm_sw* h, int n, int* sizes, int max_sizes) {
       put(n);
       return count;
     }
+  }
+  if (tile_active(h)) {
+    for_tile_launches(h, n, [&](int k) {
+      put(k);
+      return static_cast<int>(LBM_SW_OK);
+    });
+    return count;
   }
   if (temporal_active(h)) {
     int plan[64];

@@ -120,6 +120,11 @@ bool temporal_mrt_supported(const int bc[4], int nx, int k);
 cudaError_t launch_step2d_temporal_mrt(const StepArgs<float>& a, const ConstsD& kd, int k, cudaStream_t st,
                                        int sm_count);
 
+// kb (1 .. 8) fused steps on tiles held in registers (tile2d.cu; FP32, BGK or MRT, any sides and
+// sizes), and the steps per launch that take the least time per step on an nx x ny grid.
+int tile_steps(int nx, int ny, int sms);
+cudaError_t launch_step2d_tile(const StepArgs<float>& a, const ConstsD& kd, int kb, cudaStream_t st, int sms);
+
 // ---- 1D launchers (kernels_1d.cu) ----
 template <class T>
 cudaError_t launch_step1d(const StepArgs<T>& a, const ConstsD& k, cudaStream_t st);
