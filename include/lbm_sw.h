@@ -108,9 +108,9 @@ typedef struct lbm_sw lbm_sw;
 #define LBM_SW_KERNEL_AUTO 0    /* library choice: TEMPORAL for 2D FP32 grids of >= 3 * 2^17 cells
                                    (628^2 and up) with every side periodic or an even
                                    temporal_steps (with MRT relaxation: >= 2^19 cells), else VEC in
-                                   2D; CLUSTER in 1D.  FP32 grids below 5 * 2^17 cells without
-                                   obstacles and with temporal_steps = 0 take 4 to 8 steps per
-                                   launch on tiles held in registers, with the same results */
+                                   2D; CLUSTER in 1D.  FP32 grids below 5 * 2^17 cells with
+                                   temporal_steps = 0 take 4 to 8 steps per launch on tiles held
+                                   in registers, with the same results */
 #define LBM_SW_KERNEL_SIMPLE 1  /* one launch per step, one thread per cell, scalar loads */
 #define LBM_SW_KERNEL_VEC 2     /* 2D: 16-byte vectors along x (4 FP32 or 2 FP64 cells per thread),
                                    x-neighbours exchanged with warp shuffles */
@@ -121,8 +121,8 @@ typedef struct lbm_sw lbm_sw;
                                     blocking: a row wavefront through shared memory, 104/k bytes of
                                     HBM traffic per cell update plus halos), BGK, or MRT with an even
                                     temporal_steps; the tail of n runs as shorter fused launches
-                                    (lbm_sw_step), obstacles use their own kernel; results equal
-                                    VEC bit for bit */
+                                    (lbm_sw_step), also with obstacles (BGK, even
+                                    temporal_steps); results equal VEC bit for bit */
 
 typedef struct lbm_sw_params {
   int dim;             /* 1 (D1Q3Q2) or 2 (D2Q5Q4Q4) */
@@ -188,9 +188,11 @@ LBM_SW_API int lbm_sw_set_state(lbm_sw* h, const double* depth, const double* hu
  *             single step), e.g. 20 = 6 + 6 + 4 + 4 at K = 6;
  *             lbm_sw_step_plan lists the launches;
  *   CLUSTER:  one launch for all n steps (1D lines up to 16384 cells);
- *   AUTO on FP32 grids below 5 * 2^17 cells without obstacles (temporal_steps = 0): launches of
- *             up to 8 steps, as even as they come (lbm_sw_step_plan);
- *   VEC, SIMPLE, obstacles: one launch per step; long runs replay a captured CUDA graph of
+ *   AUTO on FP32 grids below 5 * 2^17 cells (temporal_steps = 0): launches of up to 8 steps, as
+ *             even as they come (lbm_sw_step_plan);
+ *   TEMPORAL with obstacles: the same with K = min(temporal_steps, 6), without odd counts (BGK and
+ *             an even temporal_steps; otherwise one launch per step);
+ *   VEC, SIMPLE: one launch per step; long runs replay a captured CUDA graph of
  *             graph_chunk steps.
  * Every mapping gives the same bits.  Errors: LBM_SW_E_ARG (n < 0), LBM_SW_E_STATE (no
  * state set), LBM_SW_E_CUDA (launch failure; kernel faults surface at the next
@@ -225,7 +227,8 @@ LBM_SW_API int lbm_sw_set_relaxation(lbm_sw* h, const double* rates, int count);
  * population, the momentum family normal to the face negated.  Solid cells hold no fluid:
  * they are not collided or streamed and keep the populations they hold (also through
  * lbm_sw_set_populations(PRE_COLLISION)); their moments still count in the diagnostics.
- * With obstacles every step runs an obstacle kernel, one step per launch: the vectorised row
+ * With obstacles FP32 handles take several steps per launch as lbm_sw_step says, in kernels that
+ * know the mask; other steps run an obstacle kernel, one step per launch: the vectorised row
  * kernel (warps with no solid cell near them take the plain path), or one thread per cell
  * when the params' kernel is SIMPLE; both give the same bits.  solid == NULL removes the
  * obstacles.  The adjoint does not support them.

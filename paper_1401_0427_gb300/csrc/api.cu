@@ -70,10 +70,19 @@ bool temporal_active(const lbm_sw* h) {
   return lbm::temporal_mrt_supported(h->p.bc, h->p.nx, h->temporal_k) && (large || !h->auto_kernel);
 }
 
+// Steps per fused launch with obstacles (FP32 BGK TEMPORAL handles with an even temporal_steps; 8
+// runs as 6), 0: one step per launch.
+int obstacle_k(const lbm_sw* h) {
+  if (!h->has_obstacles || h->p.dim != 2 || h->kernel != LBM_SW_KERNEL_TEMPORAL || h->p.precision != LBM_SW_FP32 ||
+      h->mrt || h->temporal_k % 2)
+    return 0;
+  return std::min(h->temporal_k, 6);
+}
+
 // Whether lbm_sw_step takes register tiles (tile2d.cu): AUTO without a wish for temporal_steps.
 bool tile_active(const lbm_sw* h) {
   return h->auto_kernel && h->p.temporal_steps == 0 && h->p.dim == 2 && h->p.precision == LBM_SW_FP32 &&
-         !h->has_obstacles && static_cast<long long>(h->p.nx) * h->p.ny < kTileCells;
+         static_cast<long long>(h->p.nx) * h->p.ny < kTileCells;
 }
 
 // The launches of n > 0 steps on register tiles, as even as they come: launch(steps) for each.
@@ -235,6 +244,7 @@ void lbm_sw_destroy(lbm_sw* h) {
   if (h->diag_out) cudaFree(h->diag_out);
   if (h->diag_host) cudaFreeHost(h->diag_host);
   if (h->solid) cudaFree(h->solid);
+  if (h->solid_flags) cudaFree(h->solid_flags);
   delete h;
 }
 
@@ -371,14 +381,33 @@ int lbm_sw_step(lbm_sw* h, int n) {
   if (n > 0 && tile_active(h))
     return for_tile_launches(h, n, [&](int k) {
       const auto a = args<float>(h, h->cur);
-      const cudaError_t e = k == 1 ? lbm::launch_step2d<float>(a, consts(h), LBM_SW_KERNEL_VEC, h->stream)
-                                   : lbm::launch_step2d_tile(a, consts(h), k, h->stream, h->sm_count);
+      const unsigned char* flags = h->has_obstacles ? h->solid_flags : nullptr;
+      const cudaError_t e = k == 1 ? launch_one_step(h, h->cur, h->stream)
+                                   : lbm::launch_step2d_tile(a, consts(h), k, flags, h->stream, h->sm_count);
       if (e != cudaSuccess) return cuda_fail(h, e, "tile step launch");
       h->cur ^= 1;
       h->steps_done += k;
       h->launches += 1;
       return static_cast<int>(LBM_SW_OK);
     });
+  if (const int ko = obstacle_k(h)) {
+    int plan[64];
+    while (n > 0) {
+      const int count = lbm::plan_launches(ko, false, n, plan, 64);
+      for (int i = 0; i < count; ++i) {
+        const int k = plan[i];
+        const cudaError_t e = k == 1 ? launch_one_step(h, h->cur, h->stream)
+                                     : lbm::launch_step2d_temporal_obstacle(args<float>(h, h->cur), consts(h),
+                                                                            h->solid_flags, k, h->stream, h->sm_count);
+        if (e != cudaSuccess) return cuda_fail(h, e, "obstacle step launch");
+        h->cur ^= 1;
+        n -= k;
+        h->steps_done += k;
+        h->launches += 1;
+      }
+    }
+    return LBM_SW_OK;
+  }
   if (temporal_active(h)) {
     int plan[64];
     while (n > 0) {
@@ -444,10 +473,11 @@ int lbm_sw_step_plan(const lbm_sw* h, int n, int* sizes, int max_sizes) {
     });
     return count;
   }
-  if (temporal_active(h)) {
+  const int ko = obstacle_k(h);
+  if (ko || temporal_active(h)) {
     int plan[64];
     while (n > 0) {
-      const int c = plan_fused_launches(h, n, plan, 64);
+      const int c = ko ? lbm::plan_launches(ko, false, n, plan, 64) : plan_fused_launches(h, n, plan, 64);
       for (int i = 0; i < c; ++i) {
         put(plan[i]);
         n -= plan[i];
@@ -671,6 +701,13 @@ int lbm_sw_set_obstacle(lbm_sw* h, const unsigned char* solid, int on_device) {
     if (!h->solid) LBM_CUDA(h, cudaMalloc(&h->solid, n), "cudaMalloc (obstacle mask)");
     LBM_CUDA(h, cudaMemcpyAsync(h->solid, solid, n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                                 h->stream), "obstacle mask copy");
+    if (h->p.precision == LBM_SW_FP32 && (h->auto_kernel || h->kernel == LBM_SW_KERNEL_TEMPORAL)) {
+      if (!h->solid_flags)
+        LBM_CUDA(h, cudaMalloc(&h->solid_flags, static_cast<size_t>(h->plane)), "cudaMalloc (obstacle flags)");
+      LBM_CUDA(h, lbm::launch_obstacle_flags(h->solid, h->solid_flags, h->p.nx, h->p.ny, h->pitch, h->p.bc, h->stream),
+               "obstacle flags launch");
+      h->launches += 1;
+    }
     // the caller may reuse its buffer when this returns
     LBM_CUDA(h, cudaStreamSynchronize(h->stream), "set_obstacle synchronize");
     h->has_obstacles = true;

@@ -120,10 +120,22 @@ bool temporal_mrt_supported(const int bc[4], int nx, int k);
 cudaError_t launch_step2d_temporal_mrt(const StepArgs<float>& a, const ConstsD& kd, int k, cudaStream_t st,
                                        int sm_count);
 
+// Flags of a cell for the fused steps with solid cells: itself, and its neighbours at x - 1, x + 1,
+// y - 1 and y + 1 (beyond a side that is not periodic: not solid, the side's own rule applies).  A
+// solid cell has only the first.  launch_obstacle_flags makes them ([ny][pitch] bytes) from a mask.
+constexpr unsigned kSolidSelf = 1, kSolidLeft = 2, kSolidRight = 4, kSolidBelow = 8, kSolidAbove = 16;
+// k (2, 4 or 6) fused BGK steps with solid cells (temporal_obstacle.cu).
+cudaError_t launch_obstacle_flags(const unsigned char* solid, unsigned char* flags, int nx, int ny, long long pitch,
+                                  const int bc[4], cudaStream_t st);
+cudaError_t launch_step2d_temporal_obstacle(const StepArgs<float>& a, const ConstsD& kd, const unsigned char* flags,
+                                            int k, cudaStream_t st, int sm_count);
+
 // kb (1 .. 8) fused steps on tiles held in registers (tile2d.cu; FP32, BGK or MRT, any sides and
 // sizes), and the steps per launch that take the least time per step on an nx x ny grid.
 int tile_steps(int nx, int ny, int sms);
-cudaError_t launch_step2d_tile(const StepArgs<float>& a, const ConstsD& kd, int kb, cudaStream_t st, int sms);
+// flags: of solid cells, or nullptr.
+cudaError_t launch_step2d_tile(const StepArgs<float>& a, const ConstsD& kd, int kb, const unsigned char* flags,
+                               cudaStream_t st, int sms);
 
 // ---- 1D launchers (kernels_1d.cu) ----
 template <class T>
@@ -187,6 +199,7 @@ struct lbm_sw {
   bool mrt = false;          // set by lbm_sw_set_relaxation
   double mrt_rates[10] = {};
   unsigned char* solid = nullptr;  // obstacle mask [ny][nx] on the device (lbm_sw_set_obstacle)
+  unsigned char* solid_flags = nullptr;  // [ny][pitch] bytes of the fused steps with obstacles
   bool has_obstacles = false;
   int graph_chunk = 64;
   bool has_state = false;

@@ -83,10 +83,24 @@ __host__ __device__ constexpr int reg_index(int p) {
 // code generator overlap a level's loads with the previous level's collision (BGK at K = 6
 // with 256 columns +1 %, MRT +1.4 %; BGK at K = 4 and with 128 columns measured slower and
 // keeps the tests).
+//
+// OBST: solid cells inside the domain (flags: [ny][pitch] bytes, kSolid*).  The rule of a
+// fluid-solid face: the population that would come from the solid cell takes the fluid cell's own
+// reflected one, the family normal to the face negated.  Along x the pull reads the cell's own
+// opposite mover in the same shared-memory row (another offset, as at a WALL side); along y the
+// value goes where the next level pulls it from: a cell above a solid one puts its -y movers into
+// the solid cell's +y movers (which nobody else pulls), and a solid cell's -y movers become the
+// +y movers of the row below it.  All by selects on the flags of the row's cells, which a thread
+// keeps for the last rows in one 64-bit word: branches at each level (a separate path for lanes
+// with flags, or for warps) split the levels' code and measured 1.3 to 2.1 times the time.  Solid
+// cells compute values that nothing pulls; their populations are copied from the source.
+
 template <int K, int COLS, int PF, bool STORE_W, bool L0R, bool PER = true, bool MRT = false, bool ODD = true,
-          bool U3 = false, bool STEADY = false>
+          bool U3 = false, bool STEADY = false, bool OBST = false>
 __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts<float>& Kc, float* smem, int x0, int w,
-                                          int ys, int ye, float* __restrict__ wout, long long wslot) {
+                                          int ys, int ye, float* __restrict__ wout, long long wslot,
+                                          const unsigned char* __restrict__ flags = nullptr) {
+  static_assert(!OBST || (K <= 7 && !STORE_W && L0R && ODD), "obstacles: one flag byte per row, level 0 in registers");
   using S = PairShape<K, COLS, PF, L0R>;
   constexpr int RS = S::RS;
   const int c = threadIdx.x;  // pair index: tile columns 2c, 2c + 1
@@ -183,8 +197,25 @@ __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts
     }
   }
   // the pulled x movers of family fam from the +x / -x planes at this pair
-  auto pull_x = [&](int fam, const float* px, const float* mx, float2* f) {
-    if constexpr (PER) {
+  // b: OBST, the row's flags (bits 0 .. 3 lane x, 4 .. 7 lane y)
+  auto flip = [](float v, unsigned b, unsigned bit) {  // -v where the bit of b is set
+    return __uint_as_float(__float_as_uint(v) ^ (b & bit ? 0x80000000u : 0u));
+  };
+  auto pull_x = [&](int fam, const float* px, const float* mx, float2* f, unsigned b) {
+    if constexpr (OBST) {
+      f[1 + 4 * fam] = make_float2(px[b & kSolidLeft ? RS : (PER ? -1 : o_p1)], px[b & kSolidLeft << 4 ? RS + 1 : 0]);
+      f[3 + 4 * fam] = make_float2(mx[b & kSolidRight ? -RS : (PER ? 1 : o_p3x)],
+                                   mx[b & kSolidRight << 4 ? 1 - RS : (PER ? 2 : o_p3)]);
+      if (fam == 1) {
+        if (!PER) {
+          f[5].x *= sgn1x;
+          f[7].x *= sgn3.x;
+          f[7].y *= sgn3.y;
+        }
+        f[5] = make_float2(flip(f[5].x, b, kSolidLeft), flip(f[5].y, b, kSolidLeft << 4));
+        f[7] = make_float2(flip(f[7].x, b, kSolidRight), flip(f[7].y, b, kSolidRight << 4));
+      }
+    } else if constexpr (PER) {
       f[1 + 4 * fam] = make_float2(px[-1], px[0]);
       f[3 + 4 * fam] = make_float2(mx[1], mx[2]);
     } else {
@@ -196,6 +227,18 @@ __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts
         f[7].y *= sgn3.y;
       }
     }
+  };
+  // OBST, y faces: a solid cell's -y movers (ym) become the reflected +y movers of the row below (yp1),
+  // a fluid cell's reflected -y movers go to the solid cell below it (yp1)
+  auto face_y = [&](int fam, float2& ym, float2& yp1, unsigned b) {
+    auto lane = [&](float& m, float& q, unsigned s) {
+      const float rm = fam == 2 ? -m : m, rq = fam == 2 ? -q : q;
+      const float m_new = b & kSolidSelf << s ? rq : m;
+      q = b & kSolidBelow << s ? rm : q;
+      m = m_new;
+    };
+    lane(ym.x, yp1.x, 0);
+    lane(ym.y, yp1.y, 4);
   };
   // y sides: from the edge row's own -y (p4) and +y (p2) movers, the +y movers of row -1 and
   // the -y movers of row ny.
@@ -222,10 +265,21 @@ __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts
   // periodic, +1.5 % with walls at K = 6).  MRT keeps one group per row (the split measured
   // 2-3 % slower there).
   constexpr bool SPLIT = !MRT;
+  unsigned long long fl = 0;  // OBST: flags of the rows landed so far, one byte each
+  unsigned fl_next[PF] = {};  // flags of the rows in flight
   auto issue_row = [&](int j) {
     const int r = ys - K + j;
     const int gr = py ? next_gr : r;
     if (py) next_gr = next_gr + 1 == ny ? 0 : next_gr + 1;
+    if constexpr (OBST) {
+#pragma unroll
+      for (int q = 0; q + 1 < PF; ++q) fl_next[q] = fl_next[q + 1];
+      fl_next[PF - 1] = 0;
+      if (j < iters && col_live && (py || (r >= 0 && r < ny))) {
+        const unsigned char* g = flags + static_cast<long long>(gr) * A.pitch;
+        fl_next[PF - 1] = (g[gx] & 15u) | (gx2 < nx ? (g[gx2] & 15u) << 4 : 0u);
+      }
+    }
     if constexpr (SPLIT) {
       const bool live = j < iters && col_live && (py || (r >= 0 && r < ny));
       const float* g = A.src + static_cast<long long>(gr) * A.pitch + gx;
@@ -323,10 +377,20 @@ __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts
         }
       }
     }
+    float2 a0[3];  // OBST: the landed row's -y movers
+    if constexpr (OBST) {
+      fl = (fl << 8) | fl_next[0];
+#pragma unroll
+      for (int fam = 0; fam < 3; ++fam) {
+        a0[fam] = ld2(l0a + (j % S::A0) * 3 * RS + col + 2 + fam * RS);
+        face_y(fam, a0[fam], cr[0][P1][fam], static_cast<unsigned>(fl));
+      }
+    }
     issue_row(j + PF);
 #pragma unroll
     for (int t = 1; t <= K; ++t) {
       const int R = ys - K + j - t;
+      const unsigned b = OBST ? static_cast<unsigned>(fl >> (8 * t)) & 255u : 0u;
       const bool row_ok = R >= ys - K + t && R < ye + K - t;
       const bool row_live = py || (R >= 0 && R < ny);
       if (FULL ? warp_live : (row_ok && row_live && col_live && col + 1 >= t && col < w + K + KL - t)) {
@@ -340,8 +404,8 @@ __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts
             const float* px = rb + (2 * fam) * RS;      // +x movers from columns 2c - 1, 2c
             const float* mx = rb + (2 * fam + 1) * RS;  // -x movers from columns 2c + 1, 2c + 2
             f[2 + 4 * fam] = cr[0][P2][fam];
-            f[4 + 4 * fam] = ld2(ra + fam * RS);
-            pull_x(fam, px, mx, f);
+            f[4 + 4 * fam] = OBST ? a0[fam] : ld2(ra + fam * RS);
+            pull_x(fam, px, mx, f, b);
           }
         } else if (t == 1) {
           const float* ra = l0a + (j % S::A0) * 3 * RS + col + 2;
@@ -354,7 +418,7 @@ __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts
             const float* mx = rb + (2 + 2 * fam) * RS;  // -x movers from columns 2c + 1, 2c + 2
             f[2 + 4 * fam] = ld2(rc + fam * RS);
             f[4 + 4 * fam] = ld2(ra + fam * RS);
-            pull_x(fam, px, mx, f);
+            pull_x(fam, px, mx, f, b);
           }
         } else {
           const float* x = xm(t - 1, (j + 1) & 1) + col + 2;
@@ -365,7 +429,7 @@ __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts
             const float* mx = x + (2 * fam + 1) * RS;
             f[2 + 4 * fam] = cr[t - 1][P2][fam];
             f[4 + 4 * fam] = a_now[t - 1][fam];
-            pull_x(fam, px, mx, f);
+            pull_x(fam, px, mx, f, b);
           }
         }
         float2 wh, wx, wy;
@@ -390,6 +454,7 @@ __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts
             st2(x + (2 * fam + 1) * RS, f[3 + 4 * fam]);
             a_now[t][fam] = f[4 + 4 * fam];
             cr[t][PH][fam] = f[2 + 4 * fam];
+            if constexpr (OBST) face_y(fam, a_now[t][fam], cr[t][P1][fam], b);
           }
           f0r[t][PH] = f[0];
           if constexpr (!PER) {
@@ -401,6 +466,14 @@ __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts
           }
         } else if (col >= KL && col < KL + w && gx_raw < nx) {
           float* g = A.dst + static_cast<long long>(R) * A.pitch + gx_raw;
+          if (OBST && (b & (kSolidSelf | kSolidSelf << 4))) {  // solid cells keep their populations
+            const float* o = A.src + static_cast<long long>(R) * A.pitch + gx_raw;
+#pragma unroll
+            for (int p = 0; p < 13; ++p) {
+              if (b & kSolidSelf) f[p].x = o[p * A.plane];
+              if (b & kSolidSelf << 4) f[p].y = o[p * A.plane + 1];
+            }
+          }
           if (!lane_y_out) {
 #pragma unroll
             for (int p = 0; p < 13; ++p) st2(g + p * A.plane, f[p]);

@@ -46,9 +46,12 @@ struct TilePart {
   int w, h, strips, segs, kb, hl;
 };
 
-template <int R, int NW, bool MRT, bool PER>
+// OBST: solid cells (kSolid* flags): a population that would come from a solid cell is the cell's
+// own reflected one, the family normal to the face negated; solid cells keep their populations.
+template <int R, int NW, bool MRT, bool PER, bool OBST>
 __global__ void __launch_bounds__(32 * NW, 1)
-    step2d_tile(const StepArgs<float> A, const Consts<float> Kc, const TilePart P) {
+    step2d_tile(const StepArgs<float> A, const Consts<float> Kc, const TilePart P,
+                const unsigned char* __restrict__ flags) {
   extern __shared__ __align__(16) float2 smem2[];
   float2(*const edge)[NW][2][3][32] = reinterpret_cast<float2(*)[NW][2][3][32]>(smem2);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -62,6 +65,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
   pdl_wait();
 
   float2 F[R][13];
+  unsigned solid[R];  // flags of the rows' two cells (bits 0 .. 4 and 8 .. 12)
   {
     int gx = tx, gx2 = tx + 1, gy = ty;
     if (px) {
@@ -80,6 +84,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
     for (int r = 0; r < R; ++r) {
       const bool live = col_live && ty + r < y1 + P.kb && (py || (gy >= 0 && gy < ny));
       const long long row = static_cast<long long>(gy) * A.pitch;
+      if (OBST) solid[r] = live ? flags[row + gx] | (gx2 < nx ? flags[row + gx2] << 8 : 0) : 0u;
       if (live && !split) {
 #pragma unroll
         for (int p = 0; p < 13; ++p)
@@ -156,8 +161,20 @@ __global__ void __launch_bounds__(32 * NW, 1)
             up.x = last ? (wyp ? (c == 2 ? -yp.x : yp.x) : oyp ? ym.x : ip) : up.x;
             up.y = last ? (wyp ? (c == 2 ? -yp.y : yp.y) : oyp ? ym.y : ip) : up.y;
           }
+          float lb = xp.x;
+          if constexpr (OBST) {
+            const unsigned q = solid[r];
+            l = q & kSolidLeft ? (c == 1 ? -xm.x : xm.x) : l;
+            lb = q & kSolidLeft << 8 ? (c == 1 ? -xm.y : xm.y) : lb;
+            mid = q & kSolidRight ? (c == 1 ? -xp.x : xp.x) : mid;
+            rr = q & kSolidRight << 8 ? (c == 1 ? -xp.y : xp.y) : rr;
+            dn.x = q & kSolidBelow ? (c == 2 ? -ym.x : ym.x) : dn.x;
+            dn.y = q & kSolidBelow << 8 ? (c == 2 ? -ym.y : ym.y) : dn.y;
+            up.x = q & kSolidAbove ? (c == 2 ? -yp.x : yp.x) : up.x;
+            up.y = q & kSolidAbove << 8 ? (c == 2 ? -yp.y : yp.y) : up.y;
+          }
           a[1 + 4 * c] = l;
-          b[1 + 4 * c] = xp.x;
+          b[1 + 4 * c] = lb;
           a[3 + 4 * c] = mid;
           b[3 + 4 * c] = rr;
           a[2 + 4 * c] = dn.x;
@@ -170,7 +187,10 @@ __global__ void __launch_bounds__(32 * NW, 1)
         collide13_any<float, MRT>(a, Kc, h, qx, qy);
         collide13_any<float, MRT>(b, Kc, h, qx, qy);
 #pragma unroll
-        for (int p = 0; p < 13; ++p) F[r][p] = make_float2(a[p], b[p]);
+        for (int p = 0; p < 13; ++p) {
+          F[r][p].x = OBST && (solid[r] & kSolidSelf) ? F[r][p].x : a[p];
+          F[r][p].y = OBST && (solid[r] & kSolidSelf << 8) ? F[r][p].y : b[p];
+        }
       }
     };
     using std::false_type;
@@ -249,13 +269,24 @@ TileChoice tile_choose(int nx, int ny, int kb, int sms) {
   return best;
 }
 
-template <int R, int NW, bool MRT>
-cudaError_t launch_tile(const StepArgs<float>& a, const ConstsD& kd, const TilePart& P, cudaStream_t st) {
-  const size_t smem = sizeof(float2) * 2 * NW * 2 * 3 * 32;
-  static_assert(sizeof(float2) * 2 * NW * 2 * 3 * 32 <= 48 * 1024, "dynamic shared memory without an attribute");
+template <int R, int NW, bool MRT, bool OBST>
+cudaError_t launch_tile(const StepArgs<float>& a, const ConstsD& kd, const TilePart& P, const unsigned char* flags,
+                        cudaStream_t st) {
+  constexpr size_t smem = sizeof(float2) * 2 * NW * 2 * 3 * 32;
+  static_assert(smem <= 48 * 1024, "dynamic shared memory without an attribute");
   const bool per = a.bc[LBM_SW_SIDE_XM] == LBM_SW_BC_PERIODIC && a.bc[LBM_SW_SIDE_YM] == LBM_SW_BC_PERIODIC;
-  return launch_pdl(per ? step2d_tile<R, NW, MRT, true> : step2d_tile<R, NW, MRT, false>, dim3(P.strips * P.segs),
-                    dim3(32 * NW), smem, st, a, to_consts<float>(kd), P);
+  return launch_pdl(per ? step2d_tile<R, NW, MRT, true, OBST> : step2d_tile<R, NW, MRT, false, OBST>,
+                    dim3(P.strips * P.segs), dim3(32 * NW), smem, st, a, to_consts<float>(kd), P, flags);
+}
+
+template <bool OBST>
+cudaError_t launch_tile_choice(const StepArgs<float>& a, const ConstsD& kd, const TileChoice& c,
+                               const unsigned char* flags, cudaStream_t st) {
+  if (c.tall)
+    return kd.mrt ? launch_tile<3, 16, true, OBST>(a, kd, c.P, flags, st)
+                  : launch_tile<4, 12, false, OBST>(a, kd, c.P, flags, st);
+  return kd.mrt ? launch_tile<2, 16, true, OBST>(a, kd, c.P, flags, st)
+                : launch_tile<2, 16, false, OBST>(a, kd, c.P, flags, st);
 }
 
 }  // namespace
@@ -273,11 +304,11 @@ int tile_steps(int nx, int ny, int sms) {
   return best;
 }
 
-cudaError_t launch_step2d_tile(const StepArgs<float>& a, const ConstsD& kd, int kb, cudaStream_t st, int sms) {
+cudaError_t launch_step2d_tile(const StepArgs<float>& a, const ConstsD& kd, int kb, const unsigned char* flags,
+                               cudaStream_t st, int sms) {
   if (kb < 1 || kb > 8) return cudaErrorInvalidValue;
   const TileChoice c = tile_choose(a.nx, a.ny, kb, std::max(sms, 1));
-  if (c.tall) return kd.mrt ? launch_tile<3, 16, true>(a, kd, c.P, st) : launch_tile<4, 12, false>(a, kd, c.P, st);
-  return kd.mrt ? launch_tile<2, 16, true>(a, kd, c.P, st) : launch_tile<2, 16, false>(a, kd, c.P, st);
+  return flags ? launch_tile_choice<true>(a, kd, c, flags, st) : launch_tile_choice<false>(a, kd, c, nullptr, st);
 }
 
 }  // namespace lbm
