@@ -387,15 +387,19 @@ typedef struct lbm_sw_tape_info {
   int interval;            /* steps between checkpoints */
   int checkpoints;         /* ceil(T / interval) */
   int recorded;            /* 1 after lbm_sw_forward_record */
-  size_t checkpoint_bytes; /* FP64 checkpoint storage */
-  size_t replay_bytes;     /* moments of one segment, two adjoint and two replay buffers */
+  size_t checkpoint_bytes; /* FP64 checkpoints at this interval (none are stored while the moments
+                              of every step take at most 4 GB: those are kept instead) */
+  size_t replay_bytes;     /* moments of one segment or of every step, adjoint, replay and staging
+                              buffers */
 } lbm_sw_tape_info;
 
 /* Tape for `steps` >= 1 steps of 2D handle h, checkpoints every `interval` steps
  * (0 = ceil(sqrt(steps))).  Errors: LBM_SW_E_ARG (1D handle, bad counts), LBM_SW_E_NOMEM. */
 LBM_SW_API int lbm_sw_tape_create(lbm_sw* h, int steps, int interval, lbm_sw_tape** out);
 
-/* Release a tape (synchronises the owner's stream).  NULL-safe. */
+/* Release a tape.  Its device memory is kept for the handle's next tape (one block per handle, 8 GB
+ * in the process; it is freed with the handle) or, where it is not kept, freed after the owner's
+ * stream is idle.  NULL-safe. */
 LBM_SW_API void lbm_sw_tape_destroy(lbm_sw_tape* t);
 
 /* Advance h by the tape's steps from its current state (its W^0 is the state at this

@@ -15,11 +15,12 @@
 // J_C^T psi = (1 - s) psi + s M^T (D^T psi): the adjoint step pulls psi = S^T Phi^n in
 // the reverse direction (the transposed boundary rules below), then applies this local
 // product; it needs the moments W^{n-1} only, so the replay of a segment keeps three
-// planes per step.  Checkpoints of F* every `interval` steps are stored in FP64 (exact
+// planes per step (all steps' where they fit).  Checkpoints of F* every `interval` steps are stored in FP64 (exact
 // for FP32 states, so the replay repeats the forward run bit for bit).
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -322,17 +323,68 @@ dim3 grid_for(int nx, int ny, dim3 block) {
   return dim3(gx, static_cast<unsigned>(gy < 65535 ? gy : 65535));
 }
 
+std::atomic<size_t> g_tape_kept{0};  // bytes kept by all handles
+
 }  // namespace
+
+void* TapeMemory::take(size_t need, size_t* got) {
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (mem) {
+      void* const m = mem;
+      const size_t b = bytes;
+      mem = nullptr;
+      bytes = 0;
+      g_tape_kept -= b;
+      if (b >= need && b / 2 <= need) {
+        *got = b;
+        return m;
+      }
+      cudaFree(m);
+    }
+  }
+  void* m = nullptr;
+  *got = need;
+  return cudaMalloc(&m, need) == cudaSuccess ? m : nullptr;
+}
+
+bool TapeMemory::give(void* m, size_t size) {
+  std::lock_guard<std::mutex> lock(mu);
+  if (closed || mem) return false;
+  if ((g_tape_kept += size) > kTapeKeepTotal) {
+    g_tape_kept -= size;
+    return false;
+  }
+  mem = m;
+  bytes = size;
+  return true;
+}
+
+void TapeMemory::close() {
+  std::lock_guard<std::mutex> lock(mu);
+  closed = true;
+  if (mem) {
+    cudaFree(mem);
+    g_tape_kept -= bytes;
+    mem = nullptr;
+  }
+}
+
 }  // namespace lbm
 
 struct lbm_sw_tape {
   const lbm_sw* owner = nullptr;
+  cudaStream_t stream = nullptr;
+  std::shared_ptr<lbm::TapeMemory> memory;  // the handle's
+  void* mem = nullptr;                      // one allocation, cut into the pointers below
+  size_t mem_bytes = 0, used_bytes = 0;
+  bool keep_all = false;  // moments of every step kept by the forward record: no checkpoints, no replay
   int steps = 0, interval = 0, checkpoints = 0;
   bool recorded = false;
   size_t state_elems = 0;  // 13 * plane
-  double* ckpt = nullptr;  // checkpoints * 13 * plane doubles
+  double* ckpt = nullptr;  // checkpoints * 13 * plane doubles (not with keep_all)
   void* wstore = nullptr;  // wslots * 3 * plane of T
-  int wslots = 0;           // interval, plus room for the last fused replay launch to run past it
+  int wslots = 0;           // interval, plus room for the last fused replay launch to run past it (keep_all: steps + 1)
   bool last_w = false;      // the moment slots hold the last segment's W (left by the forward record)
   void* phi[2] = {nullptr, nullptr};
   void* rep[2] = {nullptr, nullptr};
@@ -341,6 +393,9 @@ struct lbm_sw_tape {
 };
 
 namespace {
+
+// Moments of every step are kept up to this size (1.4 % of the device's memory).
+constexpr size_t kTapeMomentsMost = 4ull << 30;
 
 int tfail(lbm_sw_tape* t, int code, const char* fmt, ...) {
   char buf[512];
@@ -378,25 +433,27 @@ lbm::StepArgs<T> replay_args(const lbm_sw* h, const lbm_sw_tape* t, int from) {
   return a;
 }
 
-// The last segment of a forward record (len steps from the handle's state) run by the
-// kernels of a replay, which also keep W^{k0} .. W^{k0 + len} in the moment slots, so the
-// backward pass starts without replaying it.  The same updates as lbm_sw_step, so the same
-// state; FP32 handles that fuse steps only (their slots have room for the last launch).
+// A segment of a forward record (len steps from the handle's state) by the kernels of a replay,
+// which also keep W^{k0} .. W^{k0 + len} in the moment slots from W on, so the backward pass starts
+// without replaying it.  The same updates as lbm_sw_step, so the same state, and the same moments
+// as a replay's (W^{k0} from the stored populations, the others from the pulled ones).
 template <class T>
-int record_last_segment(lbm_sw* h, lbm_sw_tape* t, int len) {
+int record_with_moments(lbm_sw* h, lbm_sw_tape* t, int len, T* W) {
   cudaStream_t st = h->stream;
   const lbm::ConstsD kd = lbm::handle_consts(h);
   const long long P = h->plane;
-  T* W = static_cast<T*>(t->wstore);
   TAPE_CUDA(t, lbm::launch_moments2d_planes<T>(lbm::handle_args<T>(h, h->cur), W, st), "record moments");
   int from = h->cur, j = 1;
   long long launches = 1;
   if constexpr (sizeof(T) == 4) {
-    const int k = replay_k(h);
-    for (; j + k - 1 <= len; j += k, from ^= 1, ++launches)
-      TAPE_CUDA(t, lbm::launch_step2d_temporal_store_w(lbm::handle_args<T>(h, from), kd, k, W + 3 * P * j, 3 * P, st,
-                                                       h->sm_count),
-                "record launch");
+    // launches of the handle's K, then of 4 and 2 for the rest
+    int k = replay_k(h);
+    if (k > 1 && lbm::temporal_store_w_supported(lbm::handle_args<float>(h, 0), k))
+      for (; k >= 2; k = k > 4 ? 4 : k - 2)
+        for (; j + k - 1 <= len; j += k, from ^= 1, ++launches)
+          TAPE_CUDA(t, lbm::launch_step2d_temporal_store_w(lbm::handle_args<T>(h, from), kd, k, W + 3 * P * j, 3 * P, st,
+                                                           h->sm_count),
+                    "record launch");
   }
   for (; j <= len; ++j, from ^= 1, ++launches)
     TAPE_CUDA(t, lbm::launch_step2d_store_w<T>(lbm::handle_args<T>(h, from), kd, W + 3 * P * j, st), "record step");
@@ -416,16 +473,17 @@ int run_adjoint(lbm_sw* h, lbm_sw_tape* t, const double* gh, const double* gu, c
   const int nx = h->p.nx, ny = h->p.ny;
   const long long P = h->plane, pitch = h->pitch;
   const dim3 block(128, 2), grid = lbm::grid_for(nx, ny, block);
-  T* W = static_cast<T*>(t->wstore);
   int cur = 0;
   lbm::adjoint_terminal<T><<<grid, block, 0, st>>>(static_cast<T*>(t->phi[cur]), gh, gu, gv, nx, ny, pitch, P);
   TAPE_CUDA(t, cudaGetLastError(), "adjoint terminal launch");
   for (int seg = t->checkpoints - 1; seg >= 0; --seg) {
     const int k0 = seg * t->interval;
     const int k1 = (k0 + t->interval < t->steps) ? k0 + t->interval : t->steps;
+    T* const W = static_cast<T*>(t->wstore) + (t->keep_all ? 3 * P * k0 : 0);  // W^{k0}
     // replay the segment from its checkpoint, keeping W^{k0} .. W^{k1-1} (the forward record
-    // left them for the last segment)
-    if (seg == t->checkpoints - 1 && t->last_w) {
+    // left them for the last segment, with keep_all for every one)
+    if (t->keep_all) {
+    } else if (seg == t->checkpoints - 1 && t->last_w) {
       t->last_w = false;
     } else {
     TAPE_CUDA(t, lbm::launch_restore_moments2d<T>(t->ckpt + static_cast<size_t>(seg) * t->state_elems,
@@ -484,7 +542,8 @@ int run_adjoint(lbm_sw* h, lbm_sw_tape* t, const double* gh, const double* gu, c
       cur ^= 1;
     }
   }
-  lbm::adjoint_gradient<T><<<grid, block, 0, st>>>(static_cast<const T*>(t->phi[cur]), W, K, nx, ny, pitch, P, dh, du,
+  lbm::adjoint_gradient<T><<<grid, block, 0, st>>>(static_cast<const T*>(t->phi[cur]),
+                                                    static_cast<const T*>(t->wstore), K, nx, ny, pitch, P, dh, du,
                                                     dv);
   TAPE_CUDA(t, cudaGetLastError(), "adjoint gradient launch");
   return LBM_SW_OK;
@@ -496,14 +555,10 @@ extern "C" {
 
 void lbm_sw_tape_destroy(lbm_sw_tape* t) {
   if (!t) return;
-  if (t->owner) cudaStreamSynchronize(t->owner->stream);
-  if (t->ckpt) cudaFree(t->ckpt);
-  if (t->wstore) cudaFree(t->wstore);
-  for (int i = 0; i < 2; ++i) {
-    if (t->phi[i]) cudaFree(t->phi[i]);
-    if (t->rep[i]) cudaFree(t->rep[i]);
+  if (t->mem && !(t->memory && t->memory->give(t->mem, t->mem_bytes))) {
+    cudaStreamSynchronize(t->stream);
+    cudaFree(t->mem);
   }
-  if (t->grad_staging) cudaFree(t->grad_staging);
   delete t;
 }
 
@@ -541,19 +596,38 @@ int lbm_sw_tape_create(lbm_sw* h, int steps, int interval, lbm_sw_tape** out) {
     t->interval = std::min(steps, round_both <= 2 * iv ? round_both : (iv + k - 1) / k * k);
   }
   t->checkpoints = (steps + t->interval - 1) / t->interval;
-  // a replay that fuses k steps per launch may run up to k - 1 steps past its segment
-  t->wslots = t->interval + replay_k(h);
+  t->stream = h->stream;
+  t->memory = h->tape_memory;
   t->state_elems = static_cast<size_t>(13) * h->plane;
   const size_t n = static_cast<size_t>(h->p.nx) * h->p.ny;
-  bool ok = cudaMalloc(&t->ckpt, sizeof(double) * t->state_elems * t->checkpoints) == cudaSuccess &&
-            cudaMalloc(&t->wstore, h->elem * 3 * h->plane * t->wslots) == cudaSuccess &&
-            cudaMalloc(&t->grad_staging, sizeof(double) * 3 * n) == cudaSuccess;
-  for (int i = 0; i < 2 && ok; ++i)
-    ok = cudaMalloc(&t->phi[i], h->elem * t->state_elems) == cudaSuccess &&
-         cudaMemsetAsync(t->phi[i], 0, h->elem * t->state_elems, h->stream) == cudaSuccess &&
-         cudaMalloc(&t->rep[i], h->elem * t->state_elems) == cudaSuccess &&
-         cudaMemsetAsync(t->rep[i], 0, h->elem * t->state_elems, h->stream) == cudaSuccess;
-  if (ok) ok = cudaMemsetAsync(t->wstore, 0, h->elem * 3 * h->plane * t->wslots, h->stream) == cudaSuccess;
+  const size_t slot = static_cast<size_t>(h->elem) * 3 * h->plane, state = static_cast<size_t>(h->elem) * t->state_elems;
+  // The moments of every step where they take little memory: the record then writes them as it
+  // goes, and the backward pass replays nothing (1024^2 FP32, 200 steps, 2.5 GB: record and adjoint
+  // 1.5 + 3.8 ms with checkpoints every 24 steps, 1.6 + 2.0 ms this way).
+  // Without room for them: checkpoints.
+  void** const parts[7] = {reinterpret_cast<void**>(&t->ckpt), &t->wstore, reinterpret_cast<void**>(&t->grad_staging),
+                           &t->phi[0], &t->phi[1], &t->rep[0], &t->rep[1]};
+  bool ok = false;
+  for (int all = (static_cast<size_t>(steps) + 1) * slot <= kTapeMomentsMost; !ok && all >= 0; --all) {
+    t->keep_all = all == 1;
+    // a replay that fuses k steps per launch may run up to k - 1 steps past its segment
+    t->wslots = t->keep_all ? steps + 1 : t->interval + replay_k(h);
+    const size_t sizes[7] = {t->keep_all ? 0 : sizeof(double) * t->state_elems * t->checkpoints, slot * t->wslots,
+                             sizeof(double) * 3 * n, state, state, t->keep_all ? 0 : state, t->keep_all ? 0 : state};
+    t->used_bytes = 0;
+    for (size_t s : sizes) t->used_bytes += (s + 255) / 256 * 256;
+    t->mem = t->memory->take(t->used_bytes, &t->mem_bytes);
+    ok = t->mem != nullptr;
+    char* at = static_cast<char*>(t->mem);
+    for (int i = 0; i < 7 && ok; ++i) {
+      *parts[i] = sizes[i] ? at : nullptr;
+      at += (sizes[i] + 255) / 256 * 256;
+    }
+  }
+  // the rows' padding is zero (it is loaded with the last cells of a row)
+  if (h->pitch != h->p.nx)
+    for (void* b : {t->phi[0], t->phi[1], t->rep[0], t->rep[1]})
+      if (ok && b) ok = cudaMemsetAsync(b, 0, state, h->stream) == cudaSuccess;
   if (!ok) {
     h->err = std::string("tape_create: device allocation failed: ") + cudaGetErrorString(cudaGetLastError());
     lbm_sw_tape_destroy(t);
@@ -573,6 +647,15 @@ int lbm_sw_forward_record(lbm_sw* h, lbm_sw_tape* t) {
   // temporal blocking (bit-identical to single steps)
   for (int seg = 0; seg < t->checkpoints; ++seg) {
     const int k0 = seg * t->interval;
+    if (t->keep_all) {
+      const int n = std::min(t->interval, t->steps - k0);
+      const size_t at = static_cast<size_t>(3) * h->plane * k0;
+      const int rc = h->p.precision == LBM_SW_FP64
+                         ? record_with_moments<double>(h, t, n, static_cast<double*>(t->wstore) + at)
+                         : record_with_moments<float>(h, t, n, static_cast<float*>(t->wstore) + at);
+      if (rc != LBM_SW_OK) return rc;
+      continue;
+    }
     double* dst = t->ckpt + static_cast<size_t>(seg) * t->state_elems;
     cudaError_t e = h->p.precision == LBM_SW_FP64
                         ? lbm::launch_convert<double, double>(static_cast<const double*>(h->buf[h->cur]), dst,
@@ -583,7 +666,7 @@ int lbm_sw_forward_record(lbm_sw* h, lbm_sw_tape* t) {
     const int len = std::min(t->interval, t->steps - k0);
     if (seg == t->checkpoints - 1 && h->p.precision == LBM_SW_FP32 && replay_k(h) > 1 &&
         lbm::temporal_store_w_supported(lbm::handle_args<float>(h, 0), replay_k(h))) {
-      const int rc = record_last_segment<float>(h, t, len);
+      const int rc = record_with_moments<float>(h, t, len, static_cast<float*>(t->wstore));
       if (rc != LBM_SW_OK) return rc;
     } else {
       t->last_w = false;
@@ -637,7 +720,7 @@ int lbm_sw_tape_get_info(const lbm_sw_tape* t, lbm_sw_tape_info* out) {
   out->checkpoints = t->checkpoints;
   out->recorded = t->recorded ? 1 : 0;
   out->checkpoint_bytes = sizeof(double) * t->state_elems * t->checkpoints;
-  out->replay_bytes = t->owner->elem * (3 * t->owner->plane * t->wslots + 4 * t->state_elems);
+  out->replay_bytes = t->used_bytes - (t->keep_all ? 0 : out->checkpoint_bytes);
   return LBM_SW_OK;
 }
 

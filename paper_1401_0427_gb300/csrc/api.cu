@@ -235,6 +235,7 @@ void lbm_sw_destroy(lbm_sw* h) {
     if (h->graph[i]) cudaGraphExecDestroy(h->graph[i]);
     if (h->buf[i]) cudaFree(h->buf[i]);
   }
+  h->tape_memory->close();
   if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
   if (h->inflow_feq) cudaFree(h->inflow_feq);
   if (h->moments_staging) cudaFree(h->moments_staging);

@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <memory>
+#include <mutex>
 #include <string>
 
 #include "../../include/lbm_sw.h"
@@ -173,6 +175,23 @@ template <class T>
 cudaError_t launch_diagnostics_blocks(const StepArgs<T>& a, int q, int nblocks, double* partials, double* out,
                                       cudaStream_t st);
 
+// Device memory of a destroyed tape, kept for the next tape of the same handle (an optimiser makes
+// one per gradient, and allocating and freeing gigabytes takes milliseconds).  At most one block
+// per handle and kTapeKeepTotal bytes in the process; freed with the handle, or when a tape that it
+// does not fit is made.  Work of the old tape and of the next one is ordered by the handle's
+// stream.  The handle and its tapes share it: a tape may be destroyed after its handle, and in
+// another thread.
+constexpr size_t kTapeKeepTotal = 8ull << 30;
+struct TapeMemory {
+  std::mutex mu;
+  void* mem = nullptr;
+  size_t bytes = 0;
+  bool closed = false;       // the handle is gone: nothing is kept any more
+  void* take(size_t need, size_t* got);  // kept or new memory of at least `need` bytes, nullptr if there is none
+  bool give(void* m, size_t size);       // true if kept, else the caller frees it
+  void close();
+};
+
 }  // namespace lbm
 
 struct lbm_sw {
@@ -208,6 +227,7 @@ struct lbm_sw {
   cudaStream_t capture_stream = nullptr;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // CUDA graph of graph_chunk steps from buffer 0 / 1
   std::string err;
+  std::shared_ptr<lbm::TapeMemory> tape_memory = std::make_shared<lbm::TapeMemory>();
 };
 
 namespace lbm {
