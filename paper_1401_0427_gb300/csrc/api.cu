@@ -125,6 +125,37 @@ cudaError_t launch_one_step(lbm_sw* h, int from, cudaStream_t st) {
                        : lbm::launch_step2d<float>(a, consts(h), variant, st);
 }
 
+// Rows of every plane between the state (src, dst: its first row) and a dense array: a kernel on the
+// device, a 2D copy per plane from or to the host.
+cudaError_t planes_out(lbm_sw* h, const char* src, void* dst, size_t row, size_t dplane, int rows, int on_device) {
+  const long long pitch = h->pitch * static_cast<long long>(h->elem), plane = h->plane * static_cast<long long>(h->elem);
+  if (on_device) {
+    h->launches += 1;
+    return lbm::copy_planes({src, pitch, plane, dst, static_cast<long long>(row), static_cast<long long>(dplane),
+                             static_cast<long long>(row), rows, h->q}, h->elem, h->stream);
+  }
+  for (int p = 0; p < h->q; ++p) {
+    const cudaError_t e = cudaMemcpy2DAsync(static_cast<char*>(dst) + p * dplane, row, src + p * plane, pitch, row, rows,
+                                            cudaMemcpyDeviceToHost, h->stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+cudaError_t planes_in(lbm_sw* h, char* dst, const void* src, size_t row, size_t dplane, int rows, int on_device) {
+  const long long pitch = h->pitch * static_cast<long long>(h->elem), plane = h->plane * static_cast<long long>(h->elem);
+  if (on_device) {
+    h->launches += 1;
+    return lbm::copy_planes({src, static_cast<long long>(row), static_cast<long long>(dplane), dst, pitch, plane,
+                             static_cast<long long>(row), rows, h->q}, h->elem, h->stream);
+  }
+  for (int p = 0; p < h->q; ++p) {
+    const cudaError_t e = cudaMemcpy2DAsync(dst + p * plane, pitch, static_cast<const char*>(src) + p * dplane, row, row,
+                                            rows, cudaMemcpyHostToDevice, h->stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // Capture graph_chunk steps starting from buffer `from` (graph_chunk is even, so the
 // chunk ends in the buffer it started from).
 int build_graph(lbm_sw* h, int from) {
@@ -545,12 +576,8 @@ int lbm_sw_get_populations(lbm_sw* h, void* dst, int on_device) {
   if (!h->has_state) return fail(h, LBM_SW_E_STATE, "get_populations: no state set");
   const size_t row = static_cast<size_t>(h->p.nx) * h->elem;
   const size_t dplane = row * h->p.ny;
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   const char* src = static_cast<const char*>(h->buf[h->cur]);
-  for (int p = 0; p < h->q; ++p)
-    LBM_CUDA(h, cudaMemcpy2DAsync(static_cast<char*>(dst) + p * dplane, row, src + p * h->plane * h->elem,
-                                  h->pitch * h->elem, row, h->p.ny, kind, h->stream),
-             "copy populations out");
+  LBM_CUDA(h, planes_out(h, src, dst, row, dplane, h->p.ny, on_device), "copy populations out");
   if (!on_device) LBM_CUDA(h, cudaStreamSynchronize(h->stream), "get_populations synchronize");
   return LBM_SW_OK;
 }
@@ -562,13 +589,9 @@ int lbm_sw_set_populations(lbm_sw* h, const void* src, int on_device, int form) 
     return fail(h, LBM_SW_E_ARG, "set_populations: form must be LBM_SW_POST_COLLISION or LBM_SW_PRE_COLLISION");
   const size_t row = static_cast<size_t>(h->p.nx) * h->elem;
   const size_t dplane = row * h->p.ny;
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   if (form == LBM_SW_POST_COLLISION) {
     char* dst = static_cast<char*>(h->buf[h->cur]);
-    for (int p = 0; p < h->q; ++p)
-      LBM_CUDA(h, cudaMemcpy2DAsync(dst + p * h->plane * h->elem, h->pitch * h->elem,
-                                    static_cast<const char*>(src) + p * dplane, row, row, h->p.ny, kind, h->stream),
-               "copy populations in");
+    LBM_CUDA(h, planes_in(h, dst, src, row, dplane, h->p.ny, on_device), "copy populations in");
   } else {
     const void* dense = src;
     if (!on_device) {
@@ -608,11 +631,7 @@ int lbm_sw_get_rows(lbm_sw* h, int y0, int nrows, void* dst, int on_device) {
   const size_t row = static_cast<size_t>(h->p.nx) * h->elem;
   const size_t dplane = row * nrows;
   const char* src = static_cast<const char*>(h->buf[h->cur]) + static_cast<size_t>(y0) * h->pitch * h->elem;
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  for (int p = 0; p < h->q; ++p)
-    LBM_CUDA(h, cudaMemcpy2DAsync(static_cast<char*>(dst) + p * dplane, row, src + p * h->plane * h->elem,
-                                  h->pitch * h->elem, row, nrows, kind, h->stream),
-             "copy rows out");
+  LBM_CUDA(h, planes_out(h, src, dst, row, dplane, nrows, on_device), "copy rows out");
   if (!on_device) LBM_CUDA(h, cudaStreamSynchronize(h->stream), "get_rows synchronize");
   return LBM_SW_OK;
 }
@@ -628,11 +647,7 @@ int lbm_sw_set_rows(lbm_sw* h, int y0, int nrows, const void* src, int on_device
   const size_t row = static_cast<size_t>(h->p.nx) * h->elem;
   const size_t dplane = row * nrows;
   char* dst = static_cast<char*>(h->buf[h->cur]) + static_cast<size_t>(y0) * h->pitch * h->elem;
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  for (int p = 0; p < h->q; ++p)
-    LBM_CUDA(h, cudaMemcpy2DAsync(dst + p * h->plane * h->elem, h->pitch * h->elem,
-                                  static_cast<const char*>(src) + p * dplane, row, row, nrows, kind, h->stream),
-             "copy rows in");
+  LBM_CUDA(h, planes_in(h, dst, src, row, dplane, nrows, on_device), "copy rows in");
   if (!on_device) LBM_CUDA(h, cudaStreamSynchronize(h->stream), "set_rows synchronize");
   return LBM_SW_OK;
 }

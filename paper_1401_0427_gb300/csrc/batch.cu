@@ -548,11 +548,18 @@ int lbm_sw_batch_get_populations(lbm_sw_batch* b, int i, void* dst, int on_devic
   const lbm::BatchInst& I = b->inst[i];
   const size_t row = static_cast<size_t>(I.nx) * b->elem, dplane = row * I.ny;
   const char* src = static_cast<const char*>(b->buf[b->cur]) + I.offset * b->elem;
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  for (int p = 0; p < 13; ++p)
-    BATCH_CUDA(b, cudaMemcpy2DAsync(static_cast<char*>(dst) + p * dplane, row, src + p * I.plane * b->elem,
-                                    I.pitch * b->elem, row, I.ny, kind, b->stream),
+  if (on_device)
+    BATCH_CUDA(b,
+               lbm::copy_planes({src, static_cast<long long>(I.pitch * b->elem), static_cast<long long>(I.plane * b->elem),
+                                 dst, static_cast<long long>(row), static_cast<long long>(dplane),
+                                 static_cast<long long>(row), I.ny, 13},
+                                b->elem, b->stream),
                "copy populations out");
+  else
+    for (int p = 0; p < 13; ++p)
+      BATCH_CUDA(b, cudaMemcpy2DAsync(static_cast<char*>(dst) + p * dplane, row, src + p * I.plane * b->elem,
+                                      I.pitch * b->elem, row, I.ny, cudaMemcpyDeviceToHost, b->stream),
+                 "copy populations out");
   if (!on_device) BATCH_CUDA(b, cudaStreamSynchronize(b->stream), "get_populations synchronize");
   return LBM_SW_OK;
 }

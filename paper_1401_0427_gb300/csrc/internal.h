@@ -66,6 +66,18 @@ cudaError_t launch_restore_moments2d(const double* ck, const StepArgs<T>& a, T* 
 template <class Tin, class Tout>
 cudaError_t launch_convert(const Tin* in, Tout* out, long long n, cudaStream_t st);
 
+// Device-to-device copy of `rows` rows of each of `planes` planes (pitches and planes in bytes) of
+// elements of `elem` (4 or 8) bytes.
+struct PlaneCopy {
+  const void* src;
+  long long src_pitch, src_plane;
+  void* dst;
+  long long dst_pitch, dst_plane;
+  long long row_bytes;
+  int rows, planes;
+};
+cudaError_t copy_planes(const PlaneCopy& c, size_t elem, cudaStream_t st);
+
 // K reverse steps of the discrete adjoint per launch (adjoint_temporal.cu; FP32; every side
 // periodic with k in {2, 4, 6, 8}, or any sides with an even nx and k in {2, 4}): Phi^{n0}
 // in a.src -> Phi^{n0 - k} in a.dst; reverse step t reads the moments W^{n0 - t} at

@@ -275,6 +275,39 @@ __global__ void restore_moments2d(const double* __restrict__ ck, const StepArgs<
   }
 }
 
+// Rows of all planes between two layouts on the device (a pitched state and a dense array): V
+// elements of the word type per access, a thread kWords of them, kCopyThreads apart.
+constexpr int kCopyThreads = 128, kCopyWords = 4;
+template <class V>
+__global__ void __launch_bounds__(kCopyThreads)
+    copy_planes_kernel(const V* __restrict__ src, long long src_pitch, long long src_plane, V* __restrict__ dst,
+                       long long dst_pitch, long long dst_plane, int words, int rows) {
+  const int x0 = blockIdx.x * (kCopyThreads * kCopyWords) + threadIdx.x;
+  src += blockIdx.z * src_plane;
+  dst += blockIdx.z * dst_plane;
+  for (int y = blockIdx.y; y < rows; y += gridDim.y) {
+    V v[kCopyWords];
+#pragma unroll
+    for (int i = 0; i < kCopyWords; ++i)
+      if (x0 + i * kCopyThreads < words) v[i] = src[y * src_pitch + x0 + i * kCopyThreads];
+#pragma unroll
+    for (int i = 0; i < kCopyWords; ++i)
+      if (x0 + i * kCopyThreads < words) dst[y * dst_pitch + x0 + i * kCopyThreads] = v[i];
+  }
+}
+
+template <class V>
+cudaError_t copy_planes_as(const PlaneCopy& c, cudaStream_t st) {
+  const int e = static_cast<int>(sizeof(V));
+  const int words = static_cast<int>(c.row_bytes / e);
+  const dim3 grid((words + kCopyThreads * kCopyWords - 1) / (kCopyThreads * kCopyWords),
+                  static_cast<unsigned>(std::min(c.rows, 65535)), static_cast<unsigned>(c.planes));
+  copy_planes_kernel<V><<<grid, kCopyThreads, 0, st>>>(static_cast<const V*>(c.src), c.src_pitch / e, c.src_plane / e,
+                                                        static_cast<V*>(c.dst), c.dst_pitch / e, c.dst_plane / e, words,
+                                                        c.rows);
+  return cudaGetLastError();
+}
+
 template <class Tin, class Tout>
 __global__ void convert_kernel(const Tin* __restrict__ in, Tout* __restrict__ out, long long n) {
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
@@ -310,6 +343,27 @@ dim3 cell_grid(int nx, int ny, dim3 block) {
 }
 
 }  // namespace
+
+// One kernel for all planes (a 2D copy per plane costs a launch of 2 to 3 us each: the 13 planes of
+// a 64 x 64 state 33 us, against 3), in 16-byte words where every row of both sides starts on 16
+// bytes, else in 4- or 8-byte words; addresses that are not aligned to those by 2D copies.
+cudaError_t copy_planes(const PlaneCopy& c, size_t elem, cudaStream_t st) {
+  auto aligned = [&](size_t a) {
+    return reinterpret_cast<size_t>(c.src) % a == 0 && reinterpret_cast<size_t>(c.dst) % a == 0 && c.row_bytes % a == 0 &&
+           c.src_pitch % a == 0 && c.dst_pitch % a == 0 && c.src_plane % a == 0 && c.dst_plane % a == 0;
+  };
+  if (c.rows < 1 || c.row_bytes < 1) return cudaSuccess;
+  if (aligned(16)) return copy_planes_as<uint4>(c, st);
+  if (elem == 8 && aligned(8)) return copy_planes_as<unsigned long long>(c, st);
+  if (elem == 4 && aligned(4)) return copy_planes_as<unsigned>(c, st);
+  for (int p = 0; p < c.planes; ++p) {
+    const cudaError_t e = cudaMemcpy2DAsync(static_cast<char*>(c.dst) + p * c.dst_plane, c.dst_pitch,
+                                            static_cast<const char*>(c.src) + p * c.src_plane, c.src_pitch, c.row_bytes,
+                                            c.rows, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
 
 template <class T>
 cudaError_t launch_step2d(const StepArgs<T>& a, const ConstsD& kd, int variant, cudaStream_t st) {
