@@ -677,48 +677,95 @@ cudaError_t batch_launch(const BatchWaves& w, const float* src, float* dst, cons
   return cudaGetLastError();
 }
 
-// Units of the given instances at strip width <= wmax (even widths when `even`), balanced
-// longest-first over `grid` CTAs; uploads them and the per-CTA ranges.
-cudaError_t build_list(const std::vector<int>& ids, const int* nx, const int* ny, const long long* offset,
-                       const long long* pitch, const long long* plane, int k, int wmax, bool even, int grid,
-                       WaveUnit** d_units, int** d_first, int* count) {
-  // row segments of about a sixth of a CTA's share of the strip rows, no shorter than 4k
-  long long strip_rows = 0;
-  for (int i : ids) strip_rows += static_cast<long long>((nx[i] + wmax - 1) / wmax) * ny[i];
-  const long long target = std::max<long long>(4LL * k, (strip_rows + 6LL * grid - 1) / (6LL * grid));
-  std::vector<WaveUnit> units;
-  std::vector<long long> cost;
+// A work list: the units of all CTAs, and where each CTA's begin.
+struct UnitList {
+  std::vector<WaveUnit> sorted;
+  std::vector<int> first;
+};
+
+// Whole strips (width <= wmax, even widths when `even`) of the given instances.
+std::vector<WaveUnit> batch_strips(const std::vector<int>& ids, const int* nx, const int* ny, const long long* offset,
+                                   const long long* pitch, const long long* plane, int wmax, bool even) {
+  std::vector<WaveUnit> strips;
   for (int i : ids) {
-    int strips = (nx[i] + wmax - 1) / wmax;
-    int w = (nx[i] + strips - 1) / strips;
+    int n = (nx[i] + wmax - 1) / wmax;
+    int w = (nx[i] + n - 1) / n;
     if (even) {
       w += w & 1;  // <= wmax, which is even
-      strips = (nx[i] + w - 1) / w;
+      n = (nx[i] + w - 1) / w;
     }
-    const int segs = static_cast<int>(std::max<long long>(1, (ny[i] + target - 1) / target));
-    const int rows = (ny[i] + segs - 1) / segs;
-    for (int sgi = 0; sgi < segs; ++sgi)
-      for (int st = 0; st < strips; ++st) {
-        WaveUnit u;
-        u.offset = offset[i];
-        u.plane = plane[i];
-        u.pitch = static_cast<int>(pitch[i]);
-        u.nx = nx[i];
-        u.ny = ny[i];
-        u.x0 = st * w;
-        u.w = w;
-        u.ys = sgi * rows;
-        u.ye = std::min(ny[i], u.ys + rows);
-        u.pad = 0;
-        if (u.ys >= u.ye) continue;
-        units.push_back(u);
-        cost.push_back(static_cast<long long>(u.ye - u.ys + 2 * k) * (std::min(w, nx[i] - u.x0) + 2 * k));
+    for (int s = 0; s < n; ++s)
+      strips.push_back({offset[i], plane[i], static_cast<int>(pitch[i]), nx[i], ny[i], s * w, w, 0, ny[i], 0});
+  }
+  return strips;
+}
+
+// The strips laid end to end and cut where a CTA's share ends: little fill, and every CTA ends at
+// the same time.  An iteration costs a CTA the same whatever the strip's width, and a unit 2k rows
+// of fill and a start besides its rows, so the share is the least number of iterations T for which
+// filling one CTA after the other takes at most `grid` of them.
+UnitList cut_strips(const std::vector<WaveUnit>& strips, int k, int grid) {
+  UnitList out;
+  const int fill = 2 * k + 4, least = k;  // rows of fill and start per unit; rows of a unit, at least
+  auto cut = [&](long long T, bool keep) {
+    int ctas = 0;
+    long long room = 0;
+    for (const WaveUnit& s : strips) {
+      for (int y = 0; y < s.ye;) {
+        const int left = s.ye - y;
+        if (room < fill + std::min(left, least)) {  // the next CTA
+          if (keep) out.first.push_back(static_cast<int>(out.sorted.size()));
+          ++ctas;
+          room = T;
+        }
+        int rows = static_cast<int>(std::min<long long>(left, room - fill));
+        if (left - rows > 0 && left - rows < least && rows >= 2 * least) rows = left - least;
+        if (keep) {
+          out.sorted.push_back(s);
+          out.sorted.back().ys = y;
+          out.sorted.back().ye = y + rows;
+        }
+        room -= fill + rows;
+        y += rows;
+      }
+    }
+    return ctas;
+  };
+  long long lo = fill + least, hi = lo;
+  for (const WaveUnit& s : strips) hi += fill + s.ye;
+  while (lo < hi) {
+    const long long mid = (lo + hi) / 2;
+    if (cut(mid, false) <= grid)
+      hi = mid;
+    else
+      lo = mid + 1;
+  }
+  cut(lo, true);
+  out.first.resize(grid + 1, static_cast<int>(out.sorted.size()));
+  return out;
+}
+
+// Row segments of at most `target` rows, those of the strips of an instance next to one another,
+// longest first onto the least loaded CTA: neighbouring strips tend to run at the same time and to
+// share their halo columns in L2.
+UnitList deal_segments(const std::vector<WaveUnit>& strips, int k, int grid, long long target) {
+  std::vector<WaveUnit> units;
+  for (size_t a = 0, b; a < strips.size(); a = b) {
+    for (b = a + 1; b < strips.size() && strips[b].offset == strips[a].offset;) ++b;
+    const int ny = strips[a].ny;
+    const int segs = static_cast<int>(std::max<long long>(1, (ny + target - 1) / target));
+    const int rows = (ny + segs - 1) / segs;
+    for (int y = 0; y < ny; y += rows)
+      for (size_t s = a; s < b; ++s) {
+        units.push_back(strips[s]);
+        units.back().ys = y;
+        units.back().ye = std::min(ny, y + rows);
       }
   }
-  // longest-processing-time-first onto the least loaded CTA
   std::vector<int> order(units.size());
   for (size_t u = 0; u < order.size(); ++u) order[u] = static_cast<int>(u);
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+  auto cost = [&](int u) { return static_cast<long long>(units[u].ye - units[u].ys + 2 * k); };
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(x) > cost(y); });
   using Load = std::pair<long long, int>;
   std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
   for (int b = 0; b < grid; ++b) heap.push({0, b});
@@ -727,16 +774,32 @@ cudaError_t build_list(const std::vector<int>& ids, const int* nx, const int* ny
     Load l = heap.top();
     heap.pop();
     per[l.second].push_back(u);
-    heap.push({l.first + cost[u], l.second});
+    heap.push({l.first + cost(u), l.second});
   }
-  std::vector<WaveUnit> sorted;
-  std::vector<int> first(grid + 1, 0);
-  sorted.reserve(units.size());
+  UnitList out;
   for (int b = 0; b < grid; ++b) {
-    first[b] = static_cast<int>(sorted.size());
-    for (int u : per[b]) sorted.push_back(units[u]);
+    out.first.push_back(static_cast<int>(out.sorted.size()));
+    for (int u : per[b]) out.sorted.push_back(units[u]);
   }
-  first[grid] = static_cast<int>(sorted.size());
+  out.first.push_back(static_cast<int>(out.sorted.size()));
+  return out;
+}
+
+// The work list of the given instances over `grid` CTAs, uploaded.  Shares of 120 k rows or more
+// per CTA are dealt as segments of a sixth, whose fill is then below a tenth; smaller ones are cut
+// end to end.  MLUPS dealt (by cells, as narrow strips do not cost) / cut: 64 grids of sides 64 to
+// 1024 199k / 224k, 8 of 500 x 400 113k / 177k, 16 of about 150 x 130 52k / 81k; 256 grids of sides
+// 64 to 1024 231k by cells, 247k by rows, 223k cut.
+cudaError_t build_list(const std::vector<int>& ids, const int* nx, const int* ny, const long long* offset,
+                       const long long* pitch, const long long* plane, int k, int wmax, bool even, int grid,
+                       WaveUnit** d_units, int** d_first, int* count) {
+  const std::vector<WaveUnit> strips = batch_strips(ids, nx, ny, offset, pitch, plane, wmax, even);
+  long long rows = 0;
+  for (const WaveUnit& s : strips) rows += s.ny;
+  const long long share = (rows + grid - 1) / grid;
+  const UnitList list = share >= 120LL * k ? deal_segments(strips, k, grid, (share + 5) / 6) : cut_strips(strips, k, grid);
+  const std::vector<WaveUnit>& sorted = list.sorted;
+  const std::vector<int>& first = list.first;
   cudaError_t e = cudaMalloc(d_units, std::max<size_t>(1, sorted.size()) * sizeof(WaveUnit));
   if (e == cudaSuccess) e = cudaMalloc(d_first, first.size() * sizeof(int));
   if (e == cudaSuccess && !sorted.empty())
