@@ -111,10 +111,12 @@ static_assert(64 > lbm::kMaxTail, "plan buffers of lbm_sw_step and lbm_sw_step_p
 // takes single steps with the VEC kernel).
 cudaError_t launch_one_step(lbm_sw* h, int from, cudaStream_t st) {
   const int variant = h->kernel == LBM_SW_KERNEL_TEMPORAL ? LBM_SW_KERNEL_VEC : h->kernel;
-  if (h->has_obstacles)
+  if (h->has_obstacles) {
+    const unsigned char* mask = variant == LBM_SW_KERNEL_SIMPLE ? h->solid : h->solid_flags;
     return h->p.precision == LBM_SW_FP64
-               ? lbm::launch_step2d_obstacle<double>(args<double>(h, from), consts(h), h->solid, variant, st)
-               : lbm::launch_step2d_obstacle<float>(args<float>(h, from), consts(h), h->solid, variant, st);
+               ? lbm::launch_step2d_obstacle<double>(args<double>(h, from), consts(h), mask, variant, st)
+               : lbm::launch_step2d_obstacle<float>(args<float>(h, from), consts(h), mask, variant, st);
+  }
   if (h->p.precision == LBM_SW_FP64) {
     auto a = args<double>(h, from);
     return h->p.dim == 1 ? lbm::launch_step1d<double>(a, consts(h), st)
@@ -717,7 +719,7 @@ int lbm_sw_set_obstacle(lbm_sw* h, const unsigned char* solid, int on_device) {
     if (!h->solid) LBM_CUDA(h, cudaMalloc(&h->solid, n), "cudaMalloc (obstacle mask)");
     LBM_CUDA(h, cudaMemcpyAsync(h->solid, solid, n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                                 h->stream), "obstacle mask copy");
-    if (h->p.precision == LBM_SW_FP32 && (h->auto_kernel || h->kernel == LBM_SW_KERNEL_TEMPORAL)) {
+    if (h->kernel != LBM_SW_KERNEL_SIMPLE) {
       if (!h->solid_flags)
         LBM_CUDA(h, cudaMalloc(&h->solid_flags, static_cast<size_t>(h->plane)), "cudaMalloc (obstacle flags)");
       LBM_CUDA(h, lbm::launch_obstacle_flags(h->solid, h->solid_flags, h->p.nx, h->p.ny, h->pitch, h->p.bc, h->stream),

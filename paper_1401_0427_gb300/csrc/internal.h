@@ -33,6 +33,11 @@ struct ConstsD {  // scheme constants before conversion to T
   double rates[10] = {};   // MRT rates (Consts::r order); unused when mrt is false
 };
 
+// Flags of a cell with obstacles: itself, and its neighbours at x - 1, x + 1,
+// y - 1 and y + 1 (beyond a side that is not periodic: not solid, the side's own rule applies).  A
+// solid cell has only the first.  launch_obstacle_flags makes them ([ny][pitch] bytes) from a mask.
+constexpr unsigned kSolidSelf = 1, kSolidLeft = 2, kSolidRight = 4, kSolidBelow = 8, kSolidAbove = 16;
+
 // ---- 2D launchers (kernels_2d.cu) ----
 template <class T>
 cudaError_t launch_step2d(const StepArgs<T>& a, const ConstsD& k, int variant, cudaStream_t st);
@@ -42,10 +47,10 @@ cudaError_t launch_init2d(const StepArgs<T>& a, const ConstsD& k, const double* 
 template <class T>
 cudaError_t launch_collide2d_dense(const StepArgs<T>& a, const ConstsD& k, const T* dense,
                                   const unsigned char* solid, cudaStream_t st);
-// one step with obstacles (solid: [ny][nx] device mask, nonzero = solid); variant SIMPLE:
-// one thread per cell, otherwise the vectorised row kernel
+// one step with obstacles; variant SIMPLE: one thread per cell, with the mask [ny][nx] (nonzero =
+// solid), otherwise the row kernel, with the cells' flags [ny][pitch] (kSolid*)
 template <class T>
-cudaError_t launch_step2d_obstacle(const StepArgs<T>& a, const ConstsD& k, const unsigned char* solid, int variant,
+cudaError_t launch_step2d_obstacle(const StepArgs<T>& a, const ConstsD& k, const unsigned char* mask, int variant,
                                    cudaStream_t st);
 template <class T>
 cudaError_t launch_moments2d(const StepArgs<T>& a, double* h, double* hu, double* hv, cudaStream_t st);
@@ -134,10 +139,6 @@ bool temporal_mrt_supported(const int bc[4], int nx, int k);
 cudaError_t launch_step2d_temporal_mrt(const StepArgs<float>& a, const ConstsD& kd, int k, cudaStream_t st,
                                        int sm_count);
 
-// Flags of a cell for the fused steps with solid cells: itself, and its neighbours at x - 1, x + 1,
-// y - 1 and y + 1 (beyond a side that is not periodic: not solid, the side's own rule applies).  A
-// solid cell has only the first.  launch_obstacle_flags makes them ([ny][pitch] bytes) from a mask.
-constexpr unsigned kSolidSelf = 1, kSolidLeft = 2, kSolidRight = 4, kSolidBelow = 8, kSolidAbove = 16;
 // k (2, 4 or 6) fused BGK steps with solid cells (temporal_obstacle.cu).
 cudaError_t launch_obstacle_flags(const unsigned char* solid, unsigned char* flags, int nx, int ny, long long pitch,
                                   const int bc[4], cudaStream_t st);

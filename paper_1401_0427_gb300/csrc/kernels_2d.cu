@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
+#include <utility>
 
 #include "internal.h"
 #include "scheme.cuh"
@@ -147,35 +149,37 @@ __global__ void __launch_bounds__(256)
 // its writes to be visible (griddepcontrol.wait: before any read of src or write of dst, so
 // neither the previous step's output nor its input is touched early), and signals when its
 // own rows are done (griddepcontrol.launch_dependents).  Launched without it, both are no-ops.
-template <class T, int BY, bool MRT>
-__global__ void __launch_bounds__(32 * BY) step2d_vec(const StepArgs<T> A, const Consts<T> K) {
-  constexpr int V = V16<T>::n;
+template <class T, int BY, bool MRT, int RES>
+__global__ void __launch_bounds__(32 * BY, RES) step2d_vec(const StepArgs<T> A, const Consts<T> K) {
+  constexpr int V = RowVec<T>::n;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int x0 = (blockIdx.x * 32 + threadIdx.x) * V;
   for (int y = blockIdx.y * BY + threadIdx.y; y < A.ny; y += gridDim.y * BY)  // warp-uniform
-    vec_row<T, false, MRT>(A, K, y, x0, threadIdx.x, nullptr);
+    vec_row<T, false, MRT, false, RowVec<T>>(A, K, y, x0, threadIdx.x, nullptr);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // The same step with solid cells inside the domain (mirror walls on their faces; OBST in
 // vec_row), launched like step2d_vec.
-template <class T, int BY, bool MRT>
-__global__ void __launch_bounds__(32 * BY)
-    step2d_vec_obstacle(const StepArgs<T> A, const Consts<T> K, const unsigned char* __restrict__ solid) {
-  constexpr int V = V16<T>::n;
+template <class T, int BY, bool MRT, int RES>
+__global__ void __launch_bounds__(32 * BY, RES)
+    step2d_vec_obstacle(const StepArgs<T> A, const Consts<T> K, const unsigned char* __restrict__ flags) {
+  constexpr int V = RowVec<T>::n;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int x0 = (blockIdx.x * 32 + threadIdx.x) * V;
   for (int y = blockIdx.y * BY + threadIdx.y; y < A.ny; y += gridDim.y * BY)  // warp-uniform
-    vec_row<T, false, MRT, true>(A, K, y, x0, threadIdx.x, nullptr, solid);
+    vec_row<T, false, MRT, true, RowVec<T>>(A, K, y, x0, threadIdx.x, nullptr, flags);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // The same step, also writing the moments (h, hu, hv) of the new state to three planes
 // (used by the replay of the discrete adjoint).
 template <class T, int BY>
 __global__ void __launch_bounds__(32 * BY) step2d_vec_w(const StepArgs<T> A, const Consts<T> K, T* w_out) {
-  constexpr int V = V16<T>::n;
+  constexpr int V = RowVec<T>::n;
   const int x0 = (blockIdx.x * 32 + threadIdx.x) * V;
   for (int y = blockIdx.y * BY + threadIdx.y; y < A.ny; y += gridDim.y * BY)
-    vec_row<T, true>(A, K, y, x0, threadIdx.x, w_out);
+    vec_row<T, true, false, false, RowVec<T>>(A, K, y, x0, threadIdx.x, w_out);
 }
 
 // --------------------------------------------------------------------------
@@ -365,6 +369,40 @@ cudaError_t copy_planes(const PlaneCopy& c, size_t elem, cudaStream_t st) {
   return cudaSuccess;
 }
 
+// Rows (warps) per CTA: FP64 one, so that the warps spread evenly over the quarters of the SMs whose
+// FP64 units bound the kernel (1536^2: 152.5 us per step, 158.2 with four, 16 warps per SM).
+template <class T>
+constexpr int kRowsPerCta = sizeof(T) == 8 ? 1 : 4;
+
+// FP64: registers for 16 warps per SM on small grids, which have few (480 x 120: 5.7 us per step,
+// 6.1 with 24), for 24 on others (512^2 18.0 against 19.1, 1536^2 140 against 151).
+template <class T, class F>
+cudaError_t with_residency(const StepArgs<T>& a, F&& launch) {
+  if constexpr (sizeof(T) == 4)
+    return launch(std::integral_constant<int, 1>{});
+  else if (static_cast<long long>(a.nx) * a.ny >= (1LL << 17))
+    return launch(std::integral_constant<int, 24>{});
+  else
+    return launch(std::integral_constant<int, 16>{});
+}
+
+// Launch of a row kernel, a warp per 32 V cells of a row and BY rows per CTA, with programmatic
+// dependent launch.
+template <class T, int BY, class... KArgs, class... Args>
+cudaError_t launch_rows(void (*kernel)(KArgs...), const StepArgs<T>& a, cudaStream_t st, Args&&... args) {
+  constexpr int V = RowVec<T>::n;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((a.nx + 32 * V - 1) / (32 * V), static_cast<unsigned>(std::min<long long>((a.ny + BY - 1) / BY, 65535)));
+  cfg.blockDim = dim3(32, BY);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a, std::forward<Args>(args)...);
+}
+
 template <class T>
 cudaError_t launch_step2d(const StepArgs<T>& a, const ConstsD& kd, int variant, cudaStream_t st) {
   const Consts<T> K = to_consts<T>(kd);
@@ -374,55 +412,40 @@ cudaError_t launch_step2d(const StepArgs<T>& a, const ConstsD& kd, int variant, 
       step2d_simple<T, true><<<cell_grid(a.nx, a.ny, block), block, 0, st>>>(a, K);
     else
       step2d_simple<T, false><<<cell_grid(a.nx, a.ny, block), block, 0, st>>>(a, K);
-  } else {
-    constexpr int BY = 4;
-    constexpr int V = V16<T>::n;
-    const dim3 block(32, BY);
-    const dim3 grid((a.nx + 32 * V - 1) / (32 * V),
-                    static_cast<unsigned>(std::min<long long>((a.ny + BY - 1) / BY, 65535)));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return kd.mrt ? cudaLaunchKernelEx(&cfg, step2d_vec<T, BY, true>, a, K)
-                  : cudaLaunchKernelEx(&cfg, step2d_vec<T, BY, false>, a, K);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
+  return with_residency<T>(a, [&](auto res) {
+    constexpr int BY = kRowsPerCta<T>, RES = decltype(res)::value;
+    return kd.mrt ? launch_rows<T, BY>(step2d_vec<T, BY, true, RES>, a, st, K)
+                  : launch_rows<T, BY>(step2d_vec<T, BY, false, RES>, a, st, K);
+  });
 }
 
+// mask: the solid cells ([ny][nx]) for SIMPLE, else their flags ([ny][pitch], kSolid*)
 template <class T>
-cudaError_t launch_step2d_obstacle(const StepArgs<T>& a, const ConstsD& kd, const unsigned char* solid, int variant,
+cudaError_t launch_step2d_obstacle(const StepArgs<T>& a, const ConstsD& kd, const unsigned char* mask, int variant,
                                    cudaStream_t st) {
   const Consts<T> K = to_consts<T>(kd);
   if (variant == LBM_SW_KERNEL_SIMPLE) {  // one thread per cell
     const dim3 block(32, 8);
     if (kd.mrt)
-      step2d_obstacle<T, true><<<cell_grid(a.nx, a.ny, block), block, 0, st>>>(a, K, solid);
+      step2d_obstacle<T, true><<<cell_grid(a.nx, a.ny, block), block, 0, st>>>(a, K, mask);
     else
-      step2d_obstacle<T, false><<<cell_grid(a.nx, a.ny, block), block, 0, st>>>(a, K, solid);
+      step2d_obstacle<T, false><<<cell_grid(a.nx, a.ny, block), block, 0, st>>>(a, K, mask);
     return cudaGetLastError();
   }
-  constexpr int BY = 4;
-  constexpr int V = V16<T>::n;
-  const dim3 block(32, BY);
-  const dim3 grid((a.nx + 32 * V - 1) / (32 * V), static_cast<unsigned>(std::min<long long>((a.ny + BY - 1) / BY, 65535)));
-  if (kd.mrt)
-    step2d_vec_obstacle<T, BY, true><<<grid, block, 0, st>>>(a, K, solid);
-  else
-    step2d_vec_obstacle<T, BY, false><<<grid, block, 0, st>>>(a, K, solid);
-  return cudaGetLastError();
+  return with_residency<T>(a, [&](auto res) {
+    constexpr int BY = kRowsPerCta<T>, RES = decltype(res)::value;
+    return kd.mrt ? launch_rows<T, BY>(step2d_vec_obstacle<T, BY, true, RES>, a, st, K, mask)
+                  : launch_rows<T, BY>(step2d_vec_obstacle<T, BY, false, RES>, a, st, K, mask);
+  });
 }
 
 template <class T>
 cudaError_t launch_step2d_store_w(const StepArgs<T>& a, const ConstsD& kd, T* w_out, cudaStream_t st) {
   const Consts<T> K = make_consts<T>(kd.g, kd.lambda, kd.s, kd.a);
   constexpr int BY = 4;
-  constexpr int V = V16<T>::n;
+  constexpr int V = RowVec<T>::n;
   const dim3 block(32, BY);
   const dim3 grid((a.nx + 32 * V - 1) / (32 * V),
                   static_cast<unsigned>(std::min<long long>((a.ny + BY - 1) / BY, 65535)));

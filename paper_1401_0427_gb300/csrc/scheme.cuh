@@ -99,7 +99,16 @@ struct Consts {
   T s_4;    // s / 4
   // 1D, FP64: f0 = a_2 h + a_4g u^2
   T a_2, a_4g;
+  // 2D, FP64 (collide13_fixed): |1 - s|, s / 4 and s c in units of 2^-64, and whether they are below one
+  unsigned long long x_om, x_s4, x_sc;
+  bool om_neg, fixed_ok;
 };
+
+// |v| <= 1 in units of 2^-64 (saturated)
+inline __host__ unsigned long long in_2_64(double v) {
+  const double a = v < 0 ? -v : v;
+  return a >= 1.0 ? ~0ull : static_cast<unsigned long long>(a * 18446744073709551616.0);
+}
 
 template <class T>
 __host__ void set_mrt_folded(Consts<T>& k) {
@@ -125,6 +134,11 @@ __host__ Consts<T> make_consts(double g, double lambda, double s, double a) {
   k.s_4 = static_cast<T>(st / 4.0);
   k.a_2 = static_cast<T>(a / 2.0);
   k.a_4g = static_cast<T>(-a / (4.0 * g));
+  k.x_om = in_2_64(1.0 - st);
+  k.x_s4 = in_2_64(st / 4.0);
+  k.x_sc = in_2_64(st * c);
+  k.om_neg = st > 1.0;
+  k.fixed_ok = st >= 0.0 && st <= 2.0 && st * c < 1.0;
   for (int i = 0; i < 10; ++i) k.r[i] = k.s;
   set_mrt_folded(k);
   return k;
@@ -145,6 +159,74 @@ __device__ __forceinline__ void moments13(const T f[13], T& h, T& qx, T& qy) {
   h = add(f[0], add(add(f[1], f[3]), add(f[2], f[4])));
   qx = add(add(f[5], f[7]), add(f[6], f[8]));
   qy = add(add(f[9], f[11]), add(f[10], f[12]));
+}
+
+// ---- FP64 sums and relaxation in 64-bit integers ----
+// An FP64 instruction takes 64 cycles of a quarter of an SM, in which its integer pipe takes 40 or
+// so.  Values of like size are therefore added as 64-bit integers in units of 2^-59 of the
+// power of two below the largest of them (`e`: that value's exponent field, in place) and rounded
+// once to a double, to nearest even.  What an operand loses is below one unit.  Operations work on
+// magnitudes and signs, so exact negatives give exact negatives (mirror-image cells), and sums
+// do not depend on the order.
+__device__ __forceinline__ int exp_field(double x) { return __double2hiint(x) & 0x7ff00000; }
+// exponents for which every shift and result below stays inside the normal range
+__device__ __forceinline__ bool exp_fits(int e) { return e >= (64 << 20) && e <= (2000 << 20); }
+__device__ __forceinline__ unsigned long long mantissa(double x) {  // 53 bits (a zero: 2^52, shifted out by its exponent)
+  return (static_cast<unsigned long long>((__double2hiint(x) & 0xfffff) | 0x100000) << 32) |
+         static_cast<unsigned>(__double2loint(x));
+}
+// |x| in units of e's, for exponents up to e
+__device__ __forceinline__ unsigned long long fix_mag(double x, int e) {
+  return (mantissa(x) << 7) >> min((e - exp_field(x)) >> 20, 63);
+}
+__device__ __forceinline__ long long with_sign(unsigned long long m, int hi) {  // the sign bit of hi
+  const long long s = hi >> 31;
+  return (static_cast<long long>(m) ^ s) - s;
+}
+// x in units of e's, for exponents up to e + 1; ok: cleared beyond
+__device__ __forceinline__ long long fix_one_more(double x, int e, bool& ok) {
+  const int d = ((e - exp_field(x)) >> 20) + 1;
+  ok = ok && d >= 0;
+  return with_sign((mantissa(x) << 8) >> (d & 63) >> (d > 63 ? 63 : 0), __double2hiint(x));
+}
+// m c / 2^64 without the last partial product (less than 3 units too small)
+__device__ __forceinline__ unsigned long long times_2_64(unsigned long long m, unsigned long long c) {
+  const unsigned mh = static_cast<unsigned>(m >> 32), ml = static_cast<unsigned>(m);
+  const unsigned ch = static_cast<unsigned>(c >> 32), cl = static_cast<unsigned>(c);
+  return static_cast<unsigned long long>(mh) * ch + __umulhi(mh, cl) + __umulhi(ml, ch);
+}
+// the double of v (|v| < 2^63) in units of e's, rounded to nearest even
+__device__ __forceinline__ double unfix(long long v, int e) {
+  const int s = static_cast<int>(v >> 63);
+  unsigned long long a = static_cast<unsigned long long>((v ^ s) - s);
+  const int lz = __clzll(static_cast<long long>(a));
+  a <<= (lz - 1) & 63;  // leading bit 62
+  a += 0x1ff + (static_cast<unsigned>(a >> 10) & 1);
+  const int hi = static_cast<int>(static_cast<unsigned>(a >> 42) + e + ((3 - lz) << 20)) | (s & static_cast<int>(0x80000000u));
+  return v == 0 ? 0.0 : __hiloint2double(hi, static_cast<int>(a >> 10));
+}
+
+// The sum of N <= 5 values rounded once; infinities, NaN and sums near either end of the
+// exponent's range are added in FP64.
+template <int N>
+__device__ __forceinline__ double sum_once(const double (&x)[N]) {
+  int e = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) e = max(e, exp_field(x[i]));
+  if (!exp_fits(e)) {
+    const double s = add(add(x[0], x[1]), add(x[2], x[3]));
+    return N == 5 ? add(x[N - 1], s) : s;
+  }
+  long long v = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) v += with_sign(fix_mag(x[i], e), __double2hiint(x[i]));
+  return unfix(v, e);
+}
+
+__device__ __forceinline__ void moments13(const double f[13], double& h, double& qx, double& qy) {
+  h = sum_once<5>({f[1], f[3], f[2], f[4], f[0]});
+  qx = sum_once<4>({f[5], f[7], f[6], f[8]});
+  qy = sum_once<4>({f[9], f[11], f[10], f[12]});
 }
 
 template <class T>
@@ -223,12 +305,11 @@ __device__ __forceinline__ void collide13(T f[13], const Consts<T>& k, T& h, T& 
   f[12] = fmad(om, f[12], sub(y4, pyy));
 }
 
-// FP64: the same operator in 52 operations of the FP64 unit instead of 59 (the unit bounds every
-// FP64 kernel: 64 cycles per warp instruction on its quarter of an SM).  The two terms of each
-// equilibrium meet in one fused multiply-add, s r +- s c q and s q / 4 +- (s c h) t with
-// t = u^2 + g h / 2, v^2 + g h / 2 or u v, so the products s c q and s c (q u + p) are not formed;
-// each population rounds once less than above.  Mirror images still round alike.
-__device__ __forceinline__ void collide13(double f[13], const Consts<double>& k, double& h, double& qx, double& qy) {
+// FP64: the same operator in 42 operations of the FP64 unit instead of 59, the moments' 10 additions
+// aside (sum_once).  The two terms of each equilibrium meet in one fused multiply-add, s r +- s c q
+// and s q / 4 +- (s c h) t with t = u^2 + g h / 2, v^2 + g h / 2 or u v, so the products s c q and
+// s c (q u + p) are not formed.  Mirror images still round alike.
+__device__ __forceinline__ void collide13_fma(double f[13], const Consts<double>& k, double& h, double& qx, double& qy) {
   moments13(f, h, qx, qy);
   const double rh = recip(h);
   const double u = mul(qx, rh), v = mul(qy, rh);
@@ -251,6 +332,71 @@ __device__ __forceinline__ void collide13(double f[13], const Consts<double>& k,
   f[10] = fmad(om, f[10], fmad(hc, ty, y4));
   f[11] = fmad(om, f[11], fmad(-hc, uv, y4));
   f[12] = fmad(om, f[12], fmad(-hc, ty, y4));
+}
+
+// FP64, the usual case: the sums, s c q, s q / 4 and the relaxation of the twelve moving
+// populations in integers (above), each population rounded once: 19 operations of the FP64 unit.
+// False, and nothing changed, where the values of a family differ too much in size (an equilibrium
+// term more than twice the power of two of the largest population, as at the front of a
+// jump; exponents near the ends of the range): collide13_fma takes the cell then.
+//
+// 1536^2 cells, us per step: 278 with 59 operations in the FP64 unit, 218 with 52, 197 with the
+// moments in integers, 140 this way.  Error against quadruple precision after 300
+// steps of a dam break on 40^2 cells: h 1.2e-15 and q 9e-15 with 59 operations, 3e-16 and 3e-15.
+__device__ __forceinline__ bool collide13_fixed(double f[13], const Consts<double>& k, double& h, double& qx, double& qy) {
+  int ef = exp_field(f[0]), ex = 0, ey = 0;
+#pragma unroll
+  for (int i = 1; i < 5; ++i) {
+    ef = max(ef, exp_field(f[i]));
+    ex = max(ex, exp_field(f[4 + i]));
+    ey = max(ey, exp_field(f[8 + i]));
+  }
+  if (!(k.fixed_ok && exp_fits(ef) && exp_fits(ex) && exp_fits(ey))) return false;
+  unsigned long long m[13];
+  long long v[3] = {0, 0, 0};
+#pragma unroll
+  for (int i = 0; i < 13; ++i) {
+    m[i] = fix_mag(f[i], i < 5 ? ef : (i < 9 ? ex : ey));
+    v[i < 5 ? 0 : (i < 9 ? 1 : 2)] += with_sign(m[i], __double2hiint(f[i]));
+  }
+  h = unfix(v[0], ef);
+  qx = unfix(v[1], ex);
+  qy = unfix(v[2], ey);
+  const double rh = recip(h);
+  const double u = mul(qx, rh), w = mul(qy, rh);
+  const double uu = mul(u, u), ww = mul(w, w), uw = mul(u, w);
+  const double z = fmad(add(uu, ww), k.s_a4g, mul(k.s_a2, h));  // -s f0^eq / 4
+  const double r = fmad(h, k.s_4, z);                           // s (h - f0^eq) / 4
+  const double hc = mul(h, k.s_c);
+  const double pxx = mul(hc, fmad(k.half_g, h, uu)), pyy = mul(hc, fmad(k.half_g, h, ww)), pxy = mul(hc, uw);
+  bool ok = true;
+  const int sx = static_cast<int>(v[1] >> 32), sy = static_cast<int>(v[2] >> 32);  // their sign bits
+  const unsigned long long ax = static_cast<unsigned long long>(v[1] < 0 ? -v[1] : v[1]);
+  const unsigned long long ay = static_cast<unsigned long long>(v[2] < 0 ? -v[2] : v[2]);
+  // s c q in units of the f family's: shifted by the exponents' difference
+  auto to_f = [&](unsigned long long q, int e) {
+    const int d = (ef - e) >> 20;
+    ok = ok && d >= -6;
+    return d >= 0 ? q >> min(d, 63) : q << (-d & 7);
+  };
+  const long long cx = with_sign(to_f(times_2_64(ax, k.x_sc), ex), sx), cy = with_sign(to_f(times_2_64(ay, k.x_sc), ey), sy);
+  const long long x4 = with_sign(times_2_64(ax, k.x_s4), sx), y4 = with_sign(times_2_64(ay, k.x_s4), sy);
+  const long long fr = fix_one_more(r, ef, ok);
+  const long long fxx = fix_one_more(pxx, ex, ok), fxy = fix_one_more(pxy, ex, ok);
+  const long long fyx = fix_one_more(pxy, ey, ok), fyy = fix_one_more(pyy, ey, ok);
+  if (!ok) return false;
+  f[0] = fmad(k.om, f[0], times_pow2<2, true>(z));
+  const int flip = k.om_neg ? static_cast<int>(0x80000000u) : 0;
+  const long long eq[13] = {0,        fr + cx,  fr + cy,  fr - cx,  fr - cy,  x4 + fxx, x4 + fxy,
+                            x4 - fxx, x4 - fxy, y4 + fyx, y4 + fyy, y4 - fyx, y4 - fyy};
+#pragma unroll
+  for (int i = 1; i < 13; ++i)
+    f[i] = unfix(with_sign(times_2_64(m[i], k.x_om), __double2hiint(f[i]) ^ flip) + eq[i], i < 5 ? ef : (i < 9 ? ex : ey));
+  return true;
+}
+
+__device__ __forceinline__ void collide13(double f[13], const Consts<double>& k, double& h, double& qx, double& qy) {
+  if (!collide13_fixed(f, k, h, qx, qy)) collide13_fma(f, k, h, qx, qy);
 }
 
 template <class T>
