@@ -57,9 +57,10 @@ __global__ void __launch_bounds__(256) step1d(const StepArgs<T> A, const Consts<
 //
 // What bounds it is the collision's chain of one warp: in FP64 every instruction takes 64 cycles
 // of its quarter of an SM (half a lane per clock, whatever the number of active lanes), so the
-// line is spread over as many quarters as it fills.  1000 cells, FP64: 1.23 us per step, against
-// 1.44 with one cluster of 16 SMs (windows of 63 + 16 cells in shared memory, a cluster barrier
-// per 8 steps); 16000 cells: 1.66 against 9.82.  FP32: 0.17 against 0.39 and 0.18 against 0.69.
+// line is spread over as many quarters as it fills.  With the former collision (32 FP64 operations)
+// 1000 cells took 1.23 us per step in FP64, against 1.44 with one cluster of 16 SMs (windows of
+// 63 + 16 cells in shared memory, a cluster barrier per 8 steps), 16000 cells 1.66 against 9.82;
+// with the one in integers 0.98 and 1.25.  FP32: 0.16 against 0.39 and 0.17 against 0.69.
 //
 // Exchange: a mailbox in global memory with two slots per cell, used by turns.  Each 8-byte
 // word carries 4 bytes of payload and the number of the exchange, written and read as one
@@ -162,9 +163,11 @@ __global__ void __launch_bounds__(32) step1d_windows(const StepArgs<T> A, const 
           }
         }
       }
-      collide5_any<T, MRT>(n, K);
+      if (sizeof(T) == 4 || cell >= 0) {  // FP64 lanes outside keep their values (noise leaves the integers' path)
+        collide5_any<T, MRT>(n, K);
 #pragma unroll
-      for (int p = 0; p < 5; ++p) f[p] = n[p];
+        for (int p = 0; p < 5; ++p) f[p] = n[p];
+      }
     }
     done += kb;
     if (done >= nsteps) break;
@@ -273,18 +276,22 @@ size_t mail1d_bytes(int nx) {
 }
 
 // Steps between exchanges (the halo's width) for a line of nx cells: an exchange takes about
-// 0.5 us, so wide halos while the warps they make find free quarters of SMs, narrower ones (fewer
-// warps) on longer lines.  FP64, us per step with halos of 4 / 6 / 8 / 10: 3000 cells 1.31 / 1.25
-// / 1.26 / 1.21, 8000 cells 1.32 / 1.25 / 1.32 / 1.64, 16000 cells 1.66 / 1.85 / 2.10 / -.  FP32
-// with 6 / 8 / 10: 3000 cells 0.20 / 0.18 / 0.16, 16000 cells 0.23 / 0.18 / 0.20.  Two or four
-// cells per lane were slower at every length (16000 cells, FP64: 2.3 and 4.6).
+// 0.5 us, so wide halos while the warps they make find free quarters of SMs (with some to spare: they
+// are not dealt evenly), narrower ones (fewer warps) on longer lines.  FP64, us per step with halos
+// of 4 / 6 / 8 / 10: 3000 cells 1.06 / 1.02 / 1.03 / 0.98, 8000 cells 1.08 / 1.01 / 1.00 / 1.25,
+// 12000 cells 1.09 / 1.02 / 1.24 / 1.24, 16000 cells 1.34 / 1.30 / 1.26 / 1.63.  FP32 with 6 / 8 /
+// 10: 3000 cells 0.20 / 0.18 / 0.16, 16000 cells 0.23 / 0.18 / 0.20.  Two or four cells per lane
+// were slower at every length.
 template <class T>
 int window_halo(int nx, int sm_count) {
   auto pieces = [&](int b) { return (nx + 32 - 2 * b - 1) / (32 - 2 * b); };
-  if constexpr (sizeof(T) == 8)
-    return pieces(10) <= 3 * sm_count ? 10 : pieces(6) <= 3 * sm_count ? 6 : 4;
-  else
+  if constexpr (sizeof(T) == 8) {
+    for (int b : {10, 8})
+      if (2 * pieces(b) <= 7 * sm_count) return b;
+    return pieces(6) <= 4 * sm_count ? 6 : 8;
+  } else {
     return pieces(10) <= 4 * sm_count ? 10 : 8;
+  }
 }
 
 template <class T>

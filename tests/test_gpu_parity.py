@@ -104,7 +104,8 @@ def test_graph_replay_equals_single_launches(precision):
 
 @pytest.mark.parametrize("precision", [lbm_sw.FP64, lbm_sw.FP32])
 @pytest.mark.parametrize("bc", [(P, P), (W, O), (I, W)], ids=str)
-@pytest.mark.parametrize("n", [9, 11, 12, 13, 21, 24, 25, 37, 5472, 5473, 7297, 9120, 9121])
+@pytest.mark.parametrize("n", [9, 11, 12, 13, 21, 24, 25, 37, 5472, 5473, 6384, 6385, 7297, 8512, 8513, 9120, 9121, 12160,
+                               12161])
 @pytest.mark.parametrize("steps", [10, 11, 61])
 def test_1d_windows_equal_the_per_step_kernel(n, bc, precision, steps):
     """Lines whose last piece is shorter than a halo, around a whole number of pieces and where
