@@ -275,7 +275,7 @@ void lbm_sw_destroy(lbm_sw* h) {
   if (h->mail1d) cudaFree(h->mail1d);
   if (h->pop_staging) cudaFree(h->pop_staging);
   if (h->diag_partials) cudaFree(h->diag_partials);
-  if (h->diag_out) cudaFree(h->diag_out);
+  if (h->diag_done) cudaFree(h->diag_done);
   if (h->diag_host) cudaFreeHost(h->diag_host);
   if (h->solid) cudaFree(h->solid);
   if (h->solid_flags) cudaFree(h->solid_flags);
@@ -339,7 +339,8 @@ int lbm_sw_create(const lbm_sw_params* p, lbm_sw** out) {
     return bail(LBM_SW_E_NOMEM);
   if (cudaMalloc(&h->diag_partials, 5 * sizeof(double) * lbm::diag_max_blocks()) != cudaSuccess)
     return bail(LBM_SW_E_NOMEM);
-  if (cudaMalloc(&h->diag_out, 8 * sizeof(double)) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
+  if (cudaMalloc(&h->diag_done, sizeof(unsigned)) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
+  if (cudaMemsetAsync(h->diag_done, 0, sizeof(unsigned), h->stream) != cudaSuccess) return bail(LBM_SW_E_CUDA);
   if (cudaMallocHost(&h->diag_host, 8 * sizeof(double)) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
   cudaError_t e;
   if (p->precision == LBM_SW_FP64)
@@ -559,12 +560,10 @@ int lbm_sw_diagnostics(lbm_sw* h, double out[4]) {
   if (!h || !out) return h ? fail(h, LBM_SW_E_ARG, "diagnostics: out is NULL") : LBM_SW_E_ARG;
   if (!h->has_state) return fail(h, LBM_SW_E_STATE, "diagnostics: no state set");
   cudaError_t e = h->p.precision == LBM_SW_FP64
-                      ? lbm::launch_diagnostics<double>(args<double>(h, h->cur), h->q, h->diag_partials, h->diag_out, h->stream)
-                      : lbm::launch_diagnostics<float>(args<float>(h, h->cur), h->q, h->diag_partials, h->diag_out, h->stream);
+                      ? lbm::launch_diagnostics<double>(args<double>(h, h->cur), h->q, h->diag_partials, h->diag_done, h->diag_host, h->sm_count, h->stream)
+                      : lbm::launch_diagnostics<float>(args<float>(h, h->cur), h->q, h->diag_partials, h->diag_done, h->diag_host, h->sm_count, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "diagnostics kernel launch");
-  h->launches += 2;
-  LBM_CUDA(h, cudaMemcpyAsync(h->diag_host, h->diag_out, 5 * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
-           "copy diagnostics");
+  h->launches += 1;
   LBM_CUDA(h, cudaStreamSynchronize(h->stream), "diagnostics synchronize");
   for (int k = 0; k < 4; ++k) out[k] = h->diag_host[k];
   if (h->diag_host[4] > 0)
@@ -664,17 +663,15 @@ int lbm_sw_diagnostics_rows(lbm_sw* h, int y0, int nrows, double out[4]) {
     auto a = args<double>(h, h->cur);
     a.src += static_cast<long long>(y0) * h->pitch;
     a.ny = nrows;
-    e = lbm::launch_diagnostics<double>(a, h->q, h->diag_partials, h->diag_out, h->stream);
+    e = lbm::launch_diagnostics<double>(a, h->q, h->diag_partials, h->diag_done, h->diag_host, h->sm_count, h->stream);
   } else {
     auto a = args<float>(h, h->cur);
     a.src += static_cast<long long>(y0) * h->pitch;
     a.ny = nrows;
-    e = lbm::launch_diagnostics<float>(a, h->q, h->diag_partials, h->diag_out, h->stream);
+    e = lbm::launch_diagnostics<float>(a, h->q, h->diag_partials, h->diag_done, h->diag_host, h->sm_count, h->stream);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "diagnostics kernel launch");
-  h->launches += 2;
-  LBM_CUDA(h, cudaMemcpyAsync(h->diag_host, h->diag_out, 5 * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
-           "copy diagnostics");
+  h->launches += 1;
   LBM_CUDA(h, cudaStreamSynchronize(h->stream), "diagnostics synchronize");
   for (int k = 0; k < 4; ++k) out[k] = h->diag_host[k];
   if (h->diag_host[4] > 0)

@@ -96,7 +96,7 @@ struct lbm_sw_batch {
   double* moments_staging = nullptr;
   size_t moments_staging_cells = 0;
   double* diag_partials = nullptr;
-  double* diag_out = nullptr;
+  unsigned* diag_done = nullptr;
   double* diag_host = nullptr;
   int sm_count = 152;
   int tile_rows = 4;
@@ -323,7 +323,7 @@ void lbm_sw_batch_destroy(lbm_sw_batch* b) {
   if (b->inflow_feq) cudaFree(b->inflow_feq);
   if (b->moments_staging) cudaFree(b->moments_staging);
   if (b->diag_partials) cudaFree(b->diag_partials);
-  if (b->diag_out) cudaFree(b->diag_out);
+  if (b->diag_done) cudaFree(b->diag_done);
   if (b->diag_host) cudaFreeHost(b->diag_host);
   for (int k = 0; k < 9; ++k) lbm::batch_waves_free(&b->waves[k]);
   delete b;
@@ -415,7 +415,8 @@ int lbm_sw_batch_create(const lbm_sw_batch_params* p, lbm_sw_batch** out) {
   }
   if (cudaMalloc(&b->inflow_feq, 4 * 13 * b->elem) != cudaSuccess) return bail(LBM_SW_E_NOMEM, "cudaMalloc");
   if (cudaMalloc(&b->diag_partials, 5 * sizeof(double) * lbm::diag_max_blocks()) != cudaSuccess ||
-      cudaMalloc(&b->diag_out, 8 * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&b->diag_done, sizeof(unsigned)) != cudaSuccess ||
+      cudaMemsetAsync(b->diag_done, 0, sizeof(unsigned), b->stream) != cudaSuccess ||
       cudaMallocHost(&b->diag_host, 8 * sizeof(double)) != cudaSuccess)
     return bail(LBM_SW_E_NOMEM, "cudaMalloc(diagnostics)");
   cudaError_t e = p->precision == LBM_SW_FP64
@@ -570,11 +571,9 @@ int lbm_sw_batch_diagnostics(lbm_sw_batch* b, int i, double out[4]) {
   if (rc) return rc;
   if (!b->has_state[i]) return bfail(b, LBM_SW_E_STATE, "diagnostics: instance %d has no state", i);
   cudaError_t e = b->p.precision == LBM_SW_FP64
-                      ? lbm::launch_diagnostics<double>(inst_args<double>(b, i, b->cur), 13, b->diag_partials, b->diag_out, b->stream)
-                      : lbm::launch_diagnostics<float>(inst_args<float>(b, i, b->cur), 13, b->diag_partials, b->diag_out, b->stream);
+                      ? lbm::launch_diagnostics<double>(inst_args<double>(b, i, b->cur), 13, b->diag_partials, b->diag_done, b->diag_host, b->sm_count, b->stream)
+                      : lbm::launch_diagnostics<float>(inst_args<float>(b, i, b->cur), 13, b->diag_partials, b->diag_done, b->diag_host, b->sm_count, b->stream);
   if (e != cudaSuccess) return bcuda(b, e, "diagnostics kernel launch");
-  BATCH_CUDA(b, cudaMemcpyAsync(b->diag_host, b->diag_out, 5 * sizeof(double), cudaMemcpyDeviceToHost, b->stream),
-             "copy diagnostics");
   BATCH_CUDA(b, cudaStreamSynchronize(b->stream), "diagnostics synchronize");
   for (int k = 0; k < 4; ++k) out[k] = b->diag_host[k];
   if (b->diag_host[4] > 0)

@@ -178,11 +178,12 @@ cudaError_t launch_inflow_feq1d(T* out, const int bc[4], const double inflow[4][
 void set_create_error(const char* msg);
 
 // ---- reductions (reduce.cu) ----
-// Block partials (5 doubles each: sum h, sum hu, sum hv, min h, bad-cell count) then a
-// fixed-order final pass into out[5].  partials must hold diag_max_blocks() * 5 doubles.
+// Sum h, sum hu, sum hv, min h, bad-cell count into out[5] (device or pinned host memory).  partials
+// must hold diag_max_blocks() * 5 doubles; *done is zero before and after.
 int diag_max_blocks();
 template <class T>
-cudaError_t launch_diagnostics(const StepArgs<T>& a, int q, double* partials, double* out, cudaStream_t st);
+cudaError_t launch_diagnostics(const StepArgs<T>& a, int q, double* partials, unsigned* done, double* out, int sms,
+                               cudaStream_t st);
 // Same reduction with an explicit number of pass-1 blocks (partials must hold nblocks * 5).
 template <class T>
 cudaError_t launch_diagnostics_blocks(const StepArgs<T>& a, int q, int nblocks, double* partials, double* out,
@@ -222,8 +223,8 @@ struct lbm_sw {
   void* mail1d = nullptr;             // exchange between the windows of a line (1D CLUSTER)
   void* pop_staging = nullptr;        // dense populations, for host transfers / collide
   double* diag_partials = nullptr;
-  double* diag_out = nullptr;         // device, 8 doubles
-  double* diag_host = nullptr;        // pinned host, 8 doubles
+  unsigned* diag_done = nullptr;      // device, counts the blocks of a reduction
+  double* diag_host = nullptr;        // pinned host, 8 doubles, written by the reduction
   int kernel = LBM_SW_KERNEL_VEC;
   int temporal_k = 4;
   bool auto_kernel = false;  // the kernel was the library's choice (LBM_SW_KERNEL_AUTO)
