@@ -79,12 +79,6 @@ int obstacle_k(const lbm_sw* h) {
   return std::min(h->temporal_k, 6);
 }
 
-// Whether lbm_sw_step takes register tiles (tile2d.cu): AUTO without a wish for temporal_steps.
-bool tile_active(const lbm_sw* h) {
-  return h->auto_kernel && h->p.temporal_steps == 0 && h->p.dim == 2 && h->p.precision == LBM_SW_FP32 &&
-         static_cast<long long>(h->p.nx) * h->p.ny < kTileCells;
-}
-
 // The launches of n > 0 steps on register tiles, as even as they come: launch(steps) for each.
 template <class F>
 int for_tile_launches(const lbm_sw* h, int n, F&& launch) {
@@ -221,6 +215,12 @@ thread_local std::string g_create_error;
 }  // namespace
 
 namespace lbm {
+// AUTO without a wish for temporal_steps.
+bool tile_active(const lbm_sw* h) {
+  return h->auto_kernel && h->p.temporal_steps == 0 && h->p.dim == 2 && h->p.precision == LBM_SW_FP32 &&
+         static_cast<long long>(h->p.nx) * h->p.ny < kTileCells;
+}
+
 void set_create_error(const char* msg) { g_create_error = msg ? msg : ""; }
 }  // namespace lbm
 
@@ -413,7 +413,7 @@ int lbm_sw_step(lbm_sw* h, int n) {
       return LBM_SW_OK;
     }
   }
-  if (n > 0 && tile_active(h))
+  if (n > 0 && lbm::tile_active(h))
     return for_tile_launches(h, n, [&](int k) {
       const auto a = args<float>(h, h->cur);
       const unsigned char* flags = h->has_obstacles ? h->solid_flags : nullptr;
@@ -501,7 +501,7 @@ int lbm_sw_step_plan(const lbm_sw* h, int n, int* sizes, int max_sizes) {
       return count;
     }
   }
-  if (tile_active(h)) {
+  if (lbm::tile_active(h)) {
     for_tile_launches(h, n, [&](int k) {
       put(k);
       return static_cast<int>(LBM_SW_OK);

@@ -91,6 +91,12 @@ bool adjoint_temporal_supported(const StepArgs<float>& a, int k);
 cudaError_t launch_adjoint_temporal(const StepArgs<float>& a, const float* w0, long long wslot, const ConstsD& kd,
                                     int k, cudaStream_t st, int sm_count);
 
+// kb (1 .. 8) reverse steps per launch on register tiles (adjoint_tile.cu; FP32, any sides and sizes),
+// arguments as above, and the steps per launch that take the least time per step.
+int adjoint_tile_steps(int nx, int ny, int sms);
+cudaError_t launch_adjoint_tile(const StepArgs<float>& a, const float* w0, long long wslot, const ConstsD& kd, int kb,
+                                cudaStream_t st, int sms);
+
 // Batched temporal blocking (temporal.cu): one wavefront unit covers rows [ys, ye) of the
 // output columns [x0, x0 + w) of one instance (clipped at nx) of a batch whose sides are
 // all periodic; a work list holds the units of every instance, grouped by CTA.
@@ -151,6 +157,13 @@ int tile_steps(int nx, int ny, int sms);
 // flags: of solid cells, or nullptr.
 cudaError_t launch_step2d_tile(const StepArgs<float>& a, const ConstsD& kd, int kb, const unsigned char* flags,
                                cudaStream_t st, int sms);
+
+// The same (BGK, no solid cells), with the moments of every step t = 1 .. kb in the three planes at
+// wout + (t - 1) * wslot.
+cudaError_t launch_step2d_tile_store_w(const StepArgs<float>& a, const ConstsD& kd, int kb, float* wout, long long wslot,
+                                       cudaStream_t st, int sms);
+// Whether a handle's steps run on register tiles (api.cu: AUTO, FP32, below 5 * 2^17 cells).
+bool tile_active(const lbm_sw* h);
 
 // ---- 1D launchers (kernels_1d.cu) ----
 template <class T>

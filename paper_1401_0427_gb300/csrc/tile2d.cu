@@ -34,24 +34,19 @@
 #include "scheme.cuh"
 #include "step2d_vec.cuh"
 #include "temporal.cuh"
+#include "tile2d.cuh"
 
 namespace lbm {
 namespace {
 
-constexpr int kTileCols = 64;
-
-// Output columns and rows per tile (w even), tiles per row of tiles, steps, left halo (kb
-// rounded up to even, so that pairs start at even columns).
-struct TilePart {
-  int w, h, strips, segs, kb, hl;
-};
-
 // OBST: solid cells (kSolid* flags): a population that would come from a solid cell is the cell's
 // own reflected one, the family normal to the face negated; solid cells keep their populations.
-template <int R, int NW, bool MRT, bool PER, bool OBST>
+// STORE_W: the moments (h, hu, hv) of every step are also written, for the tile's output cells, to
+// the three planes at wout + (step - 1) * wslot (the record of the discrete adjoint).
+template <int R, int NW, bool MRT, bool PER, bool OBST, bool STORE_W>
 __global__ void __launch_bounds__(32 * NW, 1)
     step2d_tile(const StepArgs<float> A, const Consts<float> Kc, const TilePart P,
-                const unsigned char* __restrict__ flags) {
+                const unsigned char* __restrict__ flags, float* __restrict__ wout, long long wslot) {
   extern __shared__ __align__(16) float2 smem2[];
   float2(*const edge)[NW][2][3][32] = reinterpret_cast<float2(*)[NW][2][3][32]>(smem2);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -183,9 +178,23 @@ __global__ void __launch_bounds__(32 * NW, 1)
           b[4 + 4 * c] = up.y;
           below[c] = yp;  // for row r + 1
         }
-        float h, qx, qy;
-        collide13_any<float, MRT>(a, Kc, h, qx, qy);
-        collide13_any<float, MRT>(b, Kc, h, qx, qy);
+        float2 h, qx, qy;
+        collide13_any<float, MRT>(a, Kc, h.x, qx.x, qy.x);
+        collide13_any<float, MRT>(b, Kc, h.y, qx.y, qy.y);
+        if constexpr (STORE_W) {
+          if (2 * lane >= P.hl && 2 * lane < P.hl + P.w && tx < nx && ty + r >= y0 && ty + r < y1) {
+            float* const g = wout + (s - 1) * wslot + static_cast<long long>(ty + r) * A.pitch + tx;
+            if (tx + 1 < nx) {
+              *reinterpret_cast<float2*>(g) = h;
+              *reinterpret_cast<float2*>(g + A.plane) = qx;
+              *reinterpret_cast<float2*>(g + 2 * A.plane) = qy;
+            } else {
+              g[0] = h.x;
+              g[A.plane] = qx.x;
+              g[2 * A.plane] = qy.x;
+            }
+          }
+        }
 #pragma unroll
         for (int p = 0; p < 13; ++p) {
           F[r][p].x = OBST && (solid[r] & kSolidSelf) ? F[r][p].x : a[p];
@@ -230,25 +239,6 @@ __global__ void __launch_bounds__(32 * NW, 1)
   }
 }
 
-// Tiles of a launch of kb steps: strips of equal even width, row segments for whole waves of
-// one CTA per SM.
-TilePart tile_part(int nx, int ny, int rows, int kb, int sms) {
-  TilePart P;
-  P.kb = kb;
-  P.hl = kb + (kb & 1);
-  const int wmax = (kTileCols - P.hl - kb) & ~1, hmax = rows - 2 * kb;
-  P.strips = (nx + wmax - 1) / wmax;
-  P.w = (nx + P.strips - 1) / P.strips;
-  P.w += P.w & 1;
-  P.strips = (nx + P.w - 1) / P.w;
-  const int need = (ny + hmax - 1) / hmax;
-  const int waves = (P.strips * need + sms - 1) / sms;
-  const int segs = std::max(need, std::min(waves * sms / P.strips, (ny + 3) / 4));
-  P.h = (ny + segs - 1) / segs;
-  P.segs = (ny + P.h - 1) / P.h;
-  return P;
-}
-
 // The tile of 48 rows (BGK 12 warps of 4 rows, MRT 16 warps of 3, whose transforms want the
 // registers) or of 32 (16 warps of 2: less latency per step where a wave of them covers the
 // grid), by the time in us per launch fitted to grids of 64^2 to 800^2: a wave of tiles takes
@@ -269,24 +259,30 @@ TileChoice tile_choose(int nx, int ny, int kb, int sms) {
   return best;
 }
 
-template <int R, int NW, bool MRT, bool OBST>
-cudaError_t launch_tile(const StepArgs<float>& a, const ConstsD& kd, const TilePart& P, const unsigned char* flags,
+struct TileExtra {
+  const unsigned char* flags;
+  float* wout;
+  long long wslot;
+};
+
+template <int R, int NW, bool MRT, bool OBST, bool STORE_W>
+cudaError_t launch_tile(const StepArgs<float>& a, const ConstsD& kd, const TilePart& P, const TileExtra& x,
                         cudaStream_t st) {
   constexpr size_t smem = sizeof(float2) * 2 * NW * 2 * 3 * 32;
   static_assert(smem <= 48 * 1024, "dynamic shared memory without an attribute");
   const bool per = a.bc[LBM_SW_SIDE_XM] == LBM_SW_BC_PERIODIC && a.bc[LBM_SW_SIDE_YM] == LBM_SW_BC_PERIODIC;
-  return launch_pdl(per ? step2d_tile<R, NW, MRT, true, OBST> : step2d_tile<R, NW, MRT, false, OBST>,
-                    dim3(P.strips * P.segs), dim3(32 * NW), smem, st, a, to_consts<float>(kd), P, flags);
+  return launch_pdl(per ? step2d_tile<R, NW, MRT, true, OBST, STORE_W> : step2d_tile<R, NW, MRT, false, OBST, STORE_W>,
+                    dim3(P.strips * P.segs), dim3(32 * NW), smem, st, a, to_consts<float>(kd), P, x.flags, x.wout, x.wslot);
 }
 
 template <bool OBST>
-cudaError_t launch_tile_choice(const StepArgs<float>& a, const ConstsD& kd, const TileChoice& c,
-                               const unsigned char* flags, cudaStream_t st) {
+cudaError_t launch_tile_choice(const StepArgs<float>& a, const ConstsD& kd, const TileChoice& c, const TileExtra& x,
+                               cudaStream_t st) {
   if (c.tall)
-    return kd.mrt ? launch_tile<3, 16, true, OBST>(a, kd, c.P, flags, st)
-                  : launch_tile<4, 12, false, OBST>(a, kd, c.P, flags, st);
-  return kd.mrt ? launch_tile<2, 16, true, OBST>(a, kd, c.P, flags, st)
-                : launch_tile<2, 16, false, OBST>(a, kd, c.P, flags, st);
+    return kd.mrt ? launch_tile<3, 16, true, OBST, false>(a, kd, c.P, x, st)
+                  : launch_tile<4, 12, false, OBST, false>(a, kd, c.P, x, st);
+  return kd.mrt ? launch_tile<2, 16, true, OBST, false>(a, kd, c.P, x, st)
+                : launch_tile<2, 16, false, OBST, false>(a, kd, c.P, x, st);
 }
 
 }  // namespace
@@ -308,7 +304,17 @@ cudaError_t launch_step2d_tile(const StepArgs<float>& a, const ConstsD& kd, int 
                                cudaStream_t st, int sms) {
   if (kb < 1 || kb > 8) return cudaErrorInvalidValue;
   const TileChoice c = tile_choose(a.nx, a.ny, kb, std::max(sms, 1));
-  return flags ? launch_tile_choice<true>(a, kd, c, flags, st) : launch_tile_choice<false>(a, kd, c, nullptr, st);
+  const TileExtra x{flags, nullptr, 0};
+  return flags ? launch_tile_choice<true>(a, kd, c, x, st) : launch_tile_choice<false>(a, kd, c, x, st);
+}
+
+cudaError_t launch_step2d_tile_store_w(const StepArgs<float>& a, const ConstsD& kd, int kb, float* wout, long long wslot,
+                                       cudaStream_t st, int sms) {
+  if (kb < 1 || kb > 8 || kd.mrt) return cudaErrorInvalidValue;
+  const TileChoice c = tile_choose(a.nx, a.ny, kb, std::max(sms, 1));
+  const TileExtra x{nullptr, wout, wslot};
+  return c.tall ? launch_tile<4, 12, false, false, true>(a, kd, c.P, x, st)
+                : launch_tile<2, 16, false, false, true>(a, kd, c.P, x, st);
 }
 
 }  // namespace lbm

@@ -350,3 +350,28 @@ def test_fused_adjoint_with_boundaries(nx, ny, bc, k):
     scale = max(np.abs(b).max() for b in g_b)
     for a, b in zip(g_a, g_b):
         assert np.abs(a - b).max() <= 1e-5 * scale
+
+
+@pytest.mark.parametrize("bc", [(P, P, P, P), (W, O, I, W), (O, I, W, O), (W, W, W, W), (I, W, P, P)],
+                         ids=lambda b: "".join("PWOI"[k] for k in b))
+@pytest.mark.parametrize("nx,ny,steps", [(1, 1, 3), (3, 2, 8), (1, 9, 9), (7, 5, 17), (49, 21, 8), (97, 41, 25),
+                                         (640, 50, 11)])
+def test_small_grids_record_and_reverse_on_register_tiles(nx, ny, steps, bc):
+    """FP32 handles below 5 * 2^17 cells record, and take the reverse steps, up to 8 per launch on
+    register tiles; a handle held to KERNEL_VEC takes one per launch.  The same bits of h^T, and
+    gradients that agree as those of the scalar and the vectorised reverse steps do."""
+    W0 = [x.reshape(ny, nx) for x in inputs.random_states(nx * ny, seed=510 + nx, h=(0.8, 1.4), speed=0.25)]
+    h_obs = np.ones((ny, nx))
+    kw = dict(precision=lbm_sw.FP32, bc=bc, inflow=INFLOW, stream=torch_stream())
+    grads, states = [], []
+    for kernel in (lbm_sw.KERNEL_AUTO, lbm_sw.KERNEL_VEC):
+        with lbm_sw.Simulation(nx, ny, kernel=kernel, **kw) as sim:
+            sim.set_state(*W0)
+            with lbm_sw.Tape(sim, steps) as tape:
+                tape.record()
+                states.append(sim.moments())
+                grads.append(tape.adjoint(states[-1][0] - h_obs, want_momentum=True))
+    for a, b in zip(*states):
+        assert np.array_equal(a, b)
+    for a, b in zip(*grads):
+        assert np.abs(a - b).max() <= 1e-5 * max(np.abs(a).max(), 1e-30)
