@@ -101,6 +101,9 @@ struct Consts {
   T a_2, a_4g;
   // 2D, FP64 (collide13_fixed): |1 - s|, s / 4 and s c in units of 2^-64, and whether they are below one
   unsigned long long x_om, x_s4, x_sc;
+  // the least difference of the families' exponents at which s c q stays below 2^62 units of the
+  // depths' (q is below 2^62 of its own): s c 2^-least_sc <= 1
+  int least_sc;
   // 1D, FP64 (collide5_fixed): s / 2 and s a / 4 likewise, s a / (8 g)
   unsigned long long x_s2, x_s1a;
   T s_1g;
@@ -111,6 +114,13 @@ struct Consts {
 inline __host__ unsigned long long in_2_64(double v) {
   const double a = v < 0 ? -v : v;
   return a >= 1.0 ? ~0ull : static_cast<unsigned long long>(a * 18446744073709551616.0);
+}
+
+// the most negative d >= -31 with v 2^-d <= most
+inline __host__ int least_shift(double v, double most) {
+  int d = 0;
+  while (d > -31 && v * static_cast<double>(1LL << (1 - d)) <= most) --d;
+  return d;
 }
 
 template <class T>
@@ -140,12 +150,13 @@ __host__ Consts<T> make_consts(double g, double lambda, double s, double a) {
   k.x_om = in_2_64(1.0 - st);
   k.x_s4 = in_2_64(st / 4.0);
   k.x_sc = in_2_64(st * c);
+  k.least_sc = least_shift(st * c, 1.0);
   k.om_neg = st > 1.0;
   k.fixed_ok = st >= 0.0 && st <= 2.0 && st * c < 1.0;
   k.x_s2 = in_2_64(st / 2.0);
   k.x_s1a = in_2_64(st * a / 4.0);
   k.s_1g = static_cast<T>(st * a / (8.0 * g));
-  k.fixed1_ok = k.fixed_ok && st * a < 4.0;
+  k.fixed1_ok = k.fixed_ok && st * a <= 1.0;
   for (int i = 0; i < 10; ++i) k.r[i] = k.s;
   set_mrt_folded(k);
   return k;
@@ -195,6 +206,12 @@ __device__ __forceinline__ long long fix_one_more(double x, int e, bool& ok) {
   const int d = ((e - exp_field(x)) >> 20) + 1;
   ok = ok && d >= 0;
   return with_sign((mantissa(x) << 8) >> (d & 63) >> (d > 63 ? 63 : 0), __double2hiint(x));
+}
+// m from units of an exponent d below into units of e's; ok: cleared where d < least, the d down to
+// which the result stays in range (below)
+__device__ __forceinline__ unsigned long long to_units(unsigned long long m, int d, int least, bool& ok) {
+  ok = ok && d >= least;
+  return d >= 0 ? m >> min(d, 63) : m << (-d & 31);
 }
 // m c / 2^64 without the last partial product (less than 3 units too small)
 __device__ __forceinline__ unsigned long long times_2_64(unsigned long long m, unsigned long long c) {
@@ -384,13 +401,9 @@ __device__ __forceinline__ bool collide13_fixed(double f[13], const Consts<doubl
   const int sx = static_cast<int>(v[1] >> 32), sy = static_cast<int>(v[2] >> 32);  // their sign bits
   const unsigned long long ax = static_cast<unsigned long long>(v[1] < 0 ? -v[1] : v[1]);
   const unsigned long long ay = static_cast<unsigned long long>(v[2] < 0 ? -v[2] : v[2]);
-  // s c q in units of the f family's: shifted by the exponents' difference
-  auto to_f = [&](unsigned long long q, int e) {
-    const int d = (ef - e) >> 20;
-    ok = ok && d >= -6;
-    return d >= 0 ? q >> min(d, 63) : q << (-d & 7);
-  };
-  const long long cx = with_sign(to_f(times_2_64(ax, k.x_sc), ex), sx), cy = with_sign(to_f(times_2_64(ay, k.x_sc), ey), sy);
+  // s c q, in units of the f family's
+  const long long cx = with_sign(to_units(times_2_64(ax, k.x_sc), (ef - ex) >> 20, k.least_sc, ok), sx);
+  const long long cy = with_sign(to_units(times_2_64(ay, k.x_sc), (ef - ey) >> 20, k.least_sc, ok), sy);
   const long long x4 = with_sign(times_2_64(ax, k.x_s4), sx), y4 = with_sign(times_2_64(ay, k.x_s4), sy);
   const long long fr = fix_one_more(r, ef, ok);
   const long long fxx = fix_one_more(pxx, ex, ok), fxy = fix_one_more(pxy, ex, ok);
@@ -759,10 +772,7 @@ __device__ __forceinline__ bool collide5_fixed(double f[5], const Consts<double>
   const unsigned long long aq = static_cast<unsigned long long>(v[1] < 0 ? -v[1] : v[1]);
   const long long z = fix_one_more(mul(uu, k.s_1g), ef, ok) - with_sign(times_2_64_round(ah, k.x_s1a), sh);  // -s f0^eq / 2
   const long long r = with_sign(times_2_64_round(ah, k.x_s2), sh) + z;  // s (h - f0^eq) / 2
-  const int d = (ef - eg) >> 20;
-  ok = ok && d >= -6;
-  const unsigned long long cm = times_2_64_round(aq, k.x_sc);
-  const long long c = with_sign(d >= 0 ? cm >> min(d, 63) : cm << (-d & 7), sq);
+  const long long c = with_sign(to_units(times_2_64_round(aq, k.x_sc), (ef - eg) >> 20, k.least_sc, ok), sq);
   const long long q2 = with_sign(times_2_64_round(aq, k.x_s2), sq), p = fix_one_more(pq, eg, ok);
   if (!ok) return false;
   const int flip = k.om_neg ? static_cast<int>(0x80000000u) : 0;

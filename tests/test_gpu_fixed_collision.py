@@ -56,3 +56,28 @@ def test_infinities_and_nan_stay_where_they_stream():
         want = oracle_post(F0, 2, p, 2)
     assert np.array_equal(a, b, equal_nan=True)
     assert np.array_equal(np.isfinite(a), np.isfinite(want))
+
+
+@pytest.mark.parametrize("lam", [1.0, 8.0])
+@pytest.mark.parametrize("rates", [None, [1.8] * 13, [0.0, 1.1, 1.2, 1.3, 1.4, 0.0, 1.5, 1.6, 1.7, 0.0, 1.99, 1.65, 0.9]],
+                         ids=["bgk", "mrt-equal", "mrt"])
+@pytest.mark.parametrize("dim", [1, 2])
+def test_momenta_far_above_the_depths(dim, rates, lam):
+    """Momenta up to 2^5 times the depths (further up the oracle's entropy variables lose digits):
+    s c q in units of the depths' leaves the integers' range in some cells, near it in others.  One
+    collision (a second one would divide by depths near zero)."""
+    ny, nx, q = (1, 640, 5) if dim == 1 else (10, 640, 13)
+    F0 = inputs.random_populations(q, ny, nx, seed=9720)
+    nf = 3 if dim == 1 else 5
+    F0[:nf] = 0.245 + 0.01 * (F0[:nf] - 0.25)
+    F0[nf:] *= 1e-3
+    big = inputs.uniform(9721, ny * nx, -1.0, 5.0).reshape(ny, nx)  # powers of two
+    F0[nf] += 2.0 ** big
+    if dim == 2:
+        F0[11] -= 2.0 ** inputs.uniform(9722, ny * nx, -1.0, 5.0).reshape(ny, nx)
+    bc, a = ((W, W), 0.15) if dim == 1 else ((P, P, W, W), 0.05)
+    if rates is not None and dim == 1:
+        rates = [0.0, rates[1], rates[3], 0.0, rates[10]]
+    p = oracle.params(nx, ny, a=a, lam=lam, bc=bc, inflow=None, s_moments=rates)
+    got = gpu_post(F0, 0, dim=dim, precision=lbm_sw.FP64, bc=bc, inflow=None, a=a, lam=lam, mrt_rates=rates)
+    assert rel_max(got, oracle_post(F0, 0, p, dim)) <= FP64_TOL
