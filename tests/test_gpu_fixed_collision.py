@@ -1,4 +1,4 @@
-"""The FP64 collision in 64-bit integers and its way out to fused multiply-adds: against the oracle
+"""The FP64 collisions in 64-bit integers and its way out to fused multiply-adds: against the oracle
 where the populations of a family differ much in size, and where they are zero, tiny or huge."""
 
 import numpy as np
@@ -30,6 +30,23 @@ def test_sizes_apart_match_the_oracle(s, lam, kernel):
     got = gpu_post(F0, 1, dim=2, precision=lbm_sw.FP64, bc=(P, P, W, W), inflow=None, a=0.05, kernel=kernel, lam=lam, s=s)
     want = oracle_post(F0, 1, p, 2)
     assert rel_max(got, want) <= FP64_TOL
+
+
+@pytest.mark.parametrize("kernel", [lbm_sw.KERNEL_SIMPLE, lbm_sw.KERNEL_VEC], ids=["simple", "vec"])
+def test_mrt_sizes_apart_match_the_oracle(kernel):
+    """The same inputs with every moment at its own rate, some zero."""
+    ny, nx = 21, 70
+    rates = [0.0, 1.1, 0.0, 1.3, 1.4, 0.0, 1.5, 0.0, 1.7, 0.0, 1.99, 1.65, 0.9]
+    F0 = inputs.random_populations(13, ny, nx, seed=9730)
+    k = np.floor(inputs.uniform(9731, F0.size, -70.0, 4.0)).reshape(F0.shape)
+    F0 = np.where(inputs.uniform(9732, F0.size).reshape(F0.shape) < 0.5, F0, F0 * 2.0 ** k)
+    F0[:, 3:5] = np.where(inputs.uniform(9733, F0[:, 3:5].size).reshape(F0[:, 3:5].shape) < 0.5, F0[:, 3:5], 0.0)
+    F0[0] = np.abs(F0[0]) + 0.5
+    F0[5:] *= 0.05
+    p = oracle.params(nx, ny, a=0.05, bc=(P, P, W, W), s_moments=rates)
+    got = gpu_post(F0, 1, dim=2, precision=lbm_sw.FP64, bc=(P, P, W, W), inflow=None, a=0.05, kernel=kernel,
+                   mrt_rates=rates)
+    assert rel_max(got, oracle_post(F0, 1, p, 2)) <= FP64_TOL
 
 
 @pytest.mark.parametrize("scale", [2.0 ** -600, 2.0 ** -300, 1.0, 2.0 ** 300])
