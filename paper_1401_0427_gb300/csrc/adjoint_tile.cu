@@ -2,11 +2,11 @@
 // grids below the wavefronts': the tiles of tile2d.cu with the populations Phi pulled in the reverse
 // direction (+x movers from x + 1, and so on), the transposed side rules of adjoint_step_vec, and
 // the local product (1 - s) psi + s M^T D(W)^T psi with the moments W^{n-1} of each step, which a
-// thread loads for the next step while it works on this one.  One step per launch is bound by the
-// launch and the dependent reads from L2: 4.4, 4.6 and 6.4 us per step at 128^2, 256^2 and 512^2,
-// here 2.0, 2.3 and 4.4 (walls 2.5, 2.8 and 4.9), bound by one CTA's serial rows and the loads of W.
-// Three rows per thread and 12 warps: Phi and the moments take 48 registers a row, and four rows
-// would not fit the 168 of a thread.
+// thread loads a step ahead.  One step per launch is bound by the launch and the dependent reads
+// from L2: 4.4, 4.6 and 6.4 us per step at 128^2, 256^2 and 512^2, here 1.7, 1.9 and 3.9 (walls the
+// same within 0.1), bound by the rows' chains and the recomputed halo.
+// Two rows per thread and 16 warps, 128 registers: three rows and 12 warps, 168 registers, with the
+// moments loaded behind their last use, took 2.0, 2.3 and 4.4 (walls 2.7, 2.8 and 4.9).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -21,7 +21,7 @@
 namespace lbm {
 namespace {
 
-constexpr int kRows = 3, kWarps = 12;
+constexpr int kRows = 2, kWarps = 16;
 
 template <bool PER>
 __global__ void __launch_bounds__(32 * kWarps, 1)
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
     const float* g = plane + row[r];
     return split ? make_float2(__ldg(g + gx), __ldg(g + gx2)) : __ldg(reinterpret_cast<const float2*>(g + gx));
   };
-  float2 F[R][13], W[R][3];
+  float2 F[R][13], W[R][3], N[R][3];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
 #pragma unroll
@@ -91,6 +91,11 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
     __syncthreads();
     const int rem = P.kb - s;
     if (ty + R <= y0 - rem || ty >= y1 + rem) continue;
+    if (s < P.kb)
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) N[r][c] = load(w0 - s * wslot + c * A.plane, r, 1.f);
     auto step = [&](auto xs, auto ys) {
       float2 below[3], above[3];
 #pragma unroll
@@ -144,9 +149,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
         float za[3], zb[3];
         equilibrium_vjp(W[r][0].x, W[r][1].x, W[r][2].x, a, Kc, za[0], za[1], za[2]);
         equilibrium_vjp(W[r][0].y, W[r][1].y, W[r][2].y, b, Kc, zb[0], zb[1], zb[2]);
-        if (s < P.kb)  // the next step's moments
 #pragma unroll
-          for (int c = 0; c < 3; ++c) W[r][c] = load(w0 - s * wslot + c * A.plane, r, 1.f);
+        for (int c = 0; c < 3; ++c) W[r][c] = N[r][c];
 #pragma unroll
         for (int p = 0; p < 13; ++p) {
           const int f = p < 5 ? 0 : (p < 9 ? 1 : 2);
