@@ -379,7 +379,7 @@ constexpr int kRowsPerCta = sizeof(T) == 8 ? 1 : 4;
 template <class T, class F>
 cudaError_t with_residency(const StepArgs<T>& a, F&& launch) {
   if constexpr (sizeof(T) == 4)
-    return launch(std::integral_constant<int, 1>{});
+    return launch(std::integral_constant<int, 4>{});
   else if (static_cast<long long>(a.nx) * a.ny >= (1LL << 17))
     return launch(std::integral_constant<int, 24>{});
   else
