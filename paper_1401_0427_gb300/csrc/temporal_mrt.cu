@@ -14,13 +14,15 @@
 namespace lbm {
 namespace {
 
-template <int K, int COLS, int PF, bool L0R, bool PER>
+// ODD: any nx, with the tests for pairs that straddle the seam or the last column; even widths go
+// without (us per step at 4096^2: 88.1, 96.5 with them; 1024^2 8.1 and 8.6; walls 3000^2 56.7 and 57.3).
+template <int K, int COLS, int PF, bool L0R, bool PER, bool ODD>
 __global__ void __launch_bounds__(COLS / 2, 2)
     step2d_temporal_x2_mrt(const StepArgs<float> A, const Consts<float> Kc, const Partition P) {
   extern __shared__ __align__(16) float smem[];
   pdl_wait();
   run_segment(P, A.ny, [&](int strip, int ys, int ye) {
-    pair_wave<K, COLS, PF, false, L0R, PER, true, true, false, PER>(A, Kc, smem, strip * P.w, P.w, ys, ye, nullptr, 0);
+    pair_wave<K, COLS, PF, false, L0R, PER, true, ODD, false, PER>(A, Kc, smem, strip * P.w, P.w, ys, ye, nullptr, 0);
   });
   pdl_done();
 }
@@ -28,14 +30,14 @@ __global__ void __launch_bounds__(COLS / 2, 2)
 template <int K, int COLS, int PF, bool L0R, bool PER>
 cudaError_t launch_pairs_mrt(const StepArgs<float>& a, const ConstsD& kd, cudaStream_t st, int sm_count) {
   const size_t smem = PairShape<K, COLS, PF, L0R>::floats() * sizeof(float);
-  const void* fn = reinterpret_cast<const void*>(step2d_temporal_x2_mrt<K, COLS, PF, L0R, PER>);
+  const auto fn = a.nx & 1 ? step2d_temporal_x2_mrt<K, COLS, PF, L0R, PER, true>
+                           : step2d_temporal_x2_mrt<K, COLS, PF, L0R, PER, false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  const int resident = cached_resident(fn, COLS / 2, smem);
+  const int resident = cached_resident(reinterpret_cast<const void*>(fn), COLS / 2, smem);
   const Partition Q = pair_partition(a.nx, a.ny, K, COLS, resident * std::max(sm_count, 1));
   const Consts<float> K_ = make_consts_mrt<float>(kd.g, kd.lambda, kd.s, kd.a, kd.rates, 10);
-  return launch_pdl(step2d_temporal_x2_mrt<K, COLS, PF, L0R, PER>, dim3(Q.strips * Q.segments), dim3(COLS / 2), smem,
-                    st, a, K_, Q);
+  return launch_pdl(fn, dim3(Q.strips * Q.segments), dim3(COLS / 2), smem, st, a, K_, Q);
 }
 
 // The shapes of the BGK kernel at each K.

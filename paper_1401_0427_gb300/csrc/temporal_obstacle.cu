@@ -36,32 +36,41 @@ __global__ void obstacle_flags_kernel(const unsigned char* __restrict__ solid, u
   }
 }
 
-// Every side periodic: the row loop unrolled by three, as the kernels without obstacles.
-template <int K, int COLS, int PF, bool L0R, bool PER>
+// Every side periodic: the branch-free steady state (3000 x 2000: 35.8 us per step; the row loop
+// unrolled by three 37.5).
+// ODD as in temporal_mrt.cu (odd widths: 37.0).
+template <int K, int COLS, int PF, bool L0R, bool PER, bool ODD>
 __global__ void __launch_bounds__(COLS / 2, 2)
     step2d_temporal_obstacle(const StepArgs<float> A, const Consts<float> Kc, const Partition P,
                              const unsigned char* __restrict__ flags) {
   extern __shared__ __align__(16) float smem[];
   pdl_wait();
   run_segment(P, A.ny, [&](int strip, int ys, int ye) {
-    pair_wave<K, COLS, PF, false, L0R, PER, false, true, PER, false, true>(A, Kc, smem, strip * P.w, P.w, ys, ye, nullptr,
+    pair_wave<K, COLS, PF, false, L0R, PER, false, ODD, false, PER, true>(A, Kc, smem, strip * P.w, P.w, ys, ye, nullptr,
                                                                            0, flags);
   });
   pdl_done();
 }
 
-template <int K, int COLS, int PF, bool L0R>
-cudaError_t launch_obst(const StepArgs<float>& a, const ConstsD& kd, const unsigned char* flags, cudaStream_t st,
+template <int K, int COLS, int PF, bool L0R, bool ODD>
+cudaError_t launch_obst_odd(const StepArgs<float>& a, const ConstsD& kd, const unsigned char* flags, cudaStream_t st,
                         int sm_count) {
   const size_t smem = PairShape<K, COLS, PF, L0R>::floats() * sizeof(float);
   const bool per = a.bc[LBM_SW_SIDE_XM] == LBM_SW_BC_PERIODIC && a.bc[LBM_SW_SIDE_YM] == LBM_SW_BC_PERIODIC;
-  const auto fn = per ? step2d_temporal_obstacle<K, COLS, PF, L0R, true> : step2d_temporal_obstacle<K, COLS, PF, L0R, false>;
+  const auto fn =
+      per ? step2d_temporal_obstacle<K, COLS, PF, L0R, true, ODD> : step2d_temporal_obstacle<K, COLS, PF, L0R, false, ODD>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const int resident = cached_resident(reinterpret_cast<const void*>(fn), COLS / 2, smem);
   const Partition Q = pair_partition(a.nx, a.ny, K, COLS, resident * std::max(sm_count, 1));
   return launch_pdl(fn, dim3(Q.strips * Q.segments), dim3(COLS / 2), smem, st, a,
                     make_consts<float>(kd.g, kd.lambda, kd.s, kd.a), Q, flags);
+}
+template <int K, int COLS, int PF, bool L0R>
+cudaError_t launch_obst(const StepArgs<float>& a, const ConstsD& kd, const unsigned char* flags, cudaStream_t st,
+                        int sm_count) {
+  return a.nx & 1 ? launch_obst_odd<K, COLS, PF, L0R, true>(a, kd, flags, st, sm_count)
+                  : launch_obst_odd<K, COLS, PF, L0R, false>(a, kd, flags, st, sm_count);
 }
 
 }  // namespace

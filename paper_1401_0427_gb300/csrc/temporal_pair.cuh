@@ -100,7 +100,7 @@ template <int K, int COLS, int PF, bool STORE_W, bool L0R, bool PER = true, bool
 __device__ __forceinline__ void pair_wave(const StepArgs<float>& A, const Consts<float>& Kc, float* smem, int x0, int w,
                                           int ys, int ye, float* __restrict__ wout, long long wslot,
                                           const unsigned char* __restrict__ flags = nullptr) {
-  static_assert(!OBST || (K <= 7 && !STORE_W && L0R && ODD), "obstacles: one flag byte per row, level 0 in registers");
+  static_assert(!OBST || (K <= 7 && !STORE_W && L0R), "obstacles: one flag byte per row, level 0 in registers");
   using S = PairShape<K, COLS, PF, L0R>;
   constexpr int RS = S::RS;
   const int c = threadIdx.x;  // pair index: tile columns 2c, 2c + 1
