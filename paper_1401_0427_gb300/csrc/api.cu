@@ -20,8 +20,9 @@ namespace {
 constexpr long long kAutoTemporalCells = 3LL << 17;
 
 // 2D FP32 grids below this size (cells) take several steps per launch on register tiles under
-// AUTO: 800^2 4.3 us per step against 4.5 for the wavefront (walls, inflow and outflow 5.1 / 5.4,
-// MRT 6.0 / 6.2), 900^2 5.4 against 5.3 (6.3 / 6.0, 7.5 / 7.0).
+// AUTO where the wavefront does not apply or two waves of tiles cover the grid.  us per step, tiles
+// against the wavefront, BGK and MRT: two waves 740^2 3.9 / 4.1 and 5.4 / 5.7, with walls 4.6 / 4.9
+// and 6.1 / 6.2; three waves 768^2 4.2 / 4.1 and 5.9 / 5.7, 900 x 600 with walls 5.5 / 4.6 and 7.3 / 5.8.
 constexpr long long kTileCells = 5LL << 17;
 
 int fail(lbm_sw* h, int code, const char* fmt, ...) {
@@ -217,8 +218,13 @@ thread_local std::string g_create_error;
 namespace lbm {
 // AUTO without a wish for temporal_steps.
 bool tile_active(const lbm_sw* h) {
-  return h->auto_kernel && h->p.temporal_steps == 0 && h->p.dim == 2 && h->p.precision == LBM_SW_FP32 &&
-         static_cast<long long>(h->p.nx) * h->p.ny < kTileCells;
+  if (!h->auto_kernel || h->p.temporal_steps != 0 || h->p.dim != 2 || h->p.precision != LBM_SW_FP32 ||
+      static_cast<long long>(h->p.nx) * h->p.ny >= kTileCells)
+    return false;
+  if (!temporal_active(h) && obstacle_k(h) == 0) return true;
+  int waves = 0;
+  tile_steps(h->p.nx, h->p.ny, std::max(h->sm_count, 1), &waves);
+  return waves <= 2;
 }
 
 void set_create_error(const char* msg) { g_create_error = msg ? msg : ""; }

@@ -153,7 +153,7 @@ cudaError_t launch_step2d_temporal_obstacle(const StepArgs<float>& a, const Cons
 
 // kb (1 .. 8) fused steps on tiles held in registers (tile2d.cu; FP32, BGK or MRT, any sides and
 // sizes), and the steps per launch that take the least time per step on an nx x ny grid.
-int tile_steps(int nx, int ny, int sms);
+int tile_steps(int nx, int ny, int sms, int* waves = nullptr);
 // flags: of solid cells, or nullptr.
 cudaError_t launch_step2d_tile(const StepArgs<float>& a, const ConstsD& kd, int kb, const unsigned char* flags,
                                cudaStream_t st, int sms);

@@ -287,14 +287,15 @@ cudaError_t launch_tile_choice(const StepArgs<float>& a, const ConstsD& kd, cons
 
 }  // namespace
 
-int tile_steps(int nx, int ny, int sms) {
+int tile_steps(int nx, int ny, int sms, int* waves) {
   int best = 8;
   double us = 1e300;
   for (int kb = 8; kb >= 4; --kb) {
-    const double per_step = tile_choose(nx, ny, kb, sms).us / kb;
-    if (per_step < us) {
-      us = per_step;
+    const TileChoice c = tile_choose(nx, ny, kb, sms);
+    if (c.us / kb < us) {
+      us = c.us / kb;
       best = kb;
+      if (waves) *waves = (c.P.strips * c.P.segs + sms - 1) / sms;
     }
   }
   return best;
