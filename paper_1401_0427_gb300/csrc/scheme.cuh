@@ -503,7 +503,7 @@ __device__ __forceinline__ void collide13_mrt(T f[13], const Consts<T>& k, T& h,
 // Bounds, with a family's largest population below one: 2 c q - (f1 - f3) below 6, a relaxed
 // population below 8 (the integers' range).
 //
-// us per step, before and after: 480 x 120 19.7 and 6.3, 512^2 63.7 and 19.5, 1536^2 539 and 145 (BGK
+// us per step, before and after: 480 x 120 19.7 and 6.3, 512^2 63.7 and 20.2, 1536^2 539 and 153 (BGK
 // 141).  Error against extended precision after 300 steps of a dam break on 40^2 cells: h 8.8e-17 and
 // 5.8e-17 (relative L1), q 4.2e-15 and 2.3e-15; no drift of the depths' sum over 10^5 steps in either.
 __device__ __forceinline__ bool collide13_mrt_fixed(double f[13], const Consts<double>& k, double& h, double& qx,

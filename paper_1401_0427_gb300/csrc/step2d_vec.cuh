@@ -286,7 +286,9 @@ __device__ __forceinline__ void vec_row(const StepArgs<T>& A, const Consts<T>& K
                          xm[1][k], o4[1][k], xp[2][k], o2[2][k], xm[2][k], o4[2][k]};
 #pragma unroll
       for (int p = 0; p < 13; ++p) f[p] = own[p];
-    } else {
+    } else if (sizeof(T) == 4 || x0 + k < nx) {
+      // FP64: padding cells would take their warp out of the integer collision (103 x 270: 7.9 us per step
+      // with them, 4.9 without)
       collide13_any<T, MRT>(f, K, wh, wx, wy);
     }
     const bool valid = x0 + k < nx;  // padding cells are stored as zero
