@@ -15,17 +15,20 @@
  * 2-potentiels-st-venant-1d-suite, 3-st-venant-contraintes-2, 3-st-venant-enplus),
  * with p = g h^2 / 2 (the gamma = 2 system), and the collision is the BGK form of
  * Eq. 2-relaxation (every rate equal to s).  Streaming moves each population one
- * cell per step (lambda = dx/dt).  The 2D BGK kernels evaluate f + s (f^eq - f) as
- * (1 - s) f + s f^eq with s folded into the equilibrium's constants: the same
- * operator, with 13 operations fewer per cell; a state at equilibrium settles within
- * about one unit in the last place of itself instead of mapping to itself bit for bit
- * (the MRT form, lbm_sw_set_relaxation, relaxes f^eq - f and keeps that fixed point).
+ * cell per step (lambda = dx/dt).  The BGK kernels evaluate f + s (f^eq - f) as
+ * (1 - s) f + s f^eq with s folded into the equilibrium's constants (2D, and 1D in FP64):
+ * the same operator, with 13 operations fewer per 2D cell; a state at equilibrium settles
+ * within about one unit in the last place of itself instead of mapping to itself bit for bit
+ * (the MRT form, lbm_sw_set_relaxation, relaxes f^eq - f and keeps that fixed point).  In
+ * FP64 the sums and the products with the rates are done on 64-bit integers, 59 bits below a
+ * family's largest population, wherever the sizes of its values allow it.
  *
  * Every compute step runs in hand-written CUDA kernels on the caller's stream;
  * there is no CPU fallback.  No function throws; every function that can fail
  * returns a status code (LBM_SW_OK = 0 or a negative LBM_SW_E_*), and the handle
  * keeps a message for the last failure (lbm_sw_last_error).  Many handles may
- * coexist; the library keeps no global state.
+ * coexist; the library keeps no global state but the count of the bytes that handles hold
+ * for their next tape.
  *
  * Layouts at this boundary
  *   - Moment fields (h, hu, hv) are FP64 arrays of nx*ny values, row-major
@@ -109,10 +112,11 @@ typedef struct lbm_sw lbm_sw;
                                    (628^2 and up) with every side periodic or an even
                                    temporal_steps (with MRT relaxation: >= 2^19 cells), else VEC in
                                    2D; CLUSTER in 1D.  FP32 grids below 5 * 2^17 cells with
-                                   temporal_steps = 0 take 4 to 8 steps per launch on tiles held
-                                   in registers, with the same results */
+                                   temporal_steps = 0 take up to 8 steps per launch on tiles held
+                                   in registers (where TEMPORAL applies too, if two waves of
+                                   tiles cover the grid), with the same results */
 #define LBM_SW_KERNEL_SIMPLE 1  /* one launch per step, one thread per cell, scalar loads */
-#define LBM_SW_KERNEL_VEC 2     /* 2D: 16-byte vectors along x (4 FP32 or 2 FP64 cells per thread),
+#define LBM_SW_KERNEL_VEC 2     /* 2D: 16-byte vectors along x (4 FP32 cells per thread; FP64 one),
                                    x-neighbours exchanged with warp shuffles */
 #define LBM_SW_KERNEL_CLUSTER 3 /* 1D: all n steps of lbm_sw_step in one cooperative launch, the
                                    line held in the registers of warps that exchange their
@@ -375,7 +379,8 @@ LBM_SW_API const char* lbm_sw_batch_last_error(const lbm_sw_batch* b);
  * where S is the streaming with the boundary rules (its transpose pulls in the reverse
  * direction), M sums each family, D = df^eq/dW (the equilibria of section 3) and
  * J_C = (1 - s) I + s D M is the Jacobian of the BGK collision (Eq. 2-relaxation).  A tape
- * stores the state every `interval` steps (about sqrt(T) by default) in FP64; the backward
+ * keeps the moments W^n of every step where they take at most 4 GB, and replays nothing;
+ * else it stores the state every `interval` steps (about sqrt(T) by default) in FP64; the backward
  * pass replays each segment from its checkpoint (bit for bit: widening FP32 to FP64 is
  * exact), keeping only the moments W^n (3 planes per step), then runs the adjoint steps.
  * Phi and the replay use the handle's precision.  The tape owns all of its memory; the
