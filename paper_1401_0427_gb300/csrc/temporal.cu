@@ -332,30 +332,31 @@ __global__ void __launch_bounds__(COLS, COLS == 192 ? 2 : (K <= 4 ? 5 : 3))
 }
 
 // The paired wavefront with the boundary rules of any sides (even nx; odd nx with ODD).
-template <int K, int COLS, int PF, bool STORE_W = false, bool L0R = false>
+template <int K, int COLS, int PF, bool STORE_W = false, bool L0R = false, bool ODD = false>
 __global__ void __launch_bounds__(COLS / 2, 2)
     step2d_temporal_x2(const StepArgs<float> A, const Consts<float> Kc, const Partition P,
                        float* __restrict__ wout = nullptr, long long wslot = 0) {
   extern __shared__ __align__(16) float smem[];
   pdl_wait();
   run_segment(P, A.ny, [&](int strip, int ys, int ye) {
-    pair_wave<K, COLS, PF, STORE_W, L0R, false, false, STORE_W>(A, Kc, smem, strip * P.w, P.w, ys, ye, wout, wslot);
+    pair_wave<K, COLS, PF, STORE_W, L0R, false, false, ODD>(A, Kc, smem, strip * P.w, P.w, ys, ye, wout, wslot);
   });
   pdl_done();
 }
 
-// Every side periodic.  The plain kernel runs even widths; the one that also stores the
-// moments of every level (the adjoint's replays) and the _odd kernels any width.  The
+// Every side periodic.  The plain kernel runs even widths, the one that also stores the
+// moments of every level (the adjoint's records and replays) any with ODD (even widths without it: a
+// 1024^2 gradient 3.83 -> 3.75 ms; a batch whose CTAs choose per instance: 15.9 -> 17.6, so it does not).  The
 // branch-free steady state: the 6-step 256-column plain kernel and every replay kernel
 // (-1 % per gradient at 1024^2).
-template <int K, int COLS, int PF, bool STORE_W = false, bool L0R = false>
+template <int K, int COLS, int PF, bool STORE_W = false, bool L0R = false, bool ODD = false>
 __global__ void __launch_bounds__(COLS / 2, 2)
     step2d_temporal_periodic_x2(const StepArgs<float> A, const Consts<float> Kc, const Partition P,
                                 float* __restrict__ wout = nullptr, long long wslot = 0) {
   extern __shared__ __align__(16) float smem[];
   pdl_wait();
   run_segment(P, A.ny, [&](int strip, int ys, int ye) {
-    pair_wave<K, COLS, PF, STORE_W, L0R, true, false, STORE_W, !STORE_W && K <= 6,
+    pair_wave<K, COLS, PF, STORE_W, L0R, true, false, ODD, !STORE_W && K <= 6,
               STORE_W || (K == 6 && COLS == 256)>(A, Kc, smem, strip * P.w, P.w, ys, ye, wout, wslot);
   });
   pdl_done();
@@ -482,18 +483,21 @@ cudaError_t launch_k_pairs_w(const StepArgs<float>& a, const ConstsD& kd, float*
   constexpr int PF = K <= 4 ? 2 : 1;
   constexpr bool L0R = K == 6;
   const size_t smem = PairShape<K, COLS, PF, L0R>::floats() * sizeof(float);
-  const void* fn = PER ? reinterpret_cast<const void*>(step2d_temporal_periodic_x2<K, COLS, PF, true, L0R>)
-                       : reinterpret_cast<const void*>(step2d_temporal_x2<K, COLS, PF, true, L0R>);
+  const auto kernel = [&] {
+    if constexpr (PER)
+      return a.nx & 1 ? step2d_temporal_periodic_x2<K, COLS, PF, true, L0R, true>
+                      : step2d_temporal_periodic_x2<K, COLS, PF, true, L0R, false>;
+    else
+      return a.nx & 1 ? step2d_temporal_x2<K, COLS, PF, true, L0R, true> : step2d_temporal_x2<K, COLS, PF, true, L0R, false>;
+  }();
+  const void* fn = reinterpret_cast<const void*>(kernel);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const int resident = cached_resident(fn, COLS / 2, smem);
   const Partition Q = pair_partition(a.nx, a.ny, K, COLS, resident * std::max(sm_count, 1));
   const Consts<float> K_ = make_consts<float>(kd.g, kd.lambda, kd.s, kd.a);
   const dim3 grid(Q.strips * Q.segments), block(COLS / 2);
-  if constexpr (PER)
-    return launch_pdl(step2d_temporal_periodic_x2<K, COLS, PF, true, L0R>, grid, block, smem, st, a, K_, Q, wout, wslot);
-  else
-    return launch_pdl(step2d_temporal_x2<K, COLS, PF, true, L0R>, grid, block, smem, st, a, K_, Q, wout, wslot);
+  return launch_pdl(kernel, grid, block, smem, st, a, K_, Q, wout, wslot);
 }
 
 template <int K>
