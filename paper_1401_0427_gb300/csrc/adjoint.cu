@@ -345,7 +345,9 @@ void* TapeMemory::take(size_t need, size_t* got) {
   }
   void* m = nullptr;
   *got = need;
-  return cudaMalloc(&m, need) == cudaSuccess ? m : nullptr;
+  if (cudaMalloc(&m, need) == cudaSuccess) return m;
+  cudaGetLastError();  // the caller may go on with less: the next launch's check must not see this failure
+  return nullptr;
 }
 
 bool TapeMemory::give(void* m, size_t size) {
@@ -650,7 +652,8 @@ int lbm_sw_tape_create(lbm_sw* h, int steps, int interval, lbm_sw_tape** out) {
     for (void* b : {t->phi[0], t->phi[1], t->rep[0], t->rep[1]})
       if (ok && b) ok = cudaMemsetAsync(b, 0, state, h->stream) == cudaSuccess;
   if (!ok) {
-    h->err = std::string("tape_create: device allocation failed: ") + cudaGetErrorString(cudaGetLastError());
+    const char* why = cudaGetErrorString(t->mem ? cudaGetLastError() : cudaErrorMemoryAllocation);
+    h->err = std::string("tape_create: device allocation failed: ") + why;
     lbm_sw_tape_destroy(t);
     return LBM_SW_E_NOMEM;
   }

@@ -1,0 +1,94 @@
+"""A tape whose memory for the moments of every step is not there falls back to checkpoints.
+
+The library's objects are linked here once more with cudaMalloc wrapped: requests above a limit go to
+the real cudaMalloc as a request of 2^60 bytes, which fails and leaves the runtime's last error as an
+exhausted device would, without using memory.  A child process loads that library."""
+
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+from paper_1401_0427_gb300 import build as libbuild
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+HOOK = r"""
+#include <cuda_runtime.h>
+extern "C" cudaError_t __real_cudaMalloc(void**, size_t);
+static size_t limit = ~size_t(0);
+static int refused = 0;
+extern "C" __attribute__((visibility("default"))) int refuse_above(size_t bytes) {
+  limit = bytes;
+  return refused;
+}
+extern "C" cudaError_t __wrap_cudaMalloc(void** p, size_t n) {
+  if (n <= limit) return __real_cudaMalloc(p, n);
+  ++refused;
+  return __real_cudaMalloc(p, size_t(1) << 60);
+}
+"""
+
+PRELUDE = r"""
+import ctypes, json, sys
+import numpy as np
+import torch
+from paper_1401_0427_gb300 import inputs, lbm_sw
+lib = lbm_sw.load(sys.argv[1])
+lib.refuse_above.argtypes, lib.refuse_above.restype = [ctypes.c_size_t], ctypes.c_int
+NEVER = 2 ** 64 - 1
+torch.zeros(1, device="cuda")
+"""
+
+
+@pytest.fixture(scope="module")
+def library(tmp_path_factory):
+    libbuild.build()
+    objs = [os.path.join(libbuild.BUILD, os.path.basename(s)[:-3] + ".o") for s in libbuild.sources()]
+    d = tmp_path_factory.mktemp("refusing")
+    src, so = d / "hook.cu", str(d / "liblbm_sw_refusing.so")
+    src.write_text(HOOK)
+    r = subprocess.run([libbuild.nvcc(), *libbuild.ARCH, "-Xcompiler", "-fPIC", "-shared", "-cudart", "static", "-o", so,
+                        str(src), *objs, "-Xlinker", "--wrap=cudaMalloc"], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return so
+
+
+def _run(library, script):
+    r = subprocess.run([sys.executable, "-c", PRELUDE + script, library], capture_output=True, text=True, cwd=ROOT,
+                       env={**os.environ, "PYTHONPATH": ROOT}, timeout=300)
+    assert r.returncode == 0, r.stderr
+    return json.loads(r.stdout.splitlines()[-1])
+
+
+@pytest.mark.parametrize("precision", ["FP32", "FP64"])
+def test_without_memory_for_the_moments_the_tape_takes_checkpoints(library, precision):
+    """The record and the gradient after a refused allocation of the moments of 200 steps; the
+    gradient agrees with that of a tape that keeps them as gradients of other launch splits do."""
+    out = _run(library, r"""
+prec = lbm_sw.%s
+nx, ny, steps = 96, 64, 200
+W0 = [x.reshape(ny, nx) for x in inputs.random_states(nx * ny, seed=7, h=(0.95, 1.05), speed=0.02)]
+with lbm_sw.Simulation(nx, ny, precision=prec, stream=torch.cuda.current_stream().cuda_stream) as sim:
+    plane = sim.info().pitch * ny
+    all_steps = 3 * (steps + 1) * plane * np.dtype(sim.dtype).itemsize
+    grads, kept = [], []
+    for limit in (NEVER, all_steps):
+        before = lib.refuse_above(limit)
+        sim.set_state(*W0)
+        with lbm_sw.Tape(sim, steps) as tape:
+            tape.record()
+            grads.append(tape.adjoint(sim.moments()[0] - 1.0))
+            kept.append(tape.info().replay_bytes >= all_steps)
+        refused = lib.refuse_above(NEVER) - before
+        # the kept memory of the first tape would serve the second
+        sim.close()
+        sim.__init__(nx, ny, precision=prec, stream=torch.cuda.current_stream().cuda_stream)
+print(json.dumps({"kept": kept, "refused": refused, "off": float(np.abs(grads[0] - grads[1]).max() / np.abs(grads[0]).max())}))
+""" % precision)
+    assert out["kept"] == [True, False] and out["refused"] == 1
+    assert out["off"] <= (1e-5 if precision == "FP32" else 1e-12)
