@@ -739,11 +739,9 @@ def shock_reflection_variant(stream, lbm_sw, torch, steps: int = 2000):
 
 def adjoint_variant(stream, lbm_sw, torch, steps: int = 200):
     """Inverse-problem workload: 1024 x 1024 periodic, 8 Gaussian bumps on depth 1, T = 200,
-    FP32 states with FP64 checkpoints every ceil(sqrt(T)) steps.  One gradient = recorded
-    forward run + adjoint (segment replays + adjoint steps), against 2T plain steps.  Also
-    timed: the other end of the tape's memory / time trade-off, one checkpoint interval of
-    T steps, where the recorded forward run keeps the moments of every step (T + K slots of
-    3 planes) and the backward pass replays nothing."""
+    FP32 states; the recorded forward run keeps the moments of every step (2.5 GB) and the
+    backward pass replays nothing.  One gradient = recorded forward run + adjoint, against 2T
+    plain steps.  Also timed: one interval of T steps, asked for by name."""
     from paper_1401_0427_gb300 import inputs
 
     n = 1024

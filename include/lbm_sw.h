@@ -379,9 +379,9 @@ LBM_SW_API const char* lbm_sw_batch_last_error(const lbm_sw_batch* b);
  * where S is the streaming with the boundary rules (its transpose pulls in the reverse
  * direction), M sums each family, D = df^eq/dW (the equilibria of section 3) and
  * J_C = (1 - s) I + s D M is the Jacobian of the BGK collision (Eq. 2-relaxation).  A tape
- * keeps the moments W^n of every step where they take at most 4 GB, and replays nothing;
- * else it stores the state every `interval` steps (about sqrt(T) by default) in FP64; the backward
- * pass replays each segment from its checkpoint (bit for bit: widening FP32 to FP64 is
+ * with the library's interval (0), or one of T steps, keeps the moments W^n of every step where
+ * they take at most 4 GB and there is memory for them, and replays nothing; else it stores the
+ * state every `interval` steps (about sqrt(T) by default) in FP64; the backward pass replays each segment from its checkpoint (bit for bit: widening FP32 to FP64 is
  * exact), keeping only the moments W^n (3 planes per step), then runs the adjoint steps.
  * Phi and the replay use the handle's precision.  The tape owns all of its memory; the
  * handle's own state is not touched by lbm_sw_adjoint. */
@@ -392,14 +392,15 @@ typedef struct lbm_sw_tape_info {
   int interval;            /* steps between checkpoints */
   int checkpoints;         /* ceil(T / interval) */
   int recorded;            /* 1 after lbm_sw_forward_record */
-  size_t checkpoint_bytes; /* FP64 checkpoints at this interval (none are stored while the moments
-                              of every step take at most 4 GB: those are kept instead) */
+  size_t checkpoint_bytes; /* FP64 checkpoints at this interval (none are stored by a tape that keeps
+                              the moments of every step instead; replay_bytes then is all it holds) */
   size_t replay_bytes;     /* moments of one segment or of every step, adjoint, replay and staging
                               buffers */
 } lbm_sw_tape_info;
 
 /* Tape for `steps` >= 1 steps of 2D handle h, checkpoints every `interval` steps
- * (0 = ceil(sqrt(steps))).  Errors: LBM_SW_E_ARG (1D handle, bad counts), LBM_SW_E_NOMEM. */
+ * (0 = ceil(sqrt(steps)), or none where the moments of every step are kept).  An interval below
+ * `steps` bounds the tape's memory: its checkpoints and the moments of one segment.  Errors: LBM_SW_E_ARG (1D handle, bad counts), LBM_SW_E_NOMEM. */
 LBM_SW_API int lbm_sw_tape_create(lbm_sw* h, int steps, int interval, lbm_sw_tape** out);
 
 /* Release a tape.  Its device memory is kept for the handle's next tape (one block per handle, 8 GB

@@ -1,6 +1,8 @@
 """Gradients of the 2D scheme through time for PyTorch: a torch.autograd.Function whose
 forward runs T fused steps from an equilibrium start at rest, f = f^eq(h0, 0, 0), and
-whose backward runs the discrete adjoint with sqrt(T) checkpointing (lbm_sw_adjoint).
+whose backward runs the discrete adjoint (lbm_sw_adjoint) on the moments of every step,
+kept by the forward run where they take at most 4 GB, else replayed from about sqrt(T)
+checkpoints; an `interval` of the caller's below `steps` asks for checkpoints.
 
 Only device memory and streams come from PyTorch; every step, replay and adjoint
 step runs in the CUDA library.
@@ -18,9 +20,9 @@ class ShallowWaterRun(torch.autograd.Function):
 
     The forward pass runs on the caller's Simulation: it overwrites that handle's state
     (set_state(h0, 0, 0), then `steps` steps), so afterwards `sim` holds the state at step T.
-    Its checkpoint tape owns its own device memory and is released when the autograd graph
-    that holds it is freed, so backward may run more than once (retain_graph=True); each
-    backward replays the tape's checkpoints and leaves the handle's state alone."""
+    Its tape owns its own device memory and is released when the autograd graph that holds it
+    is freed, so backward may run more than once (retain_graph=True); each backward reads the
+    tape (replaying its checkpoints, if it has them) and leaves the handle's state alone."""
 
     @staticmethod
     def forward(ctx, h0: torch.Tensor, sim: lbm_sw.Simulation, steps: int, interval: int = 0):

@@ -624,14 +624,16 @@ int lbm_sw_tape_create(lbm_sw* h, int steps, int interval, lbm_sw_tape** out) {
   t->state_elems = static_cast<size_t>(13) * h->plane;
   const size_t n = static_cast<size_t>(h->p.nx) * h->p.ny;
   const size_t slot = static_cast<size_t>(h->elem) * 3 * h->plane, state = static_cast<size_t>(h->elem) * t->state_elems;
-  // The moments of every step where they take little memory: the record then writes them as it
-  // goes, and the backward pass replays nothing (1024^2 FP32, 200 steps, 2.5 GB: record and adjoint
-  // 1.5 + 3.8 ms with checkpoints every 24 steps, 1.6 + 2.0 ms this way).
-  // Without room for them: checkpoints.
+  // The moments of every step where they take little memory and the caller leaves the interval to
+  // the library or asks for one of all steps: the record then writes them as it goes, and the
+  // backward pass replays nothing (1024^2 FP32, 200 steps, 2.5 GB: record and adjoint 1.5 + 3.8 ms
+  // with checkpoints every 24 steps, 1.6 + 2.0 ms this way).  A smaller interval of the caller's
+  // bounds the tape's memory.  Without room for the moments: checkpoints.
   void** const parts[7] = {reinterpret_cast<void**>(&t->ckpt), &t->wstore, reinterpret_cast<void**>(&t->grad_staging),
                            &t->phi[0], &t->phi[1], &t->rep[0], &t->rep[1]};
   bool ok = false;
-  for (int all = (static_cast<size_t>(steps) + 1) * slot <= kTapeMomentsMost; !ok && all >= 0; --all) {
+  const bool may_keep = (interval == 0 || interval == steps) && (static_cast<size_t>(steps) + 1) * slot <= kTapeMomentsMost;
+  for (int all = may_keep; !ok && all >= 0; --all) {
     t->keep_all = all == 1;
     // a replay that fuses k steps per launch may run up to k - 1 steps past its segment
     t->wslots = t->keep_all ? steps + 1 : t->interval + replay_k(h);

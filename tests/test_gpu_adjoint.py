@@ -375,3 +375,36 @@ def test_small_grids_record_and_reverse_on_register_tiles(nx, ny, steps, bc):
         assert np.array_equal(a, b)
     for a, b in zip(*grads):
         assert np.abs(a - b).max() <= 1e-5 * max(np.abs(a).max(), 1e-30)
+
+
+@pytest.mark.parametrize("precision", [lbm_sw.FP32, lbm_sw.FP64])
+@pytest.mark.parametrize("kernel,k", [(lbm_sw.KERNEL_AUTO, 0), (lbm_sw.KERNEL_TEMPORAL, 6), (lbm_sw.KERNEL_VEC, 0)],
+                         ids=["auto", "temporal6", "vec"])
+@pytest.mark.parametrize("interval", [7, 12])
+def test_an_interval_bounds_the_memory_and_replays(interval, kernel, k, precision):
+    """A tape with an interval below T holds its checkpoints and the moments of one segment (with a
+    fused launch's overshoot), fewer than those of every step; its replayed gradient, the first
+    and the second time, is that of a tape that keeps every step's moments (T = 61: the last segment
+    is short).  Bounds as for other launch splits."""
+    if precision == lbm_sw.FP64 and kernel == lbm_sw.KERNEL_TEMPORAL:
+        pytest.skip("the wavefront is FP32")
+    nx, ny, steps = 130, 33, 61
+    W0 = [x.reshape(ny, nx) for x in inputs.random_states(nx * ny, seed=560, h=(0.8, 1.4), speed=0.25)]
+    out = []
+    with lbm_sw.Simulation(nx, ny, precision=precision, kernel=kernel, temporal_steps=k, stream=torch_stream()) as sim:
+        slot = 3 * sim.info().pitch * ny * np.dtype(sim.dtype).itemsize
+        for iv in (0, interval):
+            sim.set_state(*W0)
+            with lbm_sw.Tape(sim, steps, iv) as tape:
+                tape.record()
+                hT = sim.moments()[0]
+                g = [tape.adjoint(hT - 1.0, want_momentum=True) for _ in range(2)]
+                moments = tape.info().replay_bytes - (4 * 13 * slot // 3 if iv else 2 * 13 * slot // 3)
+                assert (moments < (interval + 8 + 2 * 3) * slot) if iv else (moments >= (steps + 1) * slot)
+                out.append((hT, g))
+    (h_a, g_a), (h_b, g_b) = out
+    assert np.array_equal(h_a, h_b)
+    tol = 1e-5 if precision == lbm_sw.FP32 else 1e-12
+    for first, second, ref in zip(*g_b, g_a[0]):
+        assert np.array_equal(first, second)
+        assert np.abs(first - ref).max() <= tol * np.abs(ref).max()
