@@ -233,6 +233,8 @@ __device__ __forceinline__ unsigned long long times_2_64(unsigned long long m, u
 __device__ __forceinline__ unsigned long long times_2_64_round(unsigned long long m, unsigned long long c) {
   return __umul64hi(m, c) + (m * c >> 63);
 }
+// v / 4, rounded to nearest even
+__device__ __forceinline__ long long quarter(long long v) { return (v + 1 + (static_cast<unsigned>(v) >> 2 & 1)) >> 2; }
 // the double of v (|v| < 2^63) in units of e's, rounded to nearest even
 __device__ __forceinline__ double unfix(long long v, int e) {
   const int s = static_cast<int>(v >> 63);
@@ -372,15 +374,26 @@ __device__ __forceinline__ void collide13_fma(double f[13], const Consts<double>
   f[12] = fmad(om, f[12], fmad(-hc, ty, y4));
 }
 
-// FP64, the usual case: the sums, s c q, s q / 4 and the relaxation of the twelve moving
-// populations in integers (above), each population rounded once: 19 operations of the FP64 unit.
+// FP64, the usual case: the sums, s c q and the relaxation of the twelve moving populations in
+// integers (above), each population rounded once: 18 operations of the FP64 unit.  The parts that
+// the four populations of an equilibrium share, s (h - f0^eq) / 4 and s q / 4, are a quarter of what the relaxed
+// populations leave of the integer sum (rounded to even), so the sums of depths and momenta
+// keep their values but for the last rounding of each population, whatever the products lose.
 // False, and nothing changed, where the values of a family differ too much in size (an equilibrium
 // term more than twice the power of two of the largest population, as at the front of a
 // jump; exponents near the ends of the range): collide13_fma takes the cell then.
+// Bounds: the depths' units are 2^-59 of the power of two above their largest population, the
+// momenta's of the one below, so populations are below 1/2 and 1 of 2^60 units and the remainders of
+// the sums below 13/2 and 8; s c q is below 4; a relaxed population is below 25/4 (the
+// integers' range is 8).
 //
 // 1536^2 cells, us per step: 278 with 59 operations in the FP64 unit, 218 with 52, 197 with the
-// moments in integers, 140 this way.  Error against quadruple precision after 300
-// steps of a dam break on 40^2 cells: h 1.2e-15 and q 9e-15 with 59 operations, 3e-16 and 3e-15.
+// moments in integers, 144 this way (141 with s h / 4 and s q / 4 as truncated products, which lean one
+// way; 158 with rounded ones).  Relative drift of the depths' sum of a dam break on 56^2
+// cells after 20,000 steps, s = 1.8, 1.95 and 1.99: 8e-14, 1.8e-14 and 4e-15 with 59 operations, 5e-14,
+// 3.3e-14 and 3.1e-14 with truncated products, at most 3e-16 this way.  Error against quadruple precision after
+// 200 steps on 40^2 cells at s = 1.8: h 7.5e-16 and q 3.3e-15 with 59 operations, 1.1e-16 and 3.3e-16 (rates from
+// 0.5 to 1.99, at rest, in a flow and in waves of 1e-2: 0.1 to 0.85 of the former error).
 __device__ __forceinline__ bool collide13_fixed(double f[13], const Consts<double>& k, double& h, double& qx, double& qy) {
   int ef = exp_field(f[0]), ex = 0, ey = 0;
 #pragma unroll
@@ -389,6 +402,7 @@ __device__ __forceinline__ bool collide13_fixed(double f[13], const Consts<doubl
     ex = max(ex, exp_field(f[4 + i]));
     ey = max(ey, exp_field(f[8 + i]));
   }
+  ef += 1 << 20;  // of the power of two above: the remainder of the sum, up to s h, has to fit
   if (!(k.fixed_ok && exp_fits(ef) && exp_fits(ex) && exp_fits(ey))) return false;
   unsigned long long m[13];
   long long v[3] = {0, 0, 0};
@@ -404,7 +418,6 @@ __device__ __forceinline__ bool collide13_fixed(double f[13], const Consts<doubl
   const double u = mul(qx, rh), w = mul(qy, rh);
   const double uu = mul(u, u), ww = mul(w, w), uw = mul(u, w);
   const double z = fmad(add(uu, ww), k.s_a4g, mul(k.s_a2, h));  // -s f0^eq / 4
-  const double r = fmad(h, k.s_4, z);                           // s (h - f0^eq) / 4
   const double hc = mul(h, k.s_c);
   const double pxx = mul(hc, fmad(k.half_g, h, uu)), pyy = mul(hc, fmad(k.half_g, h, ww)), pxy = mul(hc, uw);
   bool ok = true;
@@ -414,18 +427,24 @@ __device__ __forceinline__ bool collide13_fixed(double f[13], const Consts<doubl
   // s c q, in units of the f family's
   const long long cx = with_sign(to_units(times_2_64(ax, k.x_sc), (ef - ex) >> 20, k.least_sc, ok), sx);
   const long long cy = with_sign(to_units(times_2_64(ay, k.x_sc), (ef - ey) >> 20, k.least_sc, ok), sy);
-  const long long x4 = with_sign(times_2_64(ax, k.x_s4), sx), y4 = with_sign(times_2_64(ay, k.x_s4), sy);
-  const long long fr = fix_one_more(r, ef, ok);
+  const double f0 = fmad(k.om, f[0], times_pow2<2, true>(z));  // relaxed
+  const long long F0 = fix_one_more(f0, ef, ok);
   const long long fxx = fix_one_more(pxx, ex, ok), fxy = fix_one_more(pxy, ex, ok);
   const long long fyx = fix_one_more(pxy, ey, ok), fyy = fix_one_more(pyy, ey, ok);
   if (!ok) return false;
-  f[0] = fmad(k.om, f[0], times_pow2<2, true>(z));
   const int flip = k.om_neg ? static_cast<int>(0x80000000u) : 0;
+  long long t[13], rest[3] = {v[0] - F0, v[1], v[2]};
+#pragma unroll
+  for (int i = 1; i < 13; ++i) {
+    t[i] = with_sign(times_2_64(m[i], k.x_om), __double2hiint(f[i]) ^ flip);
+    rest[i < 5 ? 0 : (i < 9 ? 1 : 2)] -= t[i];
+  }
+  const long long fr = quarter(rest[0]), x4 = quarter(rest[1]), y4 = quarter(rest[2]);
   const long long eq[13] = {0,        fr + cx,  fr + cy,  fr - cx,  fr - cy,  x4 + fxx, x4 + fxy,
                             x4 - fxx, x4 - fxy, y4 + fyx, y4 + fyy, y4 - fyx, y4 - fyy};
+  f[0] = f0;
 #pragma unroll
-  for (int i = 1; i < 13; ++i)
-    f[i] = unfix(with_sign(times_2_64(m[i], k.x_om), __double2hiint(f[i]) ^ flip) + eq[i], i < 5 ? ef : (i < 9 ? ex : ey));
+  for (int i = 1; i < 13; ++i) f[i] = unfix(t[i] + eq[i], i < 5 ? ef : (i < 9 ? ex : ey));
   return true;
 }
 
@@ -504,7 +523,7 @@ __device__ __forceinline__ void collide13_mrt(T f[13], const Consts<T>& k, T& h,
 // population below 8 (the integers' range).
 //
 // us per step, before and after: 480 x 120 19.7 and 6.3, 512^2 63.7 and 20.2, 1536^2 539 and 153 (BGK
-// 141).  Error against extended precision after 300 steps of a dam break on 40^2 cells: h 8.8e-17 and
+// 144).  Error against extended precision after 300 steps of a dam break on 40^2 cells: h 8.8e-17 and
 // 5.8e-17 (relative L1), q 4.2e-15 and 2.3e-15; no drift of the depths' sum over 10^5 steps in either.
 __device__ __forceinline__ bool collide13_mrt_fixed(double f[13], const Consts<double>& k, double& h, double& qx,
                                                     double& qy) {

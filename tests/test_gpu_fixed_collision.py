@@ -1,6 +1,8 @@
 """The FP64 collisions in 64-bit integers and its way out to fused multiply-adds: against the oracle
 where the populations of a family differ much in size, and where they are zero, tiny or huge."""
 
+import math
+
 import numpy as np
 import pytest
 
@@ -98,3 +100,22 @@ def test_momenta_far_above_the_depths(dim, rates, lam):
     p = oracle.params(nx, ny, a=a, lam=lam, bc=bc, inflow=None, s_moments=rates)
     got = gpu_post(F0, 0, dim=dim, precision=lbm_sw.FP64, bc=bc, inflow=None, a=a, lam=lam, mrt_rates=rates)
     assert rel_max(got, oracle_post(F0, 0, p, dim)) <= FP64_TOL
+
+
+@pytest.mark.parametrize("u", [0.0, 0.2])
+@pytest.mark.parametrize("s", [1.0, 1.8, 1.95, 1.99])
+def test_depths_and_momenta_do_not_drift(s, u):
+    """The sums of depths and momenta over 20,000 periodic steps.  Each population is rounded to nearest
+    once per step; unbiased roundings of half an ulp, 2^-54 of the depth, walk by about
+    2^-54 sqrt(20000 / 56^2) = 1.4e-16 of the sum.  The bar is seven times that."""
+    n = 56
+    y, x = np.mgrid[0:n, 0:n]
+    h = np.where(np.hypot(x - n / 2, y - n / 2) < 0.2 * n, 2.0, 1.0) + 1e-3 * inputs.uniform(9740, n * n).reshape(n, n)
+    with lbm_sw.Simulation(n, n, precision=lbm_sw.FP64, s=s) as sim:
+        sim.set_state(h, u * h, np.zeros_like(h))
+        before = sim.populations()
+        sim.step(20000)
+        after = sim.populations()
+    total = [[math.fsum(F[a:b].ravel()) for a, b in ((0, 5), (5, 9), (9, 13))] for F in (before, after)]
+    for k in range(3):
+        assert abs(total[1][k] - total[0][k]) <= 1e-15 * total[0][0], (k, total)
