@@ -15,13 +15,13 @@
  * 2-potentiels-st-venant-1d-suite, 3-st-venant-contraintes-2, 3-st-venant-enplus),
  * with p = g h^2 / 2 (the gamma = 2 system), and the collision is the BGK form of
  * Eq. 2-relaxation (every rate equal to s).  Streaming moves each population one
- * cell per step (lambda = dx/dt).  The BGK kernels evaluate f + s (f^eq - f) as
- * (1 - s) f + s f^eq with s folded into the equilibrium's constants (2D, and 1D in FP64):
- * the same operator, with 13 operations fewer per 2D cell; a state at equilibrium settles
- * within about one unit in the last place of itself instead of mapping to itself bit for bit
- * (the MRT form, lbm_sw_set_relaxation, relaxes f^eq - f and keeps that fixed point).  In
- * FP64 the sums and the products with the rates are done on 64-bit integers, 59 bits below a
- * family's largest population, wherever the sizes of its values allow it.
+ * cell per step (lambda = dx/dt).  The 2D BGK kernels evaluate f + s (f^eq - f) as
+ * (1 - s) f + s f^eq with s folded into the equilibrium's constants: the same
+ * operator, with 13 operations fewer per cell; a state at equilibrium settles within
+ * about one unit in the last place of itself instead of mapping to itself bit for bit
+ * (1D, and the MRT form, lbm_sw_set_relaxation, relax f^eq - f and keep that fixed point).  In
+ * FP64 the sums and the products with the rates are done on 64-bit integers, about 59 bits below
+ * a family's largest population, wherever the sizes of its values allow it.
  *
  * Every compute step runs in hand-written CUDA kernels on the caller's stream;
  * there is no CPU fallback.  No function throws; every function that can fail

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256) step1d(const StepArgs<T> A, const Consts<
 // line is spread over as many quarters as it fills.  With the former collision (32 FP64 operations)
 // 1000 cells took 1.23 us per step in FP64, against 1.44 with one cluster of 16 SMs (windows of
 // 63 + 16 cells in shared memory, a cluster barrier per 8 steps), 16000 cells 1.66 against 9.82;
-// with the one in integers 0.98 and 1.25.  FP32: 0.16 against 0.39 and 0.17 against 0.69.
+// with the one in integers 0.92 and 1.13.  FP32: 0.16 against 0.39 and 0.17 against 0.69.
 //
 // Exchange: a mailbox in global memory with two slots per cell, used by turns.  Each 8-byte
 // word carries 4 bytes of payload and the number of the exchange, written and read as one

@@ -119,3 +119,18 @@ def test_depths_and_momenta_do_not_drift(s, u):
     total = [[math.fsum(F[a:b].ravel()) for a, b in ((0, 5), (5, 9), (9, 13))] for F in (before, after)]
     for k in range(3):
         assert abs(total[1][k] - total[0][k]) <= 1e-15 * total[0][0], (k, total)
+
+
+def test_1d_lakes_at_rest_keep_their_bits():
+    """A uniform depth at rest between walls whose populations add up to it (rounded once) is a
+    fixed point of f + s (f^eq - f): no bit changes in 1,000 steps."""
+    kept = 0
+    for h in inputs.uniform(9750, 150, 0.5, 3.0):
+        with lbm_sw.Simulation(8, 1, dim=1, precision=lbm_sw.FP64, bc=(W, W), a=0.15) as sim:
+            sim.set_state(np.full(8, h), np.zeros(8))
+            F = sim.populations()
+            sim.step(1000)
+            if math.fsum(F.reshape(5, 8)[:3, 0]) == h:
+                kept += 1
+                assert np.array_equal(sim.populations(), F), h
+    assert kept >= 140
