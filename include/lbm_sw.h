@@ -75,7 +75,8 @@ typedef struct lbm_sw lbm_sw;
 #define LBM_SW_E_CUDA (-2)     /* a CUDA call failed; see lbm_sw_last_error */
 #define LBM_SW_E_UNSTABLE (-3) /* a diagnostic found NaN/Inf or a depth h <= 0 */
 /* (-4 is not used: no kernel of this library waits on another grid; the warps of one 1D launch
- * wait for one another with a bound, and store NaN if it runs out) */
+ * wait for one another with a bound, and where it runs out every cell that depends on what did not
+ * come is NaN, which diagnostics report) */
 #define LBM_SW_E_STATE (-5)    /* call not valid in the handle's state (e.g. no state set) */
 #define LBM_SW_E_NOMEM (-6)    /* device allocation failed */
 

@@ -67,8 +67,10 @@ __global__ void __launch_bounds__(256) step1d(const StepArgs<T> A, const Consts<
 // access, so a reader that sees the number has the payload: one trip through L2 and no fence.  A
 // slot is written again two exchanges later, when its writer has read the exchange between from
 // the same neighbours, who had read the slot before they published that one.  The launch is
-// cooperative, so every warp is resident; a wait gives up after kWaitPolls polls all the same,
-// and the results of that launch are then stored as NaN, which diagnostics report.
+// cooperative, so every warp is resident; a wait gives up after `wait_polls` polls all the same.  A
+// warp that gave up holds NaN from there on, and publishes it, and waits for nothing any more (a
+// neighbour that misses an exchange for that gives up too): every cell that depends on what never
+// came is stored as NaN, which diagnostics report, and every other cell is right.
 constexpr int kWaitPolls = 1 << 22;
 constexpr unsigned kAllLanes = 0xffffffffu;
 
@@ -110,7 +112,7 @@ __device__ __forceinline__ bool mail_get(const unsigned long long* w, double& v,
 
 template <class T, bool MRT>
 __global__ void __launch_bounds__(32) step1d_windows(const StepArgs<T> A, const Consts<T> K, int nsteps, int B,
-                                                     unsigned long long* __restrict__ mail) {
+                                                     int wait_polls, unsigned long long* __restrict__ mail) {
   constexpr int MW = MailWords<T>::n;
   const int nx = A.nx;
   const int out = 32 - 2 * B;                   // cells of a piece
@@ -184,17 +186,20 @@ __global__ void __launch_bounds__(32) step1d_windows(const StepArgs<T> A, const 
 #pragma unroll
         for (int p = 0; p < 5; ++p) ok &= mail_get(w + p * MW, f[p], epoch);
         if (ok) break;
-        if (failed || polls >= kWaitPolls) {  // one exhausted wait ends the later ones at once
+        if (failed || polls >= wait_polls) {  // one exhausted wait ends the later ones at once
           failed = true;
           break;
         }
       }
     }
     failed = __any_sync(kAllLanes, failed);
+    if (failed)
+#pragma unroll
+      for (int p = 0; p < 5; ++p) f[p] = T(NAN);
   }
   if (own)
 #pragma unroll
-    for (int p = 0; p < 5; ++p) A.dst[p * A.plane + g] = failed ? T(NAN) : f[p];
+    for (int p = 0; p < 5; ++p) A.dst[p * A.plane + g] = f[p];
 }
 
 template <class T>
@@ -313,7 +318,7 @@ cudaError_t launch_step1d_windows(const StepArgs<T>& a, const ConstsD& kd, int n
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kd.mrt ? step1d_windows<T, true> : step1d_windows<T, false>, a, consts1<T>(kd),
-                            nsteps, b, static_cast<unsigned long long*>(mail));
+                            nsteps, b, kWaitPolls, static_cast<unsigned long long*>(mail));
 }
 
 template <class T>
