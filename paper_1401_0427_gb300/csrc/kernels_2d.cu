@@ -348,18 +348,32 @@ dim3 cell_grid(int nx, int ny, dim3 block) {
 
 }  // namespace
 
+// Whether a kernel may dereference p: memory of the current device, or managed memory.
+static bool kernel_reaches(const void* p) {
+  cudaPointerAttributes a{};
+  int device = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&device) != cudaSuccess) {
+    cudaGetLastError();  // the copy will say what is wrong with the pointer
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == device);
+}
+
 // One kernel for all planes (a 2D copy per plane costs a launch of 2 to 3 us each: the 13 planes of
 // a 64 x 64 state 33 us, against 3), in 16-byte words where every row of both sides starts on 16
-// bytes, else in 4- or 8-byte words; addresses that are not aligned to those by 2D copies.
+// bytes, else in 4- or 8-byte words.  By 2D copies: addresses that are not aligned to those, and memory that
+// is not this device's (a peer's, host memory), which the copies take or refuse.
 cudaError_t copy_planes(const PlaneCopy& c, size_t elem, cudaStream_t st) {
   auto aligned = [&](size_t a) {
     return reinterpret_cast<size_t>(c.src) % a == 0 && reinterpret_cast<size_t>(c.dst) % a == 0 && c.row_bytes % a == 0 &&
            c.src_pitch % a == 0 && c.dst_pitch % a == 0 && c.src_plane % a == 0 && c.dst_plane % a == 0;
   };
   if (c.rows < 1 || c.row_bytes < 1) return cudaSuccess;
-  if (aligned(16)) return copy_planes_as<uint4>(c, st);
-  if (elem == 8 && aligned(8)) return copy_planes_as<unsigned long long>(c, st);
-  if (elem == 4 && aligned(4)) return copy_planes_as<unsigned>(c, st);
+  if (kernel_reaches(c.src) && kernel_reaches(c.dst)) {
+    if (aligned(16)) return copy_planes_as<uint4>(c, st);
+    if (elem == 8 && aligned(8)) return copy_planes_as<unsigned long long>(c, st);
+    if (elem == 4 && aligned(4)) return copy_planes_as<unsigned>(c, st);
+  }
   for (int p = 0; p < c.planes; ++p) {
     const cudaError_t e = cudaMemcpy2DAsync(static_cast<char*>(c.dst) + p * c.dst_plane, c.dst_pitch,
                                             static_cast<const char*>(c.src) + p * c.src_plane, c.src_pitch, c.row_bytes,

@@ -1,21 +1,13 @@
 """A tape whose memory for the moments of every step is not there falls back to checkpoints.
 
-The library's objects are linked here once more with cudaMalloc wrapped: requests above a limit go to
-the real cudaMalloc as a request of 2^60 bytes, which fails and leaves the runtime's last error as an
-exhausted device would, without using memory.  A child process loads that library."""
-
-import json
-import os
-import subprocess
-import sys
+cudaMalloc is wrapped: requests above a limit go to the real cudaMalloc as a request of 2^60 bytes,
+which fails and leaves the runtime's last error as an exhausted device would, without using memory."""
 
 import pytest
 
-from paper_1401_0427_gb300 import build as libbuild
+import wrapped_library
 
 pytestmark = pytest.mark.gpu
-
-ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 HOOK = r"""
 #include <cuda_runtime.h>
@@ -33,43 +25,22 @@ extern "C" cudaError_t __wrap_cudaMalloc(void** p, size_t n) {
 }
 """
 
-PRELUDE = r"""
-import ctypes, json, sys
-import numpy as np
-import torch
-from paper_1401_0427_gb300 import inputs, lbm_sw
-lib = lbm_sw.load(sys.argv[1])
+LIMIT = """
 lib.refuse_above.argtypes, lib.refuse_above.restype = [ctypes.c_size_t], ctypes.c_int
 NEVER = 2 ** 64 - 1
-torch.zeros(1, device="cuda")
 """
 
 
 @pytest.fixture(scope="module")
 def library(tmp_path_factory):
-    libbuild.build()
-    objs = [os.path.join(libbuild.BUILD, os.path.basename(s)[:-3] + ".o") for s in libbuild.sources()]
-    d = tmp_path_factory.mktemp("refusing")
-    src, so = d / "hook.cu", str(d / "liblbm_sw_refusing.so")
-    src.write_text(HOOK)
-    r = subprocess.run([libbuild.nvcc(), *libbuild.ARCH, "-Xcompiler", "-fPIC", "-shared", "-cudart", "static", "-o", so,
-                        str(src), *objs, "-Xlinker", "--wrap=cudaMalloc"], capture_output=True, text=True)
-    assert r.returncode == 0, r.stderr
-    return so
-
-
-def _run(library, script):
-    r = subprocess.run([sys.executable, "-c", PRELUDE + script, library], capture_output=True, text=True, cwd=ROOT,
-                       env={**os.environ, "PYTHONPATH": ROOT}, timeout=300)
-    assert r.returncode == 0, r.stderr
-    return json.loads(r.stdout.splitlines()[-1])
+    return wrapped_library.link(str(tmp_path_factory.mktemp("refusing")), HOOK, ["cudaMalloc"])
 
 
 @pytest.mark.parametrize("precision", ["FP32", "FP64"])
 def test_without_memory_for_the_moments_the_tape_takes_checkpoints(library, precision):
     """The record and the gradient after a refused allocation of the moments of 200 steps; the
     gradient agrees with that of a tape that keeps them as gradients of other launch splits do."""
-    out = _run(library, r"""
+    out = wrapped_library.run(library, LIMIT + r"""
 prec = lbm_sw.%s
 nx, ny, steps = 96, 64, 200
 W0 = [x.reshape(ny, nx) for x in inputs.random_states(nx * ny, seed=7, h=(0.95, 1.05), speed=0.02)]
