@@ -404,9 +404,9 @@ typedef struct lbm_sw_tape_info {
  * `steps` bounds the tape's memory: its checkpoints and the moments of one segment.  Errors: LBM_SW_E_ARG (1D handle, bad counts), LBM_SW_E_NOMEM. */
 LBM_SW_API int lbm_sw_tape_create(lbm_sw* h, int steps, int interval, lbm_sw_tape** out);
 
-/* Release a tape.  Its device memory is kept for the handle's next tape (one block per handle, 8 GB
- * in the process; it is freed with the handle) or, where it is not kept, freed after the owner's
- * stream is idle.  NULL-safe. */
+/* Release a tape (synchronises the owner's stream).  Its device memory is kept for the handle's next
+ * tape (one block per handle, 8 GB in the process; it is freed with the handle) or, where it
+ * is not kept, freed.  NULL-safe. */
 LBM_SW_API void lbm_sw_tape_destroy(lbm_sw_tape* t);
 
 /* Advance h by the tape's steps from its current state (its W^0 is the state at this

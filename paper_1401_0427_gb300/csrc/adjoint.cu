@@ -578,10 +578,8 @@ extern "C" {
 
 void lbm_sw_tape_destroy(lbm_sw_tape* t) {
   if (!t) return;
-  if (t->mem && !(t->memory && t->memory->give(t->mem, t->mem_bytes))) {
-    cudaStreamSynchronize(t->stream);
-    cudaFree(t->mem);
-  }
+  if (t->mem) cudaStreamSynchronize(t->stream);  // gradients on the device are there when this returns
+  if (t->mem && !(t->memory && t->memory->give(t->mem, t->mem_bytes))) cudaFree(t->mem);
   delete t;
 }
 

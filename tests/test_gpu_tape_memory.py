@@ -63,3 +63,25 @@ print(json.dumps({"kept": kept, "refused": refused, "off": float(np.abs(grads[0]
 """ % precision)
     assert out["kept"] == [True, False] and out["refused"] == 1
     assert out["off"] <= (1e-5 if precision == "FP32" else 1e-12)
+
+
+def test_releasing_a_tape_waits_for_its_work():
+    """lbm_sw_tape_destroy synchronises the owner's stream, also where it keeps the tape's memory: a
+    gradient on the device may then be read on any other stream."""
+    import torch
+
+    from paper_1401_0427_gb300 import inputs, lbm_sw
+
+    nx = ny = 512
+    W0 = [x.reshape(ny, nx) for x in inputs.random_states(nx * ny, seed=8, h=(0.95, 1.05), speed=0.02)]
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream), lbm_sw.Simulation(nx, ny, stream=stream.cuda_stream) as sim:
+        g = torch.full((ny, nx), 1e-3, dtype=torch.float64, device="cuda")
+        for _ in range(3):
+            sim.set_state(*W0)
+            tape = lbm_sw.Tape(sim, 400)
+            tape.record()
+            tape.adjoint(g)
+            assert not stream.query()  # 400 reverse steps: more than a millisecond
+            tape.close()
+            assert stream.query()
