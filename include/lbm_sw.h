@@ -27,8 +27,8 @@
  * there is no CPU fallback.  No function throws; every function that can fail
  * returns a status code (LBM_SW_OK = 0 or a negative LBM_SW_E_*), and the handle
  * keeps a message for the last failure (lbm_sw_last_error).  Many handles may
- * coexist; the library keeps no global state but the count of the bytes that handles hold
- * for their next tape.
+ * coexist; the library keeps no global state but a list of the memory that handles hold for
+ * their next tape.
  *
  * Layouts at this boundary
  *   - Moment fields (h, hu, hv) are FP64 arrays of nx*ny values, row-major
@@ -405,8 +405,8 @@ typedef struct lbm_sw_tape_info {
 LBM_SW_API int lbm_sw_tape_create(lbm_sw* h, int steps, int interval, lbm_sw_tape** out);
 
 /* Release a tape (synchronises the owner's stream).  Its device memory is kept for the handle's next
- * tape (one block per handle, 8 GB in the process; it is freed with the handle) or, where it
- * is not kept, freed.  NULL-safe. */
+ * tape (one block per handle, 8 GB in the process; it is freed with the handle, and when an
+ * allocation of the library finds no memory) or, where it is not kept, freed.  NULL-safe. */
 LBM_SW_API void lbm_sw_tape_destroy(lbm_sw_tape* t);
 
 /* Advance h by the tape's steps from its current state (its W^0 is the state at this

@@ -20,7 +20,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -323,55 +322,7 @@ dim3 grid_for(int nx, int ny, dim3 block) {
   return dim3(gx, static_cast<unsigned>(gy < 65535 ? gy : 65535));
 }
 
-std::atomic<size_t> g_tape_kept{0};  // bytes kept by all handles
-
 }  // namespace
-
-void* TapeMemory::take(size_t need, size_t* got) {
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    if (mem) {
-      void* const m = mem;
-      const size_t b = bytes;
-      mem = nullptr;
-      bytes = 0;
-      g_tape_kept -= b;
-      if (b >= need && b / 2 <= need) {
-        *got = b;
-        return m;
-      }
-      cudaFree(m);
-    }
-  }
-  void* m = nullptr;
-  *got = need;
-  if (cudaMalloc(&m, need) == cudaSuccess) return m;
-  cudaGetLastError();  // the caller may go on with less: the next launch's check must not see this failure
-  return nullptr;
-}
-
-bool TapeMemory::give(void* m, size_t size) {
-  std::lock_guard<std::mutex> lock(mu);
-  if (closed || mem) return false;
-  if ((g_tape_kept += size) > kTapeKeepTotal) {
-    g_tape_kept -= size;
-    return false;
-  }
-  mem = m;
-  bytes = size;
-  return true;
-}
-
-void TapeMemory::close() {
-  std::lock_guard<std::mutex> lock(mu);
-  closed = true;
-  if (mem) {
-    cudaFree(mem);
-    g_tape_kept -= bytes;
-    mem = nullptr;
-  }
-}
-
 }  // namespace lbm
 
 struct lbm_sw_tape {

@@ -325,8 +325,9 @@ int lbm_sw_create(const lbm_sw_params* p, lbm_sw** out) {
   h->graph_chunk = p->graph_chunk == 0 ? 64 : (p->graph_chunk < 0 ? 0 : p->graph_chunk + (p->graph_chunk & 1));
 
   auto bail = [&](int code) {
+    const cudaError_t last = cudaGetLastError();  // device_alloc leaves none
     g_create_error = std::string("create: ") + lbm_sw_status_string(code) + ": " +
-                     cudaGetErrorString(cudaGetLastError());
+                     cudaGetErrorString(last == cudaSuccess && code == LBM_SW_E_NOMEM ? cudaErrorMemoryAllocation : last);
     lbm_sw_destroy(h);
     return code;
   };
@@ -335,17 +336,17 @@ int lbm_sw_create(const lbm_sw_params* p, lbm_sw** out) {
     return bail(LBM_SW_E_CUDA);
   const size_t bytes = state_bytes(h);
   for (int i = 0; i < 2; ++i) {
-    if (cudaMalloc(&h->buf[i], bytes) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
+    if (lbm::device_alloc(&h->buf[i], bytes) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
     if (cudaMemsetAsync(h->buf[i], 0, bytes, h->stream) != cudaSuccess) return bail(LBM_SW_E_CUDA);
   }
-  if (cudaMalloc(&h->inflow_feq, 4 * h->q * h->elem) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
+  if (lbm::device_alloc(&h->inflow_feq, 4 * h->q * h->elem) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
   if (h->kernel == LBM_SW_KERNEL_CLUSTER && p->nx <= lbm::kWindows1dMaxCells &&
-      cudaMalloc(&h->mail1d, p->precision == LBM_SW_FP64 ? lbm::mail1d_bytes<double>(p->nx)
+      lbm::device_alloc(&h->mail1d, p->precision == LBM_SW_FP64 ? lbm::mail1d_bytes<double>(p->nx)
                                                          : lbm::mail1d_bytes<float>(p->nx)) != cudaSuccess)
     return bail(LBM_SW_E_NOMEM);
-  if (cudaMalloc(&h->diag_partials, 5 * sizeof(double) * lbm::diag_max_blocks()) != cudaSuccess)
+  if (lbm::device_alloc(&h->diag_partials, 5 * sizeof(double) * lbm::diag_max_blocks()) != cudaSuccess)
     return bail(LBM_SW_E_NOMEM);
-  if (cudaMalloc(&h->diag_done, sizeof(unsigned)) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
+  if (lbm::device_alloc(&h->diag_done, sizeof(unsigned)) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
   if (cudaMemsetAsync(h->diag_done, 0, sizeof(unsigned), h->stream) != cudaSuccess) return bail(LBM_SW_E_CUDA);
   if (cudaMallocHost(&h->diag_host, 8 * sizeof(double)) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
   cudaError_t e;
@@ -370,7 +371,7 @@ int lbm_sw_set_state(lbm_sw* h, const double* depth, const double* hu, const dou
   const double *d = depth, *u = hu, *v = (h->p.dim == 2) ? hv : nullptr;
   if (!on_device) {
     if (!h->moments_staging)
-      LBM_CUDA(h, cudaMalloc(&h->moments_staging, 3 * n * sizeof(double)), "cudaMalloc(moments staging)");
+      LBM_CUDA(h, lbm::device_alloc(&h->moments_staging, 3 * n * sizeof(double)), "cudaMalloc(moments staging)");
     double* s = h->moments_staging;
     LBM_CUDA(h, cudaMemcpyAsync(s, depth, n * sizeof(double), cudaMemcpyHostToDevice, h->stream), "copy h");
     LBM_CUDA(h, cudaMemcpyAsync(s + n, hu, n * sizeof(double), cudaMemcpyHostToDevice, h->stream), "copy hu");
@@ -538,7 +539,7 @@ int lbm_sw_get_moments(lbm_sw* h, double* depth, double* hu, double* hv, int on_
   double *d = depth, *u = hu, *v = (h->p.dim == 2) ? hv : nullptr;
   if (!on_device) {
     if (!h->moments_staging)
-      LBM_CUDA(h, cudaMalloc(&h->moments_staging, 3 * n * sizeof(double)), "cudaMalloc(moments staging)");
+      LBM_CUDA(h, lbm::device_alloc(&h->moments_staging, 3 * n * sizeof(double)), "cudaMalloc(moments staging)");
     d = h->moments_staging;
     u = d + n;
     v = (h->p.dim == 2 && hv) ? d + 2 * n : nullptr;
@@ -603,7 +604,7 @@ int lbm_sw_set_populations(lbm_sw* h, const void* src, int on_device, int form) 
     const void* dense = src;
     if (!on_device) {
       if (!h->pop_staging)
-        LBM_CUDA(h, cudaMalloc(&h->pop_staging, h->q * dplane), "cudaMalloc(population staging)");
+        LBM_CUDA(h, lbm::device_alloc(&h->pop_staging, h->q * dplane), "cudaMalloc(population staging)");
       LBM_CUDA(h, cudaMemcpyAsync(h->pop_staging, src, h->q * dplane, cudaMemcpyHostToDevice, h->stream),
                "copy populations in");
       dense = h->pop_staging;
@@ -719,12 +720,12 @@ int lbm_sw_set_obstacle(lbm_sw* h, const unsigned char* solid, int on_device) {
     h->has_obstacles = false;
   } else {
     const size_t n = static_cast<size_t>(h->p.nx) * h->p.ny;
-    if (!h->solid) LBM_CUDA(h, cudaMalloc(&h->solid, n), "cudaMalloc (obstacle mask)");
+    if (!h->solid) LBM_CUDA(h, lbm::device_alloc(&h->solid, n), "cudaMalloc (obstacle mask)");
     LBM_CUDA(h, cudaMemcpyAsync(h->solid, solid, n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                                 h->stream), "obstacle mask copy");
     if (h->kernel != LBM_SW_KERNEL_SIMPLE) {
       if (!h->solid_flags)
-        LBM_CUDA(h, cudaMalloc(&h->solid_flags, static_cast<size_t>(h->plane)), "cudaMalloc (obstacle flags)");
+        LBM_CUDA(h, lbm::device_alloc(&h->solid_flags, static_cast<size_t>(h->plane)), "cudaMalloc (obstacle flags)");
       LBM_CUDA(h, lbm::launch_obstacle_flags(h->solid, h->solid_flags, h->p.nx, h->p.ny, h->pitch, h->p.bc, h->stream),
                "obstacle flags launch");
       h->launches += 1;

@@ -247,7 +247,7 @@ int ensure_staging(lbm_sw_batch* b, size_t cells) {
   if (b->moments_staging) cudaFree(b->moments_staging);
   b->moments_staging = nullptr;
   b->moments_staging_cells = 0;
-  BATCH_CUDA(b, cudaMalloc(&b->moments_staging, 3 * cells * sizeof(double)), "cudaMalloc(moments staging)");
+  BATCH_CUDA(b, lbm::device_alloc(&b->moments_staging, 3 * cells * sizeof(double)), "cudaMalloc(moments staging)");
   b->moments_staging_cells = cells;
   return LBM_SW_OK;
 }
@@ -359,7 +359,10 @@ int lbm_sw_batch_create(const lbm_sw_batch_params* p, lbm_sw_batch** out) {
   const int V = p->precision == LBM_SW_FP64 ? 2 : 4;
 
   auto bail = [&](int code, const char* what) {
-    lbm::set_create_error((std::string("batch create: ") + what + ": " + cudaGetErrorString(cudaGetLastError())).c_str());
+    const cudaError_t last = cudaGetLastError();  // device_alloc leaves none
+    lbm::set_create_error((std::string("batch create: ") + what + ": " +
+                           cudaGetErrorString(last == cudaSuccess && code == LBM_SW_E_NOMEM ? cudaErrorMemoryAllocation : last))
+                              .c_str());
     lbm_sw_batch_destroy(b);
     return code;
   };
@@ -385,7 +388,7 @@ int lbm_sw_batch_create(const lbm_sw_batch_params* p, lbm_sw_batch** out) {
   b->total_elems = off;
   const size_t bytes = static_cast<size_t>(off) * b->elem;
   for (int i = 0; i < 2; ++i) {
-    if (cudaMalloc(&b->buf[i], bytes) != cudaSuccess) return bail(LBM_SW_E_NOMEM, "cudaMalloc(populations)");
+    if (lbm::device_alloc(&b->buf[i], bytes) != cudaSuccess) return bail(LBM_SW_E_NOMEM, "cudaMalloc(populations)");
     if (cudaMemsetAsync(b->buf[i], 0, bytes, b->stream) != cudaSuccess) return bail(LBM_SW_E_CUDA, "cudaMemset");
   }
   const int rows_list[4] = {1, 2, 4, 8};
@@ -408,14 +411,14 @@ int lbm_sw_batch_create(const lbm_sw_batch_params* p, lbm_sw_batch** out) {
         }
     }
     b->tiles[r] = static_cast<long long>(tl.size());
-    if (cudaMalloc(&b->d_tiles[r], sizeof(lbm::TileRec) * tl.size()) != cudaSuccess)
+    if (lbm::device_alloc(&b->d_tiles[r], sizeof(lbm::TileRec) * tl.size()) != cudaSuccess)
       return bail(LBM_SW_E_NOMEM, "cudaMalloc(tile list)");
     if (cudaMemcpy(b->d_tiles[r], tl.data(), sizeof(lbm::TileRec) * tl.size(), cudaMemcpyHostToDevice) != cudaSuccess)
       return bail(LBM_SW_E_CUDA, "copy tile list");
   }
-  if (cudaMalloc(&b->inflow_feq, 4 * 13 * b->elem) != cudaSuccess) return bail(LBM_SW_E_NOMEM, "cudaMalloc");
-  if (cudaMalloc(&b->diag_partials, 5 * sizeof(double) * lbm::diag_max_blocks()) != cudaSuccess ||
-      cudaMalloc(&b->diag_done, sizeof(unsigned)) != cudaSuccess ||
+  if (lbm::device_alloc(&b->inflow_feq, 4 * 13 * b->elem) != cudaSuccess) return bail(LBM_SW_E_NOMEM, "cudaMalloc");
+  if (lbm::device_alloc(&b->diag_partials, 5 * sizeof(double) * lbm::diag_max_blocks()) != cudaSuccess ||
+      lbm::device_alloc(&b->diag_done, sizeof(unsigned)) != cudaSuccess ||
       cudaMemsetAsync(b->diag_done, 0, sizeof(unsigned), b->stream) != cudaSuccess ||
       cudaMallocHost(&b->diag_host, 8 * sizeof(double)) != cudaSuccess)
     return bail(LBM_SW_E_NOMEM, "cudaMalloc(diagnostics)");

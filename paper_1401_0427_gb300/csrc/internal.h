@@ -204,20 +204,33 @@ cudaError_t launch_diagnostics_blocks(const StepArgs<T>& a, int q, int nblocks, 
 
 // Device memory of a destroyed tape, kept for the next tape of the same handle (an optimiser makes
 // one per gradient, and allocating and freeing gigabytes takes milliseconds).  At most one block
-// per handle and kTapeKeepTotal bytes in the process; freed with the handle, or when a tape that it
-// does not fit is made.  Work of the old tape and of the next one is ordered by the handle's
-// stream.  The handle and its tapes share it: a tape may be destroyed after its handle, and in
-// another thread.
+// per handle and kTapeKeepTotal bytes in the process; freed with the handle, when a tape that it
+// does not fit is made, or when an allocation of the library finds no memory (device_alloc).  The handle
+// and its tapes share it: a tape may be destroyed after its handle, and in another thread.
 constexpr size_t kTapeKeepTotal = 8ull << 30;
 struct TapeMemory {
   std::mutex mu;
   void* mem = nullptr;
   size_t bytes = 0;
   bool closed = false;       // the handle is gone: nothing is kept any more
+  TapeMemory();
+  ~TapeMemory();
   void* take(size_t need, size_t* got);  // kept or new memory of at least `need` bytes, nullptr if there is none
   bool give(void* m, size_t size);       // true if kept, else the caller frees it
+  void release();                        // frees what is kept
   void close();
 };
+
+// cudaMalloc; where it finds no memory, what handles keep for their next tapes is freed and it is
+// tried once more.  A failure leaves no error behind for the next launch's check.
+cudaError_t device_alloc(void** p, size_t bytes);
+template <class T>
+cudaError_t device_alloc(T** p, size_t bytes) {
+  void* m = nullptr;
+  const cudaError_t e = device_alloc(&m, bytes);
+  *p = static_cast<T*>(m);
+  return e;
+}
 
 }  // namespace lbm
 

@@ -804,8 +804,8 @@ cudaError_t build_list(const std::vector<int>& ids, const int* nx, const int* ny
   const UnitList list = share >= 120LL * k ? deal_segments(strips, k, grid, (share + 5) / 6) : cut_strips(strips, k, grid);
   const std::vector<WaveUnit>& sorted = list.sorted;
   const std::vector<int>& first = list.first;
-  cudaError_t e = cudaMalloc(d_units, std::max<size_t>(1, sorted.size()) * sizeof(WaveUnit));
-  if (e == cudaSuccess) e = cudaMalloc(d_first, first.size() * sizeof(int));
+  cudaError_t e = device_alloc(d_units, std::max<size_t>(1, sorted.size()) * sizeof(WaveUnit));
+  if (e == cudaSuccess) e = device_alloc(d_first, first.size() * sizeof(int));
   if (e == cudaSuccess && !sorted.empty())
     e = cudaMemcpy(*d_units, sorted.data(), sorted.size() * sizeof(WaveUnit), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(*d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice);
