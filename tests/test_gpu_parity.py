@@ -12,6 +12,7 @@ import pytest
 
 from paper_1401_0427_gb300 import inputs, lbm_sw
 
+import wrapped_library
 from gpu_helpers import FP32_ELEM_TOL, FP64_TOL, gpu_post, oracle_params, oracle_post, rel_max
 
 pytestmark = pytest.mark.gpu
@@ -116,3 +117,46 @@ def test_1d_windows_equal_the_per_step_kernel(n, bc, precision, steps):
     a = gpu_post(F0, steps, kernel=lbm_sw.KERNEL_SIMPLE, **kw)
     b = gpu_post(F0, steps, kernel=lbm_sw.KERNEL_CLUSTER, **kw)
     assert np.array_equal(a, b, equal_nan=True)  # noise on 5473 cells leaves the admissible states
+
+
+@pytest.mark.parametrize("precision", [lbm_sw.FP64, lbm_sw.FP32])
+@pytest.mark.parametrize("bc", [(P, P), (W, O), (I, W)], ids=str)
+@pytest.mark.parametrize("n", [1, 2, 5, 31, 1000, 1216, 1217, 2433, 9121])
+@pytest.mark.parametrize("steps", [1, 2, 7, 8, 9, 14, 15, 16])
+def test_1d_windows_without_an_exchange_equal_the_per_step_kernel(n, bc, precision, steps):
+    """Runs of few steps, whose halo is as wide as their number: about the widths at which lines
+    exchange, the most steps that go without (15, pieces of two cells), and the lines (152 SMs)
+    on which such pieces no longer find a quarter of an SM each."""
+    inflow = [(1.3, 0.2, 0.0), (0.9, -0.15, 0.0), None, None]
+    F0 = inputs.random_populations(5, 1, n, seed=3700 + n)
+    kw = dict(dim=1, precision=precision, bc=bc, inflow=inflow, a=0.15)
+    a = gpu_post(F0, steps, kernel=lbm_sw.KERNEL_SIMPLE, **kw)
+    b = gpu_post(F0, steps, kernel=lbm_sw.KERNEL_CLUSTER, **kw)
+    assert np.array_equal(a, b, equal_nan=True)
+
+
+def test_1d_calls_of_few_steps_clear_no_mailbox(tmp_path):
+    """A call whose steps fit one halo launches one kernel and nothing else."""
+    library = wrapped_library.link(str(tmp_path), r"""
+#include <cuda_runtime.h>
+extern "C" cudaError_t __real_cudaMemsetAsync(void*, int, size_t, cudaStream_t);
+static int cleared = 0;
+extern "C" __attribute__((visibility("default"))) int clears() { return cleared; }
+extern "C" cudaError_t __wrap_cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t st) {
+  ++cleared;
+  return __real_cudaMemsetAsync(p, v, n, st);
+}
+""", ["cudaMemsetAsync"])
+    out = wrapped_library.run(library, r"""
+counts = []
+for prec in (lbm_sw.FP32, lbm_sw.FP64):
+    h, q = inputs.dam_break_1d(1000)
+    with lbm_sw.Simulation(1000, 1, dim=1, precision=prec, bc=(lbm_sw.WALL,) * 2, a=0.15) as sim:
+        sim.set_state(h, q)
+        for n in (1, 8, 15, 40):
+            before = lib.clears()
+            sim.step(n)
+            counts.append(lib.clears() - before)
+print(json.dumps(counts))
+""")
+    assert out == [0, 0, 0, 1] * 2
