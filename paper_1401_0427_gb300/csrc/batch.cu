@@ -49,8 +49,11 @@ struct TileRec {
 
 // Persistent form: gridDim.x CTAs walk the tile list; one CTA per tile when the
 // grid has as many CTAs as there are tiles.
+// FP32: registers for 20 warps per SM (us per step, 64 grids of sides 64 to 900 and 4 of 1000^2: 244.5 and
+// 65.7; left to the compiler 276 and 74, for 16 warps 266 and 69.8).  FP64: left to the compiler (1203 and 310,
+// 8 grids of 64^2 8.3; for 16 warps 1119, 289 and 10.3).
 template <class T, int BY>
-__global__ void __launch_bounds__(32 * BY)
+__global__ void __launch_bounds__(32 * BY, sizeof(T) == 4 ? 20 / BY : 1)
     batch_step(const TileRec* __restrict__ tiles, long long total_tiles, const T* __restrict__ src,
                T* __restrict__ dst, const T* __restrict__ inflow_feq, const BcSet bc, const Consts<T> K) {
   constexpr int V = V16<T>::n;
