@@ -400,7 +400,7 @@ int record_with_moments(lbm_sw* h, lbm_sw_tape* t, int len, T* W) {
   long long launches = 1;
   if constexpr (sizeof(T) == 4) {
     if (lbm::tile_active(h)) {  // register tiles, launches as even as they come (256^2: 4.6 -> 1.5 us per step)
-      const int most = lbm::tile_steps(h->p.nx, h->p.ny, std::max(h->sm_count, 1));
+      const int most = h->tile_k;
       for (int count = (len + most - 1) / most; count > 0; --count, from ^= 1, ++launches) {
         const int k = (len - j + count) / count;  // of the len - j + 1 steps left
         TAPE_CUDA(t, lbm::launch_step2d_tile_store_w(lbm::handle_args<float>(h, from), kd, k, W + 3 * P * j, 3 * P, st,

@@ -83,7 +83,7 @@ int obstacle_k(const lbm_sw* h) {
 // The launches of n > 0 steps on register tiles, as even as they come: launch(steps) for each.
 template <class F>
 int for_tile_launches(const lbm_sw* h, int n, F&& launch) {
-  const int k = lbm::tile_steps(h->p.nx, h->p.ny, std::max(h->sm_count, 1));
+  const int k = h->tile_k;
   const int count = (n + k - 1) / k, base = n / count, extra = n % count;
   for (int i = 0; i < count; ++i) {
     const int rc = launch(i < extra ? base + 1 : base);
@@ -218,13 +218,7 @@ thread_local std::string g_create_error;
 namespace lbm {
 // AUTO without a wish for temporal_steps.
 bool tile_active(const lbm_sw* h) {
-  if (!h->auto_kernel || h->p.temporal_steps != 0 || h->p.dim != 2 || h->p.precision != LBM_SW_FP32 ||
-      static_cast<long long>(h->p.nx) * h->p.ny >= kTileCells)
-    return false;
-  if (!temporal_active(h) && obstacle_k(h) == 0) return true;
-  int waves = 0;
-  tile_steps(h->p.nx, h->p.ny, std::max(h->sm_count, 1), &waves);
-  return waves <= 2;
+  return h->tile_k > 0 && ((!temporal_active(h) && obstacle_k(h) == 0) || h->tile_waves <= 2);
 }
 
 void set_create_error(const char* msg) { g_create_error = msg ? msg : ""; }
@@ -334,6 +328,9 @@ int lbm_sw_create(const lbm_sw_params* p, lbm_sw** out) {
   if (cudaGetDevice(&h->device) != cudaSuccess) return bail(LBM_SW_E_CUDA);
   if (cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
     return bail(LBM_SW_E_CUDA);
+  if (h->auto_kernel && p->temporal_steps == 0 && p->dim == 2 && p->precision == LBM_SW_FP32 &&
+      static_cast<long long>(p->nx) * p->ny < kTileCells)
+    h->tile_k = lbm::tile_steps(p->nx, p->ny, std::max(h->sm_count, 1), &h->tile_waves);
   const size_t bytes = state_bytes(h);
   for (int i = 0; i < 2; ++i) {
     if (lbm::device_alloc(&h->buf[i], bytes) != cudaSuccess) return bail(LBM_SW_E_NOMEM);

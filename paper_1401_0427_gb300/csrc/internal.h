@@ -261,6 +261,8 @@ struct lbm_sw {
   unsigned char* solid_flags = nullptr;  // [ny][pitch] bytes of the fused steps with obstacles
   bool has_obstacles = false;
   int graph_chunk = 64;
+  int tile_k = 0;            // steps per launch on register tiles, 0: not on these
+  int tile_waves = 0;        // waves of tiles of such a launch
   bool has_state = false;
   long long steps_done = 0;
   long long launches = 0;

@@ -65,9 +65,29 @@ __device__ __forceinline__ double times_pow2(double x) {
   return __dmul_rn(x, (NEG ? -1.0 : 1.0) * (k < 0 ? 1.0 / (1 << -k) : static_cast<double>(1 << (k < 0 ? 0 : k))));
 }
 
+// Constants of the FP64 collisions in integers; FP32 kernels have none (they are parameters of every launch).
+template <class T>
+struct FixedConsts {};
+template <>
+struct FixedConsts<double> {
+  // 1D: f0 = a_2 h + a_4g u^2
+  double a_2, a_4g;
+  // 2D (collide13_fixed): |1 - s| and s c in units of 2^-64, and whether they are below one
+  unsigned long long x_om, x_sc;
+  // the least difference of the families' exponents at which s c q stays below 2^62 units of the
+  // depths' (q is below 2^62 of its own): s c 2^-least_sc <= 1
+  int least_sc;
+  // 2D MRT (collide13_mrt_fixed): m[0], m[1], m[2] / 4, m[3] / 4, m[4 .. 9] and c likewise
+  unsigned long long x_m[10], x_c;
+  int least_c;  // c 2^-least_c <= 1/2: c q stays below 2^61 units of the depths'
+  // 1D (collide5_fixed): s / 2 likewise
+  unsigned long long x_s2;
+  bool om_neg, fixed_ok, fixed1_ok, fixed_mrt_ok;
+};
+
 // Scheme constants in the storage precision.
 template <class T>
-struct Consts {
+struct Consts : FixedConsts<T> {
   T s;       // relaxation rate
   T a;       // rest-potential weight
   T c;       // 1 / (2 lambda)
@@ -97,19 +117,6 @@ struct Consts {
   T s_p;    // s c g / 2
   T s_c;    // s c
   T s_4;    // s / 4
-  // 1D, FP64: f0 = a_2 h + a_4g u^2
-  T a_2, a_4g;
-  // 2D, FP64 (collide13_fixed): |1 - s|, s / 4 and s c in units of 2^-64, and whether they are below one
-  unsigned long long x_om, x_s4, x_sc;
-  // the least difference of the families' exponents at which s c q stays below 2^62 units of the
-  // depths' (q is below 2^62 of its own): s c 2^-least_sc <= 1
-  int least_sc;
-  // 2D MRT, FP64 (collide13_mrt_fixed): m[0], m[1], m[2] / 4, m[3] / 4, m[4 .. 9] and c likewise
-  unsigned long long x_m[10], x_c;
-  int least_c;  // c 2^-least_c <= 1/2: c q stays below 2^61 units of the depths'
-  // 1D, FP64 (collide5_fixed): s / 2 likewise
-  unsigned long long x_s2;
-  bool om_neg, fixed_ok, fixed1_ok, fixed_mrt_ok;
 };
 
 // |v| <= 1 in units of 2^-64 (saturated)
@@ -128,13 +135,15 @@ inline __host__ int least_shift(double v, double most) {
 template <class T>
 __host__ void set_mrt_folded(Consts<T>& k) {
   constexpr double scale[10] = {0.5, 0.5, 1.0, 1.0, 0.5, 0.5, 0.25, 0.5, 0.5, 0.25};
-  k.x_c = in_2_64(static_cast<double>(k.c));
-  k.least_c = least_shift(static_cast<double>(k.c), 0.5);
-  k.fixed_mrt_ok = k.c > T(0) && k.c <= T(0.5);
-  for (int i = 0; i < 10; ++i) {
-    k.m[i] = static_cast<T>(static_cast<double>(k.r[i]) * scale[i]);
-    k.x_m[i] = in_2_64(static_cast<double>(k.m[i]) * (i == 2 || i == 3 ? 0.25 : 1.0));
-    k.fixed_mrt_ok = k.fixed_mrt_ok && k.r[i] >= T(0) && k.r[i] <= T(2);
+  for (int i = 0; i < 10; ++i) k.m[i] = static_cast<T>(static_cast<double>(k.r[i]) * scale[i]);
+  if constexpr (sizeof(T) == 8) {
+    k.x_c = in_2_64(k.c);
+    k.least_c = least_shift(k.c, 0.5);
+    k.fixed_mrt_ok = k.c > 0.0 && k.c <= 0.5;
+    for (int i = 0; i < 10; ++i) {
+      k.x_m[i] = in_2_64(k.m[i] * (i == 2 || i == 3 ? 0.25 : 1.0));
+      k.fixed_mrt_ok = k.fixed_mrt_ok && k.r[i] >= 0.0 && k.r[i] <= 2.0;
+    }
   }
 }
 
@@ -154,16 +163,17 @@ __host__ Consts<T> make_consts(double g, double lambda, double s, double a) {
   k.s_p = static_cast<T>(st * c * g / 2.0);
   k.s_c = static_cast<T>(st * c);
   k.s_4 = static_cast<T>(st / 4.0);
-  k.a_2 = static_cast<T>(a / 2.0);
-  k.a_4g = static_cast<T>(-a / (4.0 * g));
-  k.x_om = in_2_64(1.0 - st);
-  k.x_s4 = in_2_64(st / 4.0);
-  k.x_sc = in_2_64(st * c);
-  k.least_sc = least_shift(st * c, 1.0);
-  k.om_neg = st > 1.0;
-  k.fixed_ok = st >= 0.0 && st <= 2.0 && st * c < 1.0;
-  k.x_s2 = in_2_64(st / 2.0);
-  k.fixed1_ok = st >= 0.0 && st <= 2.0 && c > 0.0 && c <= 1.0;
+  if constexpr (sizeof(T) == 8) {
+    k.a_2 = a / 2.0;
+    k.a_4g = -a / (4.0 * g);
+    k.x_om = in_2_64(1.0 - st);
+    k.x_sc = in_2_64(st * c);
+    k.least_sc = least_shift(st * c, 1.0);
+    k.om_neg = st > 1.0;
+    k.fixed_ok = st >= 0.0 && st <= 2.0 && st * c < 1.0;
+    k.x_s2 = in_2_64(st / 2.0);
+    k.fixed1_ok = st >= 0.0 && st <= 2.0 && c > 0.0 && c <= 1.0;
+  }
   for (int i = 0; i < 10; ++i) k.r[i] = k.s;
   set_mrt_folded(k);
   return k;
