@@ -390,10 +390,13 @@ constexpr int kRowsPerCta = sizeof(T) == 8 ? 1 : 4;
 
 // FP64: registers for 16 warps per SM on small grids, which have few (480 x 120: 5.7 us per step,
 // 6.1 with 24), for 24 on others (512^2 18.0 against 19.1, 1536^2 140 against 151).
-template <class T, class F>
+// FP32: for 20 warps per SM, with solid cells 16 (us per step with 16 / 20 / left to the compiler: BGK 780^2 8.2 / 7.3 /
+// 8.5 and 4096 x 2048 127 / 125 / 140, MRT 9.2 / 8.3 / 9.2 and 132 / 126 / 146, solid cells 9.1 / 12.5 / 9.4 and
+// 131 / 150 / 147).
+template <class T, bool OBST, class F>
 cudaError_t with_residency(const StepArgs<T>& a, F&& launch) {
   if constexpr (sizeof(T) == 4)
-    return launch(std::integral_constant<int, 4>{});
+    return launch(std::integral_constant<int, OBST ? 4 : 5>{});
   else if (static_cast<long long>(a.nx) * a.ny >= (1LL << 17))
     return launch(std::integral_constant<int, 24>{});
   else
@@ -428,7 +431,7 @@ cudaError_t launch_step2d(const StepArgs<T>& a, const ConstsD& kd, int variant, 
       step2d_simple<T, false><<<cell_grid(a.nx, a.ny, block), block, 0, st>>>(a, K);
     return cudaGetLastError();
   }
-  return with_residency<T>(a, [&](auto res) {
+  return with_residency<T, false>(a, [&](auto res) {
     constexpr int BY = kRowsPerCta<T>, RES = decltype(res)::value;
     return kd.mrt ? launch_rows<T, BY>(step2d_vec<T, BY, true, RES>, a, st, K)
                   : launch_rows<T, BY>(step2d_vec<T, BY, false, RES>, a, st, K);
@@ -448,7 +451,7 @@ cudaError_t launch_step2d_obstacle(const StepArgs<T>& a, const ConstsD& kd, cons
       step2d_obstacle<T, false><<<cell_grid(a.nx, a.ny, block), block, 0, st>>>(a, K, mask);
     return cudaGetLastError();
   }
-  return with_residency<T>(a, [&](auto res) {
+  return with_residency<T, true>(a, [&](auto res) {
     constexpr int BY = kRowsPerCta<T>, RES = decltype(res)::value;
     return kd.mrt ? launch_rows<T, BY>(step2d_vec_obstacle<T, BY, true, RES>, a, st, K, mask)
                   : launch_rows<T, BY>(step2d_vec_obstacle<T, BY, false, RES>, a, st, K, mask);
