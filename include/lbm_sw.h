@@ -194,7 +194,7 @@ LBM_SW_API int lbm_sw_set_state(lbm_sw* h, const double* depth, const double* hu
  *             lbm_sw_step_plan lists the launches;
  *   CLUSTER:  one launch for all n steps (1D lines up to 16384 cells);
  *   AUTO on FP32 grids below 5 * 2^17 cells (temporal_steps = 0): launches of up to 8 steps, as
- *             even as they come (lbm_sw_step_plan);
+ *             even as they come (two may run as two single ones; lbm_sw_step_plan);
  *   TEMPORAL with obstacles: the same with K = min(temporal_steps, 6), without odd counts (BGK and
  *             an even temporal_steps; otherwise one launch per step);
  *   VEC, SIMPLE: one launch per step; long runs replay a captured CUDA graph of

@@ -80,13 +80,29 @@ int obstacle_k(const lbm_sw* h) {
   return std::min(h->temporal_k, 6);
 }
 
-// The launches of n > 0 steps on register tiles, as even as they come: launch(steps) for each.
+// What takes a launch of two steps where register tiles run: tiles reload their halo for little then.
+// The wavefront where it applies, for even widths without solid cells (us, tiles / wavefront: 700 x 600 9.7 / 9.3
+// periodic and 11.3 / 9.3 with sides, 200 x 2000 10.1 / 9.8 and 11.8 / 9.9, 1024 x 512 12.1 / 11.1 and 13.1 /
+// 11.3; 801 x 601 11.4 / 13.1); two single steps for MRT with sides from 5 * 2^14 cells on (450 x 200 7.6 / 6.7,
+// 640^2 12.8 / 12.3, 1024 x 512 15.2 / 13.8; 256^2 4.6 / 5.1).
+enum class TwoSteps { tile, wave, singles };
+TwoSteps two_steps(const lbm_sw* h) {
+  const bool per = h->p.bc[LBM_SW_SIDE_XM] == LBM_SW_BC_PERIODIC && h->p.bc[LBM_SW_SIDE_YM] == LBM_SW_BC_PERIODIC;
+  if (h->has_obstacles) return TwoSteps::tile;
+  if (h->mrt) return !per && static_cast<long long>(h->p.nx) * h->p.ny >= (5LL << 14) ? TwoSteps::singles : TwoSteps::tile;
+  return temporal_active(h) && h->p.nx % 2 == 0 ? TwoSteps::wave : TwoSteps::tile;
+}
+
+// The launches of n > 0 steps where register tiles run, as even as they come: launch(steps) for each.
 template <class F>
 int for_tile_launches(const lbm_sw* h, int n, F&& launch) {
   const int k = h->tile_k;
   const int count = (n + k - 1) / k, base = n / count, extra = n % count;
   for (int i = 0; i < count; ++i) {
-    const int rc = launch(i < extra ? base + 1 : base);
+    const int steps = i < extra ? base + 1 : base;
+    const bool singles = steps == 2 && two_steps(h) == TwoSteps::singles;
+    int rc = launch(singles ? 1 : steps);
+    if (rc == LBM_SW_OK && singles) rc = launch(1);
     if (rc != LBM_SW_OK) return rc;
   }
   return LBM_SW_OK;
@@ -421,8 +437,11 @@ int lbm_sw_step(lbm_sw* h, int n) {
     return for_tile_launches(h, n, [&](int k) {
       const auto a = args<float>(h, h->cur);
       const unsigned char* flags = h->has_obstacles ? h->solid_flags : nullptr;
-      const cudaError_t e = k == 1 ? launch_one_step(h, h->cur, h->stream)
-                                   : lbm::launch_step2d_tile(a, consts(h), k, flags, h->stream, h->sm_count);
+      const cudaError_t e =
+          k == 1 ? launch_one_step(h, h->cur, h->stream)
+          : k == 2 && two_steps(h) == TwoSteps::wave
+              ? lbm::launch_step2d_temporal(a, consts(h), 2, h->stream, h->sm_count)
+              : lbm::launch_step2d_tile(a, consts(h), k, flags, h->stream, h->sm_count);
       if (e != cudaSuccess) return cuda_fail(h, e, "tile step launch");
       h->cur ^= 1;
       h->steps_done += k;

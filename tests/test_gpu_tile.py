@@ -41,3 +41,19 @@ def test_tile_launch_plan():
             before = sim.info().kernel_launches
             sim.step(n)
             assert sim.info().kernel_launches - before == len(plan)
+
+
+@pytest.mark.parametrize("nx,ny,bc,mrt,plan", [
+    (700, 600, (P, P, P, P), None, [2]), (700, 600, (W, O, I, W), None, [2]), (701, 600, (W, O, I, W), None, [2]),
+    (256, 319, (W, W, W, W), RATES, [2]), (256, 320, (W, W, W, W), RATES, [1, 1]), (256, 320, (P, P, P, P), RATES, [2]),
+    (700, 600, (I, W, P, P), RATES, [1, 1]), (640, 620, (W, O, I, W), None, [2])])
+def test_two_steps(nx, ny, bc, mrt, plan):
+    """Two steps take what is fastest there: tiles, the wavefront (even widths from 3 * 2^17 cells on), or
+    two single steps (MRT with sides from 5 * 2^14 cells on).  The same bits as one step per launch."""
+    with lbm_sw.Simulation(nx, ny, bc=bc, inflow=INFLOW) as sim:
+        if mrt:
+            sim.set_relaxation(mrt)
+        assert sim.step_plan(2) == plan
+    F0 = inputs.random_populations(13, ny, nx, seed=9200 + nx + ny).astype(np.float32)
+    kw = dict(dim=2, precision=lbm_sw.FP32, bc=bc, inflow=INFLOW, a=0.05, mrt_rates=mrt)
+    assert np.array_equal(gpu_post(F0, 2, kernel=lbm_sw.KERNEL_VEC, **kw), gpu_post(F0, 2, **kw), equal_nan=True)
