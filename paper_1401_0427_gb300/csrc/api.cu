@@ -294,7 +294,6 @@ void lbm_sw_destroy(lbm_sw* h) {
   if (h->diag_done) cudaFree(h->diag_done);
   if (h->diag_host) cudaFreeHost(h->diag_host);
   if (h->solid) cudaFree(h->solid);
-  if (h->solid_flags) cudaFree(h->solid_flags);
   delete h;
 }
 
@@ -735,19 +734,26 @@ int lbm_sw_set_obstacle(lbm_sw* h, const unsigned char* solid, int on_device) {
   if (!solid) {
     h->has_obstacles = false;
   } else {
-    const size_t n = static_cast<size_t>(h->p.nx) * h->p.ny;
-    if (!h->solid) LBM_CUDA(h, lbm::device_alloc(&h->solid, n), "cudaMalloc (obstacle mask)");
-    LBM_CUDA(h, cudaMemcpyAsync(h->solid, solid, n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                                h->stream), "obstacle mask copy");
-    if (h->kernel != LBM_SW_KERNEL_SIMPLE) {
-      if (!h->solid_flags)
-        LBM_CUDA(h, lbm::device_alloc(&h->solid_flags, static_cast<size_t>(h->plane)), "cudaMalloc (obstacle flags)");
-      LBM_CUDA(h, lbm::launch_obstacle_flags(h->solid, h->solid_flags, h->p.nx, h->p.ny, h->pitch, h->p.bc, h->stream),
+    const size_t n = static_cast<size_t>(h->p.nx) * h->p.ny, at = static_cast<size_t>(round_up(n, 256));
+    const bool flags = h->kernel != LBM_SW_KERNEL_SIMPLE;
+    if (!h->solid) {
+      LBM_CUDA(h, lbm::device_alloc(&h->solid, at + (flags ? static_cast<size_t>(h->plane) : 0)), "cudaMalloc (obstacle mask)");
+      if (flags) h->solid_flags = h->solid + at;
+    }
+    const bool direct = on_device && flags && lbm::kernel_reaches(solid);  // the flags' kernel copies the mask too
+    if (!direct) {
+      LBM_CUDA(h, cudaMemcpyAsync(h->solid, solid, n, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                                  h->stream), "obstacle mask copy");
+      // the caller may reuse its buffer when this returns
+      LBM_CUDA(h, cudaStreamSynchronize(h->stream), "set_obstacle synchronize");
+    }
+    if (flags) {
+      LBM_CUDA(h, lbm::launch_obstacle_flags(direct ? solid : h->solid, direct ? h->solid : nullptr, h->solid_flags,
+                                             h->p.nx, h->p.ny, h->pitch, h->p.bc, h->stream),
                "obstacle flags launch");
       h->launches += 1;
     }
-    // the caller may reuse its buffer when this returns
-    LBM_CUDA(h, cudaStreamSynchronize(h->stream), "set_obstacle synchronize");
+    if (direct) LBM_CUDA(h, cudaStreamSynchronize(h->stream), "set_obstacle synchronize");
     h->has_obstacles = true;
   }
   // the captured graphs hold the previous step kernel

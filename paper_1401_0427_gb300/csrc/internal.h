@@ -82,6 +82,8 @@ struct PlaneCopy {
   int rows, planes;
 };
 cudaError_t copy_planes(const PlaneCopy& c, size_t elem, cudaStream_t st);
+// Whether a kernel may dereference p: memory of the current device, or managed memory.
+bool kernel_reaches(const void* p);
 
 // K reverse steps of the discrete adjoint per launch (adjoint_temporal.cu; FP32; every side
 // periodic with k in {2, 4, 6, 8}, or any sides with an even nx and k in {2, 4}): Phi^{n0}
@@ -146,8 +148,8 @@ cudaError_t launch_step2d_temporal_mrt(const StepArgs<float>& a, const ConstsD& 
                                        int sm_count);
 
 // k (2, 4 or 6) fused BGK steps with solid cells (temporal_obstacle.cu).
-cudaError_t launch_obstacle_flags(const unsigned char* solid, unsigned char* flags, int nx, int ny, long long pitch,
-                                  const int bc[4], cudaStream_t st);
+cudaError_t launch_obstacle_flags(const unsigned char* solid, unsigned char* copy, unsigned char* flags, int nx, int ny,
+                                  long long pitch, const int bc[4], cudaStream_t st);
 cudaError_t launch_step2d_temporal_obstacle(const StepArgs<float>& a, const ConstsD& kd, const unsigned char* flags,
                                             int k, cudaStream_t st, int sm_count);
 
@@ -258,7 +260,7 @@ struct lbm_sw {
   bool mrt = false;          // set by lbm_sw_set_relaxation
   double mrt_rates[10] = {};
   unsigned char* solid = nullptr;  // obstacle mask [ny][nx] on the device (lbm_sw_set_obstacle)
-  unsigned char* solid_flags = nullptr;  // [ny][pitch] bytes of the fused steps with obstacles
+  unsigned char* solid_flags = nullptr;  // [ny][pitch] bytes of the steps with obstacles, behind the mask in its block
   bool has_obstacles = false;
   int graph_chunk = 64;
   int tile_k = 0;            // steps per launch on register tiles, 0: not on these

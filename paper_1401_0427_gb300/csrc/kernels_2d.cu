@@ -348,8 +348,7 @@ dim3 cell_grid(int nx, int ny, dim3 block) {
 
 }  // namespace
 
-// Whether a kernel may dereference p: memory of the current device, or managed memory.
-static bool kernel_reaches(const void* p) {
+bool kernel_reaches(const void* p) {
   cudaPointerAttributes a{};
   int device = -1;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&device) != cudaSuccess) {

@@ -5,7 +5,7 @@ import pytest
 
 from paper_1401_0427_gb300 import inputs, lbm_sw
 
-from gpu_helpers import torch_stream
+from gpu_helpers import gpu_post, torch_stream
 
 pytestmark = pytest.mark.gpu
 
@@ -70,3 +70,24 @@ def test_tiles_with_obstacles_equal_single_steps(nx, ny, fraction, bc, mrt):
                 sim.step(steps)
                 out.append(sim.populations())
         assert np.array_equal(out[0], out[1], equal_nan=True), steps
+
+
+@pytest.mark.parametrize("bc", [(P, P, P, P), (W, W, W, W), (P, P, W, O), (W, O, P, P)], ids=lambda b: "".join("PWOI"[k] for k in b))
+@pytest.mark.parametrize("nx,ny", [(1, 1), (2, 1), (3, 4), (4, 1), (4, 3), (5, 2), (32, 3), (63, 9), (64, 9), (66, 7), (130, 5),
+                                   (516, 3), (1025, 2)])
+def test_masks_from_host_and_device(nx, ny, bc):
+    """The flags of the steps with obstacles come from host masks, device masks and device masks that do
+    not start on a word alike: the bits of the kernel that reads the mask itself."""
+    import torch
+
+    solid = inputs.random_obstacles(ny, nx, seed=9400 + nx, fraction=0.4)
+    F0 = inputs.random_populations(13, ny, nx, seed=9410 + nx)
+    flat = torch.zeros(nx * ny + 1, dtype=torch.uint8, device="cuda")
+    off = flat[1:]
+    off.copy_(torch.from_numpy(np.ascontiguousarray(solid, dtype=np.uint8)).cuda().reshape(-1))
+    masks = [solid, torch.from_numpy(np.ascontiguousarray(solid, dtype=np.uint8)).cuda(), off.reshape(ny, nx)]
+    for precision in (lbm_sw.FP32, lbm_sw.FP64):
+        kw = dict(dim=2, precision=precision, bc=bc, inflow=None, a=0.05)
+        want = gpu_post(F0, 3, kernel=lbm_sw.KERNEL_SIMPLE, solid=solid, **kw)
+        for mask in masks:
+            assert np.array_equal(gpu_post(F0, 3, solid=mask, **kw), want)
