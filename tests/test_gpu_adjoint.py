@@ -408,3 +408,26 @@ def test_an_interval_bounds_the_memory_and_replays(interval, kernel, k, precisio
     for first, second, ref in zip(*g_b, g_a[0]):
         assert np.array_equal(first, second)
         assert np.abs(first - ref).max() <= tol * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("bc", [(P, P, P, P), (W, O, I, W)], ids=["periodic", "sides"])
+@pytest.mark.parametrize("nx,ny", [(64, 64), (512, 512), (513, 500), (600, 601)])
+def test_long_recording_launches_on_register_tiles(nx, ny, bc):
+    """One interval of all 25 steps, so the record runs launches of up to 8: tiles of 32 rows (64^2) and of 48, in
+    one wave and two, odd widths, each with the same bits as one step per launch, and the
+    gradients as those of the small grids above."""
+    steps = 25
+    W0 = [x.reshape(ny, nx) for x in inputs.random_states(nx * ny, seed=570 + nx, h=(0.95, 1.05), speed=0.02)]
+    out = []
+    for kernel in (lbm_sw.KERNEL_AUTO, lbm_sw.KERNEL_VEC):
+        with lbm_sw.Simulation(nx, ny, kernel=kernel, bc=bc, inflow=INFLOW, stream=torch_stream()) as sim:
+            sim.set_state(*W0)
+            with lbm_sw.Tape(sim, steps, steps) as tape:
+                tape.record()
+                F = sim.populations()
+                out.append((F, tape.adjoint(sim.moments()[0] - 1.0, want_momentum=True)))
+    (F_a, g_a), (F_b, g_b) = out
+    assert np.array_equal(F_a, F_b)
+    scale = max(np.abs(b).max() for b in g_b)
+    for a, b in zip(g_a, g_b):
+        assert np.abs(a - b).max() <= 1e-5 * scale

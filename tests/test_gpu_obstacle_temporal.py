@@ -91,3 +91,16 @@ def test_masks_from_host_and_device(nx, ny, bc):
         want = gpu_post(F0, 3, kernel=lbm_sw.KERNEL_SIMPLE, solid=solid, **kw)
         for mask in masks:
             assert np.array_equal(gpu_post(F0, 3, solid=mask, **kw), want)
+
+
+@pytest.mark.parametrize("bc", [(P, P, P, P), (W, O, I, W)], ids=["periodic", "sides"])
+@pytest.mark.parametrize("nx,ny", [(900, 800), (901, 760)])
+def test_auto_takes_four_steps_on_middle_grids(nx, ny, bc):
+    """AUTO from 5 * 2^17 cells on (three waves of register tiles and more): the wavefront of four
+    steps in 128-column strips, and of two in the tail."""
+    solid = inputs.random_obstacles(ny, nx, seed=990 + nx, fraction=0.03)
+    F0 = np.concatenate([inputs.random_populations(13, 40, nx, seed=991)] * (ny // 40), axis=1).astype(np.float32)
+    a, _ = _run(F0, 22, bc, solid, lbm_sw.KERNEL_SIMPLE)
+    b, plan = _run(F0, 22, bc, solid, lbm_sw.KERNEL_AUTO)
+    assert plan == [4] * 5 + [2]
+    assert np.array_equal(a, b, equal_nan=True)
