@@ -145,7 +145,7 @@ cudaError_t planes_out(lbm_sw* h, const char* src, void* dst, size_t row, size_t
   if (on_device) {
     h->launches += 1;
     return lbm::copy_planes({src, pitch, plane, dst, static_cast<long long>(row), static_cast<long long>(dplane),
-                             static_cast<long long>(row), rows, h->q}, h->elem, h->stream);
+                             static_cast<long long>(row), rows, h->q, dst}, h->elem, h->stream);
   }
   for (int p = 0; p < h->q; ++p) {
     const cudaError_t e = cudaMemcpy2DAsync(static_cast<char*>(dst) + p * dplane, row, src + p * plane, pitch, row, rows,
@@ -159,7 +159,7 @@ cudaError_t planes_in(lbm_sw* h, char* dst, const void* src, size_t row, size_t 
   if (on_device) {
     h->launches += 1;
     return lbm::copy_planes({src, static_cast<long long>(row), static_cast<long long>(dplane), dst, pitch, plane,
-                             static_cast<long long>(row), rows, h->q}, h->elem, h->stream);
+                             static_cast<long long>(row), rows, h->q, src}, h->elem, h->stream);
   }
   for (int p = 0; p < h->q; ++p) {
     const cudaError_t e = cudaMemcpy2DAsync(dst + p * plane, pitch, static_cast<const char*>(src) + p * dplane, row, row,

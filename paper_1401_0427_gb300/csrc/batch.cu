@@ -559,7 +559,7 @@ int lbm_sw_batch_get_populations(lbm_sw_batch* b, int i, void* dst, int on_devic
     BATCH_CUDA(b,
                lbm::copy_planes({src, static_cast<long long>(I.pitch * b->elem), static_cast<long long>(I.plane * b->elem),
                                  dst, static_cast<long long>(row), static_cast<long long>(dplane),
-                                 static_cast<long long>(row), I.ny, 13},
+                                 static_cast<long long>(row), I.ny, 13, dst},
                                 b->elem, b->stream),
                "copy populations out");
   else

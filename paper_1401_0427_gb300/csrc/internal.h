@@ -72,7 +72,7 @@ template <class Tin, class Tout>
 cudaError_t launch_convert(const Tin* in, Tout* out, long long n, cudaStream_t st);
 
 // Device-to-device copy of `rows` rows of each of `planes` planes (pitches and planes in bytes) of
-// elements of `elem` (4 or 8) bytes.
+// elements of `elem` (4 or 8) bytes.  One side is the library's own memory, `theirs` the caller's pointer.
 struct PlaneCopy {
   const void* src;
   long long src_pitch, src_plane;
@@ -80,6 +80,7 @@ struct PlaneCopy {
   long long dst_pitch, dst_plane;
   long long row_bytes;
   int rows, planes;
+  const void* theirs;
 };
 cudaError_t copy_planes(const PlaneCopy& c, size_t elem, cudaStream_t st);
 // Whether a kernel may dereference p: memory of the current device, or managed memory.

@@ -368,7 +368,7 @@ cudaError_t copy_planes(const PlaneCopy& c, size_t elem, cudaStream_t st) {
            c.src_pitch % a == 0 && c.dst_pitch % a == 0 && c.src_plane % a == 0 && c.dst_plane % a == 0;
   };
   if (c.rows < 1 || c.row_bytes < 1) return cudaSuccess;
-  if (kernel_reaches(c.src) && kernel_reaches(c.dst)) {
+  if (kernel_reaches(c.theirs)) {
     if (aligned(16)) return copy_planes_as<uint4>(c, st);
     if (elem == 8 && aligned(8)) return copy_planes_as<unsigned long long>(c, st);
     if (elem == 4 && aligned(4)) return copy_planes_as<unsigned>(c, st);
