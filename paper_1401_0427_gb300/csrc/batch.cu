@@ -47,20 +47,26 @@ struct TileRec {
   int pad;
 };
 
+template <class T>
+constexpr int kTileParts = V16<T>::n / RowVec<T>::n;
+
 // Persistent form: gridDim.x CTAs walk the tile list; one CTA per tile when the
 // grid has as many CTAs as there are tiles.
+// A tile's row is 32 words of 16 bytes, which a warp takes (FP32), or two warps of different CTAs, with one cell
+// per thread (FP64).
 // FP32: registers for 20 warps per SM (us per step, 64 grids of sides 64 to 900 and 4 of 1000^2: 244.5 and
-// 65.7; left to the compiler 276 and 74, for 16 warps 266 and 69.8).  FP64: left to the compiler (1203 and 310,
-// 8 grids of 64^2 8.3; for 16 warps 1119, 289 and 10.3).
+// 65.7; left to the compiler 276 and 74, for 16 warps 266 and 69.8).  FP64: one cell per thread, for 24 warps
+// (1068 and 280, 8 grids of 64^2 8.3; two cells, left to the compiler 1203 and 310, for 16 warps 1119, 289 and 10.3).
 template <class T, int BY>
-__global__ void __launch_bounds__(32 * BY, sizeof(T) == 4 ? 20 / BY : 1)
+__global__ void __launch_bounds__(32 * BY, (sizeof(T) == 4 ? 20 : 24) / BY)
     batch_step(const TileRec* __restrict__ tiles, long long total_tiles, const T* __restrict__ src,
                T* __restrict__ dst, const T* __restrict__ inflow_feq, const BcSet bc, const Consts<T> K) {
-  constexpr int V = V16<T>::n;
-  for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x) {
-    const TileRec r = tiles[t];
-    const int y = r.y0 + threadIdx.y;
-    if (y >= r.ny) continue;  // warp-uniform
+  constexpr int V = RowVec<T>::n;
+  constexpr int S = kTileParts<T>;
+  for (long long t = blockIdx.x; t < total_tiles * S; t += gridDim.x) {
+    const TileRec r = tiles[t / S];
+    const int y = r.y0 + threadIdx.y, x0 = r.x0 + static_cast<int>(t % S) * 32 * V;
+    if (y >= r.ny || x0 >= r.nx) continue;  // warp-uniform
     StepArgs<T> A;
     A.src = src + r.offset;
     A.dst = dst + r.offset;
@@ -71,7 +77,7 @@ __global__ void __launch_bounds__(32 * BY, sizeof(T) == 4 ? 20 / BY : 1)
     A.plane = r.plane;
 #pragma unroll
     for (int s = 0; s < 4; ++s) A.bc[s] = bc.bc[s];
-    vec_row<T, false>(A, K, y, r.x0 + threadIdx.x * V, threadIdx.x, nullptr);
+    vec_row<T, false, false, false, RowVec<T>>(A, K, y, x0 + threadIdx.x * V, threadIdx.x, nullptr);
   }
 }
 
@@ -162,8 +168,8 @@ template <class T>
 cudaError_t launch_batch_t(const lbm_sw_batch* b, int from, int rows, int ctas, cudaStream_t st) {
   const int ri = rows_index(rows);
   const long long tiles = b->tiles[ri];
-  const long long want = ctas > 0 ? static_cast<long long>(b->sm_count) * ctas : tiles;  // 0: one CTA per tile
-  const unsigned grid = static_cast<unsigned>(tiles < want ? tiles : want);
+  const long long want = ctas > 0 ? static_cast<long long>(b->sm_count) * ctas : tiles * lbm::kTileParts<T>;  // 0: one CTA per part of a tile
+  const unsigned grid = static_cast<unsigned>(std::min(tiles * lbm::kTileParts<T>, want));
   lbm::BcSet bc;
   for (int s = 0; s < 4; ++s) bc.bc[s] = b->p.bc[s];
   const lbm::Consts<T> K = lbm::make_consts<T>(b->p.g, b->p.lambda, b->p.s, b->p.a);
