@@ -73,8 +73,14 @@ __device__ __forceinline__ T pull_one(const StepArgs<T>& A, int p, int x, int y)
   }
 }
 
+// CTAs per SM that the one-thread-per-cell kernels have registers for.  us per step on 1500 x 1000 cells, left to the
+// compiler / with 3 / 4 / 5: FP32 BGK 31.5 / 35.6 / 32.4 / 28.1, with solid cells 93 / 93 / 75 / 62; FP64 BGK 112 /
+// 102 / 101 / 138, with solid cells 196 / 165 / 159 / 186.
+template <class T>
+constexpr int kSimpleCtas = sizeof(T) == 4 ? 5 : 4;
+
 template <class T, bool MRT>
-__global__ void __launch_bounds__(256) step2d_simple(const StepArgs<T> A, const Consts<T> K) {
+__global__ void __launch_bounds__(256, kSimpleCtas<T>) step2d_simple(const StepArgs<T> A, const Consts<T> K) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   for (int y = blockIdx.y * blockDim.y + threadIdx.y; y < A.ny; y += gridDim.y * blockDim.y) {
     if (x >= A.nx) continue;
@@ -96,7 +102,7 @@ __global__ void __launch_bounds__(256) step2d_simple(const StepArgs<T> A, const 
 // Solid cells hold no fluid and keep their populations (copied to the new buffer).
 // --------------------------------------------------------------------------
 template <class T, bool MRT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, kSimpleCtas<T>)
     step2d_obstacle(const StepArgs<T> A, const Consts<T> K, const unsigned char* __restrict__ solid) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   for (int y = blockIdx.y * blockDim.y + threadIdx.y; y < A.ny; y += gridDim.y * blockDim.y) {
