@@ -393,8 +393,9 @@ cudaError_t copy_planes(const PlaneCopy& c, size_t elem, cudaStream_t st) {
 template <class T>
 constexpr int kRowsPerCta = sizeof(T) == 8 ? 1 : 4;
 
-// FP64: registers for 16 warps per SM on small grids, which have few (480 x 120: 5.7 us per step,
-// 6.1 with 24), for 24 on others (512^2 18.0 against 19.1, 1536^2 140 against 151).
+// FP64: registers for 16 warps per SM on small grids, which have few, for 24 on others.  us per step with 16 / 24:
+// BGK 480 x 120 5.8 / 6.1, 256^2 6.7 / 6.8, 300^2 9.0 / 7.9, 400^2 13.7 / 12.6, 800^2 45.4 / 42.2; MRT 256^2 7.1 / 7.5, 300^2
+// 9.7 / 8.8; solid cells 256^2 6.8 / 7.4, 300^2 9.1 / 8.5, 362^2 11.0 / 11.6, 400^2 13.3 / 13.1.
 // FP32: for 20 warps per SM, with solid cells 16 (us per step with 16 / 20 / left to the compiler: BGK 780^2 8.2 / 7.3 /
 // 8.5 and 4096 x 2048 127 / 125 / 140, MRT 9.2 / 8.3 / 9.2 and 132 / 126 / 146, solid cells 9.1 / 12.5 / 9.4 and
 // 131 / 150 / 147).
@@ -402,7 +403,7 @@ template <class T, bool OBST, class F>
 cudaError_t with_residency(const StepArgs<T>& a, F&& launch) {
   if constexpr (sizeof(T) == 4)
     return launch(std::integral_constant<int, OBST ? 4 : 5>{});
-  else if (static_cast<long long>(a.nx) * a.ny >= (1LL << 17))
+  else if (static_cast<long long>(a.nx) * a.ny >= (5LL << 14))
     return launch(std::integral_constant<int, 24>{});
   else
     return launch(std::integral_constant<int, 16>{});
