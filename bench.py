@@ -62,10 +62,10 @@ def temporal_kernel_name(k: int, cells: int = 4096 * 4096) -> str:
 # kernel sources it was taken on.
 NCU_TRAFFIC = {
     "step2d_temporal_periodic_x2<6, 256, 1, 0, 1>": {
-        "src_sha256": "645876b793caf71a5988af7076cb879c976a547b4b3c0741e1ea57482e2fbfae",
-        "sources": ("temporal.cu", "temporal.cuh", "temporal_pair.cuh", "scheme.cuh"), "bytes_per_launch": 1746.04e6,
+        "src_sha256": "f5b40c773f8c5e2e69fe97cffae1fe917c3efff45342111a167e9f1497fddc9b",
+        "sources": ("temporal.cu", "temporal.cuh", "temporal_pair.cuh", "scheme.cuh"), "bytes_per_launch": 1745.76e6,
         "case": "ncu dram__bytes_read.sum + dram__bytes_write.sum (1 pass) of the 5 launches of "
-                "bench.py --quick --skip-cpu --steps 12 --warmup 3 (4096x4096): 921.55 MB read + 824.49 MB "
+                "bench.py --quick --skip-cpu --steps 12 --warmup 3 (4096x4096): 921.31 MB read + 824.45 MB "
                 "written per launch (mean)"},
 }
 
@@ -788,7 +788,7 @@ def shock_tube_variant(stream, lbm_sw, torch, steps: int = 500):
     with lbm_sw.Simulation(n, 1, dim=1, precision=lbm_sw.FP64, lam=LAM, s=S_RATE, a=0.15,
                            bc=(lbm_sw.WALL, lbm_sw.WALL), stream=stream.cuda_stream) as sim:
         sim.set_state(h, q)
-        sim.step(4)
+        sim.step(64)  # the launch that is timed (few steps take another one)
         t = _timed(stream, torch, lambda: sim.step(steps))
     return {"MLUPS": n * steps / t / 1e6, "ms_per_run": t * 1e3, "steps": steps}
 

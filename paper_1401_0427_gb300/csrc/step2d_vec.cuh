@@ -58,7 +58,7 @@ struct V1 {
 };
 // Cells per thread of the single-grid row kernels: FP32 16-byte vectors (bound by HBM); FP64 one
 // cell, as its collision is a long chain in two pipes and wants warps (two cells per thread, us per
-// step: 1536^2 158, 701 x 401 27, 480 x 120 with obstacles 14; one: 140, 21.6 and 5.7).
+// step: 1536^2 158, 701 x 401 27, 480 x 120 with obstacles 14; one: 144, 19.3 and 6.0).
 template <class T>
 struct RowVec : V16<T> {};
 template <>
