@@ -301,9 +301,13 @@ int lbm_sw_create(const lbm_sw_params* p, lbm_sw** out) {
   if (!out) return LBM_SW_E_ARG;
   *out = nullptr;
   if (!p) return LBM_SW_E_ARG;
-  lbm_sw* h = new (std::nothrow) lbm_sw;
-  if (!h) return LBM_SW_E_NOMEM;
   g_create_error.clear();
+  lbm_sw* h = nullptr;
+  try {
+    h = new lbm_sw;  // allocates for its members too
+  } catch (const std::bad_alloc&) {
+    return LBM_SW_E_NOMEM;
+  }
   int rc = validate(p, h);
   if (rc != LBM_SW_OK) {
     g_create_error = h->err;  // the handle is not returned: keep the message per thread

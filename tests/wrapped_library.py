@@ -13,9 +13,11 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 PRELUDE = """
 import ctypes, json, sys
 import numpy as np
-import torch
 from paper_1401_0427_gb300 import inputs, lbm_sw
 lib = lbm_sw.load(sys.argv[1])
+"""
+ON_GPU = """
+import torch
 torch.zeros(1, device="cuda")
 """
 
@@ -34,9 +36,9 @@ def link(folder, hook: str, wrapped) -> str:
     return so
 
 
-def run(library: str, script: str):
+def run(library: str, script: str, on_gpu: bool = True):
     """The JSON value of the last line that the script prints in a child process with the library."""
-    r = subprocess.run([sys.executable, "-c", PRELUDE + script, library], capture_output=True, text=True, cwd=ROOT,
+    r = subprocess.run([sys.executable, "-c", PRELUDE + (ON_GPU if on_gpu else "") + script, library], capture_output=True, text=True, cwd=ROOT,
                        env={**os.environ, "PYTHONPATH": ROOT}, timeout=300)
     assert r.returncode == 0, r.stderr
     return json.loads(r.stdout.splitlines()[-1])
