@@ -85,6 +85,9 @@ int obstacle_k(const lbm_sw* h) {
 // periodic and 11.3 / 9.3 with sides, 200 x 2000 10.1 / 9.8 and 11.8 / 9.9, 1024 x 512 12.1 / 11.1 and 13.1 /
 // 11.3; 801 x 601 11.4 / 13.1); two single steps for MRT with sides from 5 * 2^14 cells on (450 x 200 7.6 / 6.7,
 // 640^2 12.8 / 12.3, 1024 x 512 15.2 / 13.8; 256^2 4.6 / 5.1).
+// Four steps (four at a time): BGK on even widths by the estimates of both (us, tiles / wavefront: 700 x 600 periodic 14.4 /
+// 13.4, 900 x 500 15.8 / 14.1, 1024 x 512 16.7 / 15.3 and with sides 20.7 / 18.3; 640^2 13.7 / 15.2 and 16.1 / 17.9).  Launches of
+// other sizes run on tiles: six steps 18 to 21 against 23 to 31.
 enum class TwoSteps { tile, wave, singles };
 TwoSteps two_steps(const lbm_sw* h) {
   const bool per = h->p.bc[LBM_SW_SIDE_XM] == LBM_SW_BC_PERIODIC && h->p.bc[LBM_SW_SIDE_YM] == LBM_SW_BC_PERIODIC;
@@ -350,6 +353,10 @@ int lbm_sw_create(const lbm_sw_params* p, lbm_sw** out) {
   if (h->auto_kernel && p->temporal_steps == 0 && p->dim == 2 && p->precision == LBM_SW_FP32 &&
       static_cast<long long>(p->nx) * p->ny < kTileCells)
     h->tile_k = lbm::tile_steps(p->nx, p->ny, std::max(h->sm_count, 1), &h->tile_waves);
+  // (not where launches are of five steps at most, so that longer runs take fours too: 760 x 740 3.9 us per step on tiles
+  // against 4.05, with sides 4.3 and 4.9)
+  h->wave4 = h->tile_k > 5 && p->nx % 2 == 0 && lbm::temporal4_us(p->nx, p->ny, all_periodic, h->sm_count) <
+                                                    lbm::tile4_us(p->nx, p->ny, all_periodic, h->sm_count);
   const size_t bytes = state_bytes(h);
   for (int i = 0; i < 2; ++i) {
     if (lbm::device_alloc(&h->buf[i], bytes) != cudaSuccess) return bail(LBM_SW_E_NOMEM);
@@ -442,8 +449,8 @@ int lbm_sw_step(lbm_sw* h, int n) {
       const unsigned char* flags = h->has_obstacles ? h->solid_flags : nullptr;
       const cudaError_t e =
           k == 1 ? launch_one_step(h, h->cur, h->stream)
-          : k == 2 && two_steps(h) == TwoSteps::wave
-              ? lbm::launch_step2d_temporal(a, consts(h), 2, h->stream, h->sm_count)
+          : (k == 2 && two_steps(h) == TwoSteps::wave) || (k == 4 && h->wave4 && !h->mrt && temporal_active(h))
+              ? lbm::launch_step2d_temporal(a, consts(h), k, h->stream, h->sm_count)
               : lbm::launch_step2d_tile(a, consts(h), k, flags, h->stream, h->sm_count);
       if (e != cudaSuccess) return cuda_fail(h, e, "tile step launch");
       h->cur ^= 1;

@@ -165,6 +165,10 @@ cudaError_t launch_step2d_tile(const StepArgs<float>& a, const ConstsD& kd, int 
 // wout + (t - 1) * wslot.
 cudaError_t launch_step2d_tile_store_w(const StepArgs<float>& a, const ConstsD& kd, int kb, float* wout, long long wslot,
                                        cudaStream_t st, int sms);
+// us of a launch of four BGK steps on tiles, and by the wavefront on an even width (128-column strips, at most
+// four CTAs per SM), to choose between the two.
+double tile4_us(int nx, int ny, bool periodic, int sms);
+double temporal4_us(int nx, int ny, bool periodic, int sms);
 // Whether a handle's steps run on register tiles (api.cu: AUTO, FP32, below 5 * 2^17 cells).
 bool tile_active(const lbm_sw* h);
 
@@ -266,6 +270,7 @@ struct lbm_sw {
   int graph_chunk = 64;
   int tile_k = 0;            // steps per launch on register tiles, 0: not on these
   int tile_waves = 0;        // waves of tiles of such a launch
+  bool wave4 = false;        // four steps by the wavefront, where it applies
   bool has_state = false;
   long long steps_done = 0;
   long long launches = 0;

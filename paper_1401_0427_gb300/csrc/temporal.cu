@@ -575,6 +575,14 @@ cudaError_t launch_step2d_temporal_store_w(const StepArgs<float>& a, const Const
   }
 }
 
+// An iteration of the K = 4 wavefront takes 0.84 us with up to three CTAs per SM and 0.955 with four, with sides 1.065 and
+// 1.14: within 2 % of launches on grids of 3 to 5 * 2^17 cells and even widths.
+double temporal4_us(int nx, int ny, bool periodic, int sms) {
+  const Partition P = pair_partition(nx, ny, 4, 128, 4 * std::max(sms, 1));
+  const bool three = P.strips * P.segments <= 3 * std::max(sms, 1);
+  return (P.rows_per_cta + 8) * (periodic ? (three ? 0.84 : 0.955) : (three ? 1.065 : 1.14));
+}
+
 cudaError_t launch_step2d_temporal(const StepArgs<float>& a, const ConstsD& kd, int k, cudaStream_t st,
                                    int sm_count) {
   switch (k) {

@@ -57,3 +57,13 @@ def test_two_steps(nx, ny, bc, mrt, plan):
     F0 = inputs.random_populations(13, ny, nx, seed=9200 + nx + ny).astype(np.float32)
     kw = dict(dim=2, precision=lbm_sw.FP32, bc=bc, inflow=INFLOW, a=0.05, mrt_rates=mrt)
     assert np.array_equal(gpu_post(F0, 2, kernel=lbm_sw.KERNEL_VEC, **kw), gpu_post(F0, 2, **kw), equal_nan=True)
+
+
+@pytest.mark.parametrize("bc", [(P, P, P, P), (W, O, I, W)], ids=["periodic", "sides"])
+@pytest.mark.parametrize("nx,ny", [(640, 640), (700, 600), (701, 600), (1024, 512), (760, 740)])
+def test_four_steps(nx, ny, bc):
+    """Launches of four steps by tiles or by the wavefront, whichever is estimated faster: the same bits."""
+    F0 = inputs.random_populations(13, ny, nx, seed=9300 + nx + ny).astype(np.float32)
+    kw = dict(dim=2, precision=lbm_sw.FP32, bc=bc, inflow=INFLOW, a=0.05)
+    for steps in (4, 8):
+        assert np.array_equal(gpu_post(F0, steps, kernel=lbm_sw.KERNEL_VEC, **kw), gpu_post(F0, steps, **kw), equal_nan=True)
