@@ -62,10 +62,10 @@ def temporal_kernel_name(k: int, cells: int = 4096 * 4096) -> str:
 # kernel sources it was taken on.
 NCU_TRAFFIC = {
     "step2d_temporal_periodic_x2<6, 256, 1, 0, 1>": {
-        "src_sha256": "f5b40c773f8c5e2e69fe97cffae1fe917c3efff45342111a167e9f1497fddc9b",
-        "sources": ("temporal.cu", "temporal.cuh", "temporal_pair.cuh", "scheme.cuh"), "bytes_per_launch": 1745.76e6,
+        "src_sha256": "9e80c0cefde2265d14bdb12278541cb20ce33c8d37625af7149d32a0b9edb1d8",
+        "sources": ("temporal.cu", "temporal.cuh", "temporal_pair.cuh", "scheme.cuh"), "bytes_per_launch": 1746.24e6,
         "case": "ncu dram__bytes_read.sum + dram__bytes_write.sum (1 pass) of the 5 launches of "
-                "bench.py --quick --skip-cpu --steps 12 --warmup 3 (4096x4096): 921.31 MB read + 824.45 MB "
+                "bench.py --quick --skip-cpu --steps 12 --warmup 3 (4096x4096): 921.76 MB read + 824.49 MB "
                 "written per launch (mean)"},
 }
 
